@@ -992,6 +992,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 template <int D>
 __global__ void __launch_bounds__(D) combine_kernel(const AttnParams p) {
     pdl_wait();                        // the decode kernel's partials are complete and visible
+    pdl_launch_dependents();
     const int b = blockIdx.x / p.Hq;
     const int ctx = min(p.ctx_lens[b], p.max_ctx);     // as the decode kernel: never beyond the host's bound
     if (ctx <= 0) return;
@@ -1030,6 +1031,7 @@ kv_write_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new
                 uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
                 const int32_t* __restrict__ block_table, int max_blocks, int S, long long total_new, int Hkv,
                 int vec_per_head /* d*2/16 */, int page_size, int num_pages, int* dev_status) {
+    pdl_wait();
     pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid
     __shared__ long long dst_base[KVW_TOK];     // vector index of (page, head 0, row, 0), or -1
     const long long tok0 = static_cast<long long>(blockIdx.x) * KVW_TOK;
@@ -1099,18 +1101,7 @@ static cudaError_t launch_attn_t(dim3 grid, const CUtensorMap& tmQ, const CUtens
                                     static_cast<int>(AttnSmem<D>::ALLOC));
     });
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(ATTN_THREADS);
-    cfg.dynamicSmemBytes = AttnSmem<D>::ALLOC;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, p);
+    return launch_pdl(kern, grid, ATTN_THREADS, AttnSmem<D>::ALLOC, stream, 1, tmQ, tmK, tmV, p);
 }
 
 cudaError_t launch_attn(int d, int mode, dim3 grid, const CUtensorMap& tmQ, const CUtensorMap& tmK,
@@ -1126,19 +1117,8 @@ cudaError_t launch_attn(int d, int mode, dim3 grid, const CUtensorMap& tmQ, cons
 }
 
 cudaError_t launch_combine(int d, const AttnParams& p, int B, cudaStream_t stream) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(B) * p.Hq);
-    cfg.blockDim = dim3(d);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();  // exactly one of the launches below runs
-    if (d == 128) return cudaLaunchKernelEx(&cfg, combine_kernel<128>, p);
-    return cudaLaunchKernelEx(&cfg, combine_kernel<64>, p);
+    return launch_pdl(d == 128 ? combine_kernel<128> : combine_kernel<64>, dim3(static_cast<unsigned>(B) * p.Hq),
+                      static_cast<unsigned>(d), 0, stream, 1, p);
 }
 
 cudaError_t launch_kv_write(const void* k_new, const void* v_new, const int32_t* cu_new,
@@ -1147,18 +1127,12 @@ cudaError_t launch_kv_write(const void* k_new, const void* v_new, const int32_t*
                             int Hkv, int d, int page_size, int num_pages, int* dev_status,
                             cudaStream_t stream) {
     if (total_new <= 0) return cudaSuccess;
-    count_launch();  // exactly one of the launches below runs
-    if (total_new >= 4096)
-        kv_write_kernel<8><<<static_cast<unsigned>((total_new + 7) / 8), KVW_THREADS, 0, stream>>>(
-            static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), cu_new, ctx_lens,
-            static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), block_table, max_blocks, S, total_new, Hkv,
-            d * 2 / 16, page_size, num_pages, dev_status);
-    else
-        kv_write_kernel<1><<<static_cast<unsigned>(total_new), KVW_THREADS, 0, stream>>>(
-            static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), cu_new, ctx_lens,
-            static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), block_table, max_blocks, S, total_new, Hkv,
-            d * 2 / 16, page_size, num_pages, dev_status);
-    return cudaGetLastError();
+    const bool prompt = total_new >= 4096;
+    return launch_pdl(prompt ? kv_write_kernel<8> : kv_write_kernel<1>,
+                      dim3(static_cast<unsigned>(prompt ? (total_new + 7) / 8 : total_new)), KVW_THREADS, 0, stream, 1,
+                      static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), cu_new, ctx_lens,
+                      static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), block_table, max_blocks, S, total_new, Hkv,
+                      d * 2 / 16, page_size, num_pages, dev_status);
 }
 
 }  // namespace tik

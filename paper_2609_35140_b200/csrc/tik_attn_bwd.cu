@@ -64,6 +64,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     constexpr uint32_t IDESC_OUT = mma_idesc_bf16(128, D, true);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    pdl_wait();
+    pdl_launch_dependents();
+
     // ---------------------------------------------------------------- work item
     const int seq = blockIdx.z;
     const int tok0 = p.cu_seqlens[seq];
@@ -514,6 +517,8 @@ template <int D>
 __global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* __restrict__ o,
                                                        const __nv_bfloat16* __restrict__ dout,
                                                        float* __restrict__ delta, long long n_vec) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long v = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (v >= n_vec) return;
@@ -539,23 +544,15 @@ static cudaError_t launch_bwd_t(dim3 grid, const CUtensorMap& tmQ, const CUtenso
         });
         if (e != cudaSuccess) return e;
     }
-    count_launch();
-    kern<<<grid, BWD_THREADS, BwdSmem<D, MODE>::ALLOC, stream>>>(tmQ, tmK, tmV, tmDO, p);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, BWD_THREADS, BwdSmem<D, MODE>::ALLOC, stream, 1, tmQ, tmK, tmV, tmDO, p);
 }
 
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmDO, const BwdParams& p,
                             const void* o, const void* dout, long long n_vec, cudaStream_t stream) {
     const unsigned dgrid = static_cast<unsigned>((n_vec * 32 + 255) / 256);
-    count_launch();  // exactly one of the launches below runs
-    if (d == 128)
-        bwd_delta_kernel<128><<<dgrid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(o),
-                                                         static_cast<const __nv_bfloat16*>(dout), p.delta, n_vec);
-    else
-        bwd_delta_kernel<64><<<dgrid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(o),
-                                                        static_cast<const __nv_bfloat16*>(dout), p.delta, n_vec);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(d == 128 ? bwd_delta_kernel<128> : bwd_delta_kernel<64>, dim3(dgrid), 256, 0, stream, 1,
+                               static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(dout), p.delta, n_vec);
     if (e != cudaSuccess) return e;
     const dim3 gq(max_tiles, p.Hq, S), gkv(max_tiles, p.Hkv, S);
     if (d == 128) {

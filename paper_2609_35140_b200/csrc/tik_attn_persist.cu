@@ -329,6 +329,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     uint8_t* smem = smem_raw;
     const uint32_t sbase = smem_u32(smem_raw);
     if (sbase & 1023u) {     // the swizzled tiles need a 1 KiB aligned base: refuse to run otherwise
+        pdl_wait();
         if (tid == 0) atomicOr(p.dev_status, TIK_DEV_WAIT_EXPIRED);
         return;
     }
@@ -376,7 +377,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // the plan (and every input) is complete from here on.  Launched behind the single-tile grid
     // (wait_at_end) this grid starts once every CTA of that grid has started, which is after the
     // plan completed, and must not wait for that grid here: it is there to fill its tail.
-    if (!p.wait_at_end) pdl_wait();
+    if (!p.wait_at_end) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     if (warp == 3 && lane == 0) {
         // an earlier kernel on this context may have run out of a wait: then do nothing at all
         *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
@@ -933,18 +937,7 @@ static cudaError_t launch_persist_t(int ncta, const CUtensorMap& tmQ, const CUte
                                     static_cast<int>(PASmem<D>::BYTES));
     });
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(ncta));
-    cfg.blockDim = dim3(PA_THREADS);
-    cfg.dynamicSmemBytes = PASmem<D>::BYTES;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, p, plan);
+    return launch_pdl(kern, dim3(static_cast<unsigned>(ncta)), PA_THREADS, PASmem<D>::BYTES, stream, 1, tmQ, tmK, tmV, p, plan);
 }
 
 #ifdef TIK_PA_TRACE
@@ -985,19 +978,9 @@ cudaError_t launch_attn_persist(int d, bool paged, int sm_count, int S, int X, c
     // single tiles two-stage rings), with lengths up to 9 K (most items paired or short) 4 % slower
     // (three launches, two tails): it is used when the length bound exceeds 96 tiles.
     const bool split = X > 8 + (96 - 16);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    cudaError_t e = cudaLaunchKernelEx(&cfg, attn_plan_kernel, p.cu_seqlens, paged ? p.ctx_lens : static_cast<const int32_t*>(nullptr),
-                                       S, split ? 7 : X - 1, static_cast<int4*>(plan));
+    cudaError_t e = launch_pdl(attn_plan_kernel, dim3(1), 1024, 0, stream, 1, p.cu_seqlens,
+                               paged ? p.ctx_lens : static_cast<const int32_t*>(nullptr), S, split ? 7 : X - 1,
+                               static_cast<int4*>(plan));
     if (e != cudaSuccess) return e;
     AttnParams pp = p;
     if (split) {

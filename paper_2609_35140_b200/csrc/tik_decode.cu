@@ -395,18 +395,7 @@ static cudaError_t launch_decode2_t(dim3 grid, const CUtensorMap& tmQ, const CUt
                                     static_cast<int>(DCSmem<D>::BYTES));
     });
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(DC_THREADS);
-    cfg.dynamicSmemBytes = DCSmem<D>::BYTES;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, p);
+    return launch_pdl(kern, grid, DC_THREADS, DCSmem<D>::BYTES, stream, 1, tmQ, tmK, tmV, p);
 }
 
 // Decode for G <= 8 (the caller checks); grid as for attn_kernel's decode mode.

@@ -38,6 +38,8 @@ __global__ void __launch_bounds__(HN_THREADS) rmsnorm_kernel(const NormParams p)
     const uint4* w = reinterpret_cast<const uint4*>(p.weight);
     uint4* y = reinterpret_cast<uint4*>(p.y) + row * nvec;
     __shared__ float warp_tot[4];
+    pdl_wait();
+    pdl_launch_dependents();
 
     uint4 xv[NV], rv[RESIDUAL ? NV : 1];
 #pragma unroll
@@ -93,6 +95,8 @@ __global__ void __launch_bounds__(256) swiglu_kernel(const __nv_bfloat16* __rest
     const int vpr = I / 8;                                   // output vectors per row
     const long long nvec = T * vpr;
     const long long base = static_cast<long long>(blockIdx.x) * (256 * SW_VPT) + threadIdx.x;
+    pdl_wait();
+    pdl_launch_dependents();
     uint4 gv[SW_VPT], uv[SW_VPT];
 #pragma unroll
     for (int j = 0; j < SW_VPT; ++j) {
@@ -123,12 +127,9 @@ template <bool RESIDUAL>
 static cudaError_t launch_rmsnorm_t(const NormParams& p, cudaStream_t stream) {
     const unsigned grid = static_cast<unsigned>(p.T);
     const int nv = (p.H / 8 + HN_THREADS - 1) / HN_THREADS;
-    count_launch();  // exactly one of the launches below runs
-    if (nv <= 1) rmsnorm_kernel<1, RESIDUAL><<<grid, HN_THREADS, 0, stream>>>(p);
-    else if (nv <= 2) rmsnorm_kernel<2, RESIDUAL><<<grid, HN_THREADS, 0, stream>>>(p);
-    else if (nv <= 4) rmsnorm_kernel<4, RESIDUAL><<<grid, HN_THREADS, 0, stream>>>(p);
-    else rmsnorm_kernel<8, RESIDUAL><<<grid, HN_THREADS, 0, stream>>>(p);
-    return cudaGetLastError();
+    auto kern = nv <= 1 ? rmsnorm_kernel<1, RESIDUAL> : nv <= 2 ? rmsnorm_kernel<2, RESIDUAL>
+              : nv <= 4 ? rmsnorm_kernel<4, RESIDUAL> : rmsnorm_kernel<8, RESIDUAL>;
+    return launch_pdl(kern, dim3(grid), HN_THREADS, 0, stream, 1, p);
 }
 
 cudaError_t launch_rmsnorm(const NormParams& p, cudaStream_t stream) {
@@ -139,14 +140,9 @@ cudaError_t launch_rmsnorm(const NormParams& p, cudaStream_t stream) {
 cudaError_t launch_swiglu(const void* gu, void* out, long long T, int I, cudaStream_t stream) {
     if (T <= 0) return cudaSuccess;
     const long long n = T * (I / 8);
-    count_launch();  // exactly one of the launches below runs
-    if (n >= (1ll << 20))
-        swiglu_kernel<4><<<static_cast<unsigned>((n + 1023) / 1024), 256, 0, stream>>>(
-            static_cast<const __nv_bfloat16*>(gu), static_cast<__nv_bfloat16*>(out), T, I);
-    else
-        swiglu_kernel<1><<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
-            static_cast<const __nv_bfloat16*>(gu), static_cast<__nv_bfloat16*>(out), T, I);
-    return cudaGetLastError();
+    const bool large = n >= (1ll << 20);
+    return launch_pdl(large ? swiglu_kernel<4> : swiglu_kernel<1>, dim3(static_cast<unsigned>(large ? (n + 1023) / 1024 : (n + 255) / 256)),
+                      256, 0, stream, 1, static_cast<const __nv_bfloat16*>(gu), static_cast<__nv_bfloat16*>(out), T, I);
 }
 
 }  // namespace tik

@@ -61,7 +61,10 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     // 2048 rows) stays there throughout.  Same MMA chain per element.
     const bool unit_mode = PAIR && p.unit_mode != 0;
     const int u_first = static_cast<int>(blockIdx.x >> 1), u_stride = static_cast<int>(gridDim.x >> 1);
-    if (!unit_mode && (PAIR ? (tile_in_band & ~1) : tile_in_band) >= band_tiles) return;   // a pair leaves only together
+    if (!unit_mode && (PAIR ? (tile_in_band & ~1) : tile_in_band) >= band_tiles) {   // a pair leaves only together
+        pdl_wait();
+        return;
+    }
     const int row_fixed = (band * BAND + tile_in_band) * 128;
     const int col_base = sup * p.super_cols;
     const int ntp = unit_mode ? p.ntp : 1;
@@ -94,11 +97,14 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             mbar_init(bar_acc_full + 8 * b, 1);
             mbar_init(bar_acc_empty + 8 * b, PAIR ? 256 : 128);
         }
-        *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         tma_prefetch_desc(&tmY);
+        // this CTA's first weight tiles on their way to L2 while the kernel before this one drains
+        const int first_col = col_of(0) + (PAIR ? 128 * static_cast<int>(rank) : 0);
+        if (static_cast<int>(blockIdx.x) < p.sm_count && first_col < p.N)
+            for (int kb = 0; kb < min(n_kb, STAGES); ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, first_col);
     }
     if (warp == 1) {
         if (PAIR) {
@@ -109,6 +115,9 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             tmem_relinquish();
         }
     }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync_all();            // the peer's barriers exist before anything signals them
@@ -304,16 +313,22 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             mbar_init(bar_acc_full + 8 * b, 1);
             mbar_init(bar_acc_empty + 8 * b, 128);
         }
-        *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         tma_prefetch_desc(&tmY);
+        // the first 256 KiB of this CTA's weights are requested into L2 while the kernel before this
+        // one drains (an HBM-bound call whose x is a few KiB has nothing else to wait for)
+        const int ahead = min(n_kb, static_cast<int>((256u * 1024u) / (static_cast<uint32_t>(nu) * 128u)));
+        for (int kb = 0; kb < ahead; ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, static_cast<int>(blockIdx.x) * nu);
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
         tmem_relinquish();
     }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -435,9 +450,7 @@ static cudaError_t launch_linear_unit(const CUtensorMap& tmA, const CUtensorMap&
     });
     if (e != cudaSuccess) return e;
     const int grid = p.nunit < p.sm_count ? p.nunit : p.sm_count;
-    count_launch();
-    linear_unit_kernel<<<grid, lin::THREADS, linu::ALLOC, stream>>>(tmA, tmB, tmY, p);
-    return cudaGetLastError();
+    return launch_pdl(linear_unit_kernel, dim3(grid), lin::THREADS, linu::ALLOC, stream, 1, tmA, tmB, tmY, p);
 }
 
 template <bool PAIR>
@@ -460,20 +473,7 @@ static cudaError_t launch_linear_t(const CUtensorMap& tmA, const CUtensorMap& tm
         const int slots = p.sm_count / 2;
         grid = 2ll * (slots < p.nunit ? slots : p.nunit);
     }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(lin::THREADS);
-    cfg.dynamicSmemBytes = C::ALLOC;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, p);
+    return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), lin::THREADS, C::ALLOC, stream, PAIR ? 2 : 1, tmA, tmB, tmY, p);
 }
 
 // pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of a step's 256)

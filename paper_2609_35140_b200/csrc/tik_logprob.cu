@@ -48,7 +48,6 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : 128, NB, false);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;     // 0 = the CTA that issues the pair's MMAs
-    pdl_launch_dependents();           // the finish kernel may be scheduled behind this grid's last wave
 
     // raster: bands of BAND token tiles; within a band the token tile varies fastest so the
     // CTAs in flight share one lm_head super-chunk and the band's hidden rows stay in L2
@@ -77,7 +76,10 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int u_first = static_cast<int>(blockIdx.x) / (PAIR ? 2 : 1);
     const int u_stride = static_cast<int>(gridDim.x) / (PAIR ? 2 : 1);
     const int n_my_units = unit_mode ? (u_first < p.nunit ? (p.nunit - 1 - u_first) / u_stride + 1 : 0) : 0;
-    if (!unit_mode && (PAIR ? (tile_in_band & ~1) : tile_in_band) >= band_tiles) return;
+    if (!unit_mode && (PAIR ? (tile_in_band & ~1) : tile_in_band) >= band_tiles) {
+        pdl_wait();
+        return;
+    }
     const int ntp = unit_mode ? p.ntp : 1;
     const int tok_fixed = (band * BAND + tile_in_band) * 128;
     auto unit_col = [&](int sp) { return ((u_first + sp * u_stride) / ntp) * NB; };
@@ -110,10 +112,13 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             mbar_init(bar_acc_full + 8 * b, 1);
             mbar_init(bar_acc_empty + 8 * b, PAIR ? 256 : 128);   // the epilogue threads of every CTA of the pair
         }
-        *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
+        // this CTA's first lm_head tiles on their way to L2 while the kernel before this one drains
+        const int first_col = (unit_mode ? unit_col(0) : sup0 * LP_SUPER) + (PAIR ? 128 * static_cast<int>(rank) : 0);
+        if (static_cast<int>(blockIdx.x) < p.sm_count && first_col < p.V)
+            for (int kb = 0; kb < min(n_kb, STAGES); ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, first_col);
     }
     if (warp == 1) {
         if (PAIR) {
@@ -124,6 +129,9 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             tmem_relinquish();
         }
     }
+    pdl_wait();
+    pdl_launch_dependents();           // the finish kernel may be scheduled behind this grid's last wave
+    if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync_all();            // the peer's barriers exist before anything signals them
@@ -310,6 +318,7 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // One thread per token: fold the super-chunk pairs in ascending order, write the result.
 __global__ void __launch_bounds__(256) logprob_finish_kernel(const LogprobParams p) {
     pdl_wait();                        // the super-chunk pairs and target logits are complete and visible
+    pdl_launch_dependents();
     const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (t >= p.T) return;
     const float* ml = p.part_ml + 2 * t * p.nsuper;
@@ -335,6 +344,7 @@ __global__ void __launch_bounds__(256) logprob_finish_kernel(const LogprobParams
 // the super-chunks in ascending order as logprob_finish_kernel does.
 __global__ void __launch_bounds__(256) logprob_finish_tiles_kernel(const LogprobParams p) {
     pdl_wait();
+    pdl_launch_dependents();
     __shared__ float sm[256], sl[256];
     const long long t = blockIdx.x;
     const float* ml = p.part_ml + 2 * t * p.ntile128;
@@ -410,20 +420,7 @@ static cudaError_t launch_logprob_main(const CUtensorMap& tmA, const CUtensorMap
         const long long slots = PAIR ? p.sm_count / 2 : p.sm_count;
         grid = (slots < p.nunit ? slots : p.nunit) * (PAIR ? 2 : 1);
     }
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(lp::THREADS);
-    cfg.dynamicSmemBytes = C::ALLOC;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, p);
+    return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), lp::THREADS, C::ALLOC, stream, PAIR ? 2 : 1, tmA, tmB, p);
 }
 
 // pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of the 256 columns)
@@ -432,18 +429,8 @@ cudaError_t launch_logprob(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     if (p.T <= 0) return cudaSuccess;
     cudaError_t e = pair ? launch_logprob_main<true>(tmA, tmB, p, stream) : launch_logprob_main<false>(tmA, tmB, p, stream);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.unit_mode ? p.T : (p.T + 255) / 256));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launch();  // exactly one of the launches below runs
-    if (p.unit_mode) return cudaLaunchKernelEx(&cfg, logprob_finish_tiles_kernel, p);
-    return cudaLaunchKernelEx(&cfg, logprob_finish_kernel, p);
+    return launch_pdl(p.unit_mode ? logprob_finish_tiles_kernel : logprob_finish_kernel,
+                      dim3(static_cast<unsigned>(p.unit_mode ? p.T : (p.T + 255) / 256)), 256, 0, stream, 1, p);
 }
 
 }  // namespace tik

@@ -57,6 +57,7 @@ template <int D>
 __global__ void __launch_bounds__(PREP_WARPS * 32, PREP_MIN_CTAS) prep_kernel(const PrepParams p) {
     constexpr int EP = D / 32;
     constexpr int VPH = D * 2 / 16;             // 16-byte pieces of one V row
+    pdl_wait();
     pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane >> 4, l16 = lane & 15;
@@ -186,10 +187,7 @@ __global__ void __launch_bounds__(PREP_WARPS * 32, PREP_MIN_CTAS) prep_kernel(co
 cudaError_t launch_prep(int d, const PrepParams& p, int64_t total_new, cudaStream_t stream) {
     if (total_new <= 0) return cudaSuccess;
     const unsigned grid = static_cast<unsigned>((total_new + PREP_WARPS - 1) / PREP_WARPS);
-    count_launch();  // exactly one of the launches below runs
-    if (d == 128) prep_kernel<128><<<grid, PREP_WARPS * 32, 0, stream>>>(p);
-    else prep_kernel<64><<<grid, PREP_WARPS * 32, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(d == 128 ? prep_kernel<128> : prep_kernel<64>, dim3(grid), PREP_WARPS * 32, 0, stream, 1, p);
 }
 
 }  // namespace tik

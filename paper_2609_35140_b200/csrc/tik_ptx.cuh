@@ -80,8 +80,16 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity,
 // A kernel launched with the programmatic-stream-serialization attribute may start while its
 // predecessor in the stream still runs: its CTAs are scheduled once every CTA of the predecessor
 // has executed launch_dependents (or exited), and pdl_wait() blocks until the predecessor has
-// completed and its writes are visible.  Used for the small second kernel of a two-kernel call
-// (split-KV combine, log-prob finish) so that its launch latency hides under the first one's tail.
+// completed and its writes are visible.  Every kernel of the library is launched this way
+// (launch_pdl in tik_internal.h): block scheduling, barrier set-up and tensor-memory allocation of a
+// call run under the tail of the call before it.  The rules that keep a chain of such kernels
+// ordered like a plain stream:
+//   * before pdl_wait() a CTA touches no global memory except kernel parameters and L2 prefetches
+//     (writes land in L2, so a prefetched line cannot go stale);
+//   * every CTA executes pdl_wait() on every path, early exits included, so a grid completes after
+//     its predecessor;
+//   * pdl_launch_dependents() comes after pdl_wait(): when a kernel starts, everything before its
+//     immediate predecessor has completed.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -136,6 +144,12 @@ __device__ __forceinline__ void tma_prefetch_l2_4d(const CUtensorMap* m, int c0,
     asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(
                      reinterpret_cast<uint64_t>(m)),
                  "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* m, int c0, int c1) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                     reinterpret_cast<uint64_t>(m)),
+                 "r"(c0), "r"(c1)
                  : "memory");
 }
 // Tiled store shared -> global (bulk async group); never started at a negative coordinate.
