@@ -512,24 +512,50 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// delta[token][head] = sum_c dO * O in fp32: one warp per (token, head), lane chain then butterfly.
+// delta[token][head] = sum_c dO * O in fp32: a warp per (token, head), lane chain then butterfly.
+// HBM-bound: a warp takes eight vectors, all sixteen loads issued before the first sum (53 000 tokens x
+// 28 heads x 128: 180 -> 118 us = 4.3 -> 6.5 TB/s, one vector per warp before).
+constexpr int DELTA_VPW = 8;
 template <int D>
 __global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* __restrict__ o,
                                                        const __nv_bfloat16* __restrict__ dout,
                                                        float* __restrict__ delta, long long n_vec) {
     pdl_wait();
     pdl_launch_dependents();
-    const long long v = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const long long v0 = ((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * DELTA_VPW;
     const int lane = threadIdx.x & 31;
-    if (v >= n_vec) return;
-    constexpr int EPL = D / 32;                             // elements per lane (4 or 2)
-    const __nv_bfloat16* op = o + v * D + EPL * lane;
-    const __nv_bfloat16* dp = dout + v * D + EPL * lane;
-    float part = 0.0f;
+    constexpr int W = D / 64;                               // 32-bit words per lane (4 or 2 elements)
+    uint32_t ow[DELTA_VPW][W], dw[DELTA_VPW][W];
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) part = __fmaf_rn(__bfloat162float(dp[e]), __bfloat162float(op[e]), part);
-    part = hn_warp_total(part);
-    if (lane == 0) delta[v] = part;
+    for (int j = 0; j < DELTA_VPW; ++j) {
+        if (v0 + j < n_vec) {
+            const __nv_bfloat16* op = o + (v0 + j) * D + 2 * W * lane;
+            const __nv_bfloat16* dp = dout + (v0 + j) * D + 2 * W * lane;
+            if (W == 2) {
+                const uint2 a = *reinterpret_cast<const uint2*>(op), b = *reinterpret_cast<const uint2*>(dp);
+                ow[j][0] = a.x, ow[j][W - 1] = a.y, dw[j][0] = b.x, dw[j][W - 1] = b.y;
+            } else {
+                ow[j][0] = *reinterpret_cast<const uint32_t*>(op);
+                dw[j][0] = *reinterpret_cast<const uint32_t*>(dp);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < W; ++e) ow[j][e] = dw[j][e] = 0;
+        }
+    }
+    float mine = 0.0f;                                      // lane j keeps vector j's sum
+#pragma unroll
+    for (int j = 0; j < DELTA_VPW; ++j) {
+        float part = 0.0f;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {                       // bf16 -> fp32 is exact
+            part = __fmaf_rn(__uint_as_float(dw[j][e] << 16), __uint_as_float(ow[j][e] << 16), part);
+            part = __fmaf_rn(__uint_as_float(dw[j][e] & 0xffff0000u), __uint_as_float(ow[j][e] & 0xffff0000u), part);
+        }
+        part = hn_warp_total(part);
+        if (lane == j) mine = part;
+    }
+    if (lane < DELTA_VPW && v0 + lane < n_vec) delta[v0 + lane] = mine;
 }
 
 template <int D, int MODE>
@@ -550,7 +576,7 @@ static cudaError_t launch_bwd_t(dim3 grid, const CUtensorMap& tmQ, const CUtenso
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmDO, const BwdParams& p,
                             const void* o, const void* dout, long long n_vec, cudaStream_t stream) {
-    const unsigned dgrid = static_cast<unsigned>((n_vec * 32 + 255) / 256);
+    const unsigned dgrid = static_cast<unsigned>((n_vec + 8 * DELTA_VPW - 1) / (8 * DELTA_VPW));
     cudaError_t e = launch_pdl(d == 128 ? bwd_delta_kernel<128> : bwd_delta_kernel<64>, dim3(dgrid), 256, 0, stream, 1,
                                static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(dout), p.delta, n_vec);
     if (e != cudaSuccess) return e;

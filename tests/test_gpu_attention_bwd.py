@@ -92,3 +92,16 @@ def test_backward_invalid_arguments(tik):
     with pytest.raises(tik.TikError):
         tik.tik_attn_train_bwd(q, k, v, q, q, lse, cu, max(w.seq_lens), w.softmax_scale,
                                ws=torch.empty(16, dtype=torch.uint8, device="cuda"))
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d", [([9], 7, 1, 128), ([33, 2], 3, 1, 128), ([127], 5, 1, 64), ([2], 1, 1, 64)])
+def test_backward_of_a_few_rows(tik, lens, Hq, Hkv, d):
+    """Numbers of (token, head) vectors that are no multiple of what a warp or a block of the delta kernel takes."""
+    w = synth.custom_workload([1] * len(lens), [L - 1 for L in lens], Hq, Hkv, d, 64, index=57)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    do, _, _, _ = synth.make_qkv(w, "cuda", seed_offset=9)
+    got = _fwd_bwd(tik, w, q, k, v, cu, do)
+    want = oracle.attn_bwd_packed(q.float().cpu().numpy(), k.float().cpu().numpy(), v.float().cpu().numpy(),
+                                  do.float().cpu().numpy(), w.cu_seqlens(), w.softmax_scale)
+    for name, a, b in zip(("dq", "dk", "dv"), got, want):
+        _check(a, b, name)
