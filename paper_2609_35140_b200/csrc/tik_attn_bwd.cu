@@ -64,19 +64,33 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     constexpr uint32_t IDESC_OUT = mma_idesc_bf16(128, D, true);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    pdl_wait();
-    pdl_launch_dependents();
+    // Launch order and dependencies: delta kernel, dK/dV grid, dQ grid, each with a programmatic
+    // dependency.  The dK/dV grid waits for the delta kernel here.  The dQ grid starts once every CTA
+    // of the dK/dV grid has passed that wait (so everything it reads is complete) and must not wait
+    // for that grid: its CTAs fill the SMs that the dK/dV grid's last CTAs leave idle.  Only its last
+    // block waits for the dK/dV grid, at its end, so that the dQ grid completes after it (and no dQ CTA
+    // releases its dependents early).  Two sequences of 96 and 160 tokens (4/1 heads, d 64), forward and
+    // backward: 32.2 -> 27.6 us.
+    if (MODE == BWD_DKV) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
+    const bool last_block = MODE == BWD_DQ && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 &&
+                            blockIdx.z == gridDim.z - 1;
 
     // ---------------------------------------------------------------- work item
     const int seq = blockIdx.z;
     const int tok0 = p.cu_seqlens[seq];
     const int len = p.cu_seqlens[seq + 1] - tok0;
-    if (len <= 0) return;
+    if (len <= 0) {
+        if (last_block) pdl_wait();
+        return;
+    }
     const int nq = (len + 127) / 128;                      // tiles of the sequence (query and KV alike)
     int own, head = 0, kvh, n_steps;
     if (MODE == BWD_DQ) {
         own = gridDim.x - 1 - blockIdx.x;                  // query tile, heaviest first
-        if (own >= nq) return;
+        if (own >= nq) return;                             // (never the last block: its tile is 0)
         head = blockIdx.y;
         kvh = head / p.G;
         n_steps = own + 1;                                 // KV tiles 0..own
@@ -314,7 +328,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (MODE == BWD_DQ && row_abs < len) {
             const long long idx = (static_cast<long long>(tok0) + row_abs) * p.Hq + head;
             row_l2 = __fmul_rn(p.lse[idx], LOG2E_F);
-            row_dl = p.delta[idx];
+            row_dl = __ldcg(&p.delta[idx]);     // (around L1: no wait of this grid's own precedes the read)
         }
         // DKV: the scalars belong to the columns (query rows of the streamed tile).  Thread `et` < 64
         // of warpgroup h fetches those of column 64 h + et one step ahead; they reach the other
@@ -507,6 +521,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         while (globaltimer_ns() - t0 < 1000000ull) {
         }
     }
+    if (last_block) pdl_wait();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
