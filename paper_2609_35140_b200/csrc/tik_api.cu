@@ -52,11 +52,25 @@ static tik_status cuda_fail(tik_ctx* ctx, cudaError_t e, const char* where) {
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static bool page_ok(int page) { return page == 16 || page == 32 || page == 64 || page == 128; }
 static float scale_to_c(float softmax_scale) { return softmax_scale * LOG2E_F; }
-// Candidate work items per (sequence, head) for the full-sequence kernels: query tiles 0..15 go
-// in pairs (x = 0..7), tiles >= 16 one by one (x = 8 + tile - 16); see attn_kernel.
-static unsigned attn_grid_x(int max_positions) {
+// Candidate work items per (sequence, head) for the full-sequence kernels: the first 2 npair query
+// tiles go in pairs (x = 0 .. npair - 1), the others one by one (x = tile - npair); see attn_kernel.
+static unsigned attn_grid_x(int max_positions, int npair = 8) {
     const int nt = (max_positions + 127) / 128;
-    return static_cast<unsigned>(nt <= 16 ? (nt + 1) / 2 : 8 + (nt - 16));
+    return static_cast<unsigned>(nt <= 2 * npair ? (nt + 1) / 2 : nt - npair);
+}
+// How many pairs a call of one CTA per item makes.  Pairs halve the operand traffic and the number of
+// CTAs (each costs ~8 700 clk beside ~1 560 per step), which is what a call that fills the chip wants; a
+// call whose items are all resident at once takes as long as its longest one, and a pair (t, t + 1) is
+// 2 t + 3 steps where a single tile t is t + 1.  So: the fewest pairs for which every item still has
+// an SM to itself, else all eight.  One prompt, all tiles paired -> by this rule (cold L2): 1000 tokens
+// (28/4 heads) 24.6 -> 22.5 us, 1000 (12/2) 24.5 -> 18.6, 2048 (12/2) 36.9 -> 26.7; two of 1000 (12/2) 24.6 -> 20.4.
+// new_tiles: bound on the query tiles of one sequence.
+static int attn_pairs(long long seq_heads, int max_positions, long long new_tiles, int sm_count) {
+    for (int np = 0; np < 8; ++np) {
+        const long long x = attn_grid_x(max_positions, np);
+        if (seq_heads * (x < new_tiles ? x : new_tiles) <= sm_count) return np;
+    }
+    return 8;
 }
 
 // The persistent kernel runs when the caller passed a large enough, 16-byte aligned plan buffer and
@@ -243,11 +257,15 @@ tik_status tik_attn_train_fwd(tik_ctx* ctx, const void* q, const void* k, const 
     dim3 grid(attn_grid_x(max_seqlen), Hq, S);
     if (grid.y > 65535 || grid.z > 65535) return fail(ctx, TIK_ERR_UNSUPPORTED, "Hq and S must be <= 65535");
     cudaError_t e;
+    p.npair = 8;
     if (use_persistent(ws, ws_bytes, S, max_seqlen, Hq, ctx->sm_count))
         e = launch_attn_persist(d, false, ctx->sm_count, S, static_cast<int>(grid.x), tmQ, tmK, tmV, p, ws,
                                 static_cast<cudaStream_t>(stream));
-    else
+    else {
+        p.npair = attn_pairs(static_cast<long long>(S) * Hq, max_seqlen, (max_seqlen + 127ll) / 128, ctx->sm_count);
+        grid.x = attn_grid_x(max_seqlen, p.npair);
         e = launch_attn(d, 0, grid, tmQ, tmK, tmV, p, static_cast<cudaStream_t>(stream));
+    }
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_train_fwd");
 }
 
@@ -338,11 +356,16 @@ tik_status tik_attn_prefill(tik_ctx* ctx, const void* q, void* o, float* lse, co
     dim3 grid(attn_grid_x(max_ctx_len), Hq, S);
     if (grid.y > 65535 || grid.z > 65535) return fail(ctx, TIK_ERR_UNSUPPORTED, "Hq and S must be <= 65535");
     cudaError_t e;
+    p.npair = 8;
     if (use_persistent(ws, ws_bytes, S, max_ctx_len, Hq, ctx->sm_count))
         e = launch_attn_persist(d, true, ctx->sm_count, S, static_cast<int>(grid.x), tmQ, tmK, tmV, p, ws,
                                 static_cast<cudaStream_t>(stream));
-    else
+    else {
+        // (new rows may start in the middle of a tile: one tile more than whole tiles of them)
+        p.npair = attn_pairs(static_cast<long long>(S) * Hq, max_ctx_len, (max_q_len + 127ll) / 128 + 1, ctx->sm_count);
+        grid.x = attn_grid_x(max_ctx_len, p.npair);
         e = launch_attn(d, 1, grid, tmQ, tmK, tmV, p, static_cast<cudaStream_t>(stream));
+    }
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_prefill");
 }
 

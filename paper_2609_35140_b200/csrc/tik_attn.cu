@@ -99,11 +99,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     pdl_wait();
 
     // ---------------------------------------------------------------- work item
-    // Train / prefill: query tiles are aligned to absolute positions.  Tiles 0..15 (their KV
-    // range is one chunk) are taken two at a time: a CTA owns tiles 2m (A) and 2m+1 (B) of one
-    // (sequence, head), streams every K/V tile once for both, and each softmax warpgroup keeps
-    // the rows of one of the two tiles from the first KV tile to the last.  Tiles >= 16, a tile
-    // without a partner, and decode run one query tile per CTA.
+    // Train / prefill: query tiles are aligned to absolute positions.  Tiles 0 .. 2 npair - 1 (npair
+    // <= 8: their KV range is one chunk) are taken two at a time: a CTA owns tiles 2m (A) and 2m+1 (B)
+    // of one (sequence, head), streams every K/V tile once for both, and each softmax warpgroup
+    // keeps the rows of one of the two tiles from the first KV tile to the last.  The tiles from
+    // 2 npair on, a tile without a partner, and decode run one query tile per CTA.
     int seq, head, kvh, chunk = 0, ctx = 0;
     int T0 = 0, T1 = 0;        // query tile of parity 0 (single mode, or B) and of parity 1 (A)
     bool pair = false;
@@ -132,8 +132,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         }
         const int t_lo = pos0 / 128, t_hi = (ctx - 1) / 128;     // first and last query tile
         const int x = p.x_base + gridDim.x - 1 - blockIdx.x;     // heaviest candidates first
-        if (x >= 8) {
-            T0 = 16 + (x - 8);
+        if (x >= p.npair) {
+            T0 = p.npair + x;
             if (T0 < t_lo || T0 > t_hi) return;
         } else {
             const int ta = 2 * x, tb = 2 * x + 1;
@@ -441,8 +441,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     const int x2 = p.x_base + gridDim.x - 1 - bx;
                     const int t_lo2 = pos2 / 128, t_hi2 = (ctx2 - 1) / 128;
                     for (int q2 = 0; q2 < 2; ++q2) {
-                        const int Tq = (x2 >= 8) ? (16 + x2 - 8) : (2 * x2 + q2);
-                        if ((x2 >= 8 && q2 == 1) || Tq < t_lo2 || Tq > t_hi2) continue;
+                        const int Tq = (x2 >= p.npair) ? (p.npair + x2) : (2 * x2 + q2);
+                        if ((x2 >= p.npair && q2 == 1) || Tq < t_lo2 || Tq > t_hi2) continue;
                         const int row = qb2 + 128 * Tq - pos2;
                         for (int a = 0; a < NATOM; ++a) tma_prefetch_l2_3d(&tmQ, a * 64, by, row);
                     }

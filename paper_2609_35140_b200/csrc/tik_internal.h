@@ -104,6 +104,7 @@ struct AttnParams {
                                  // the result, normalised and stored by the decode kernel itself (no combine)
     int* dev_status;
     int lookahead;               // train / prefill: block distance of the query-tile L2 prefetch
+    int npair;                   // train / prefill, one CTA per item: the first 2 npair query tiles go in pairs (<= 8)
     int x_base;                  // train / prefill, one CTA per item: candidate index of the grid's last block (0, or 8: single tiles only)
     int wait_at_end;             // persistent kernel: 1 = launched behind the single-tile grid (see launch_attn_persist)
 };

@@ -115,3 +115,26 @@ def test_caller_scratch_is_used_and_too_small_scratch_falls_back(tik):
     o1 = tik.tik_attn_train_fwd(q1, k1, v1, cu1, 701, w1.softmax_scale, ws=ws1)
     assert bool((ws1 == 0).all())
     assert count_diff(o1, tik.tik_attn_train_fwd(q1, k1, v1, cu1, 701, w1.softmax_scale, ws=False)) == 0
+
+
+@pytest.mark.parametrize("S,L,Hq,Hkv,prefix", [(1, 1000, 28, 4, 0), (1, 128, 28, 4, 0), (1, 129, 70, 10, 0), (2, 2048, 4, 1, 0),
+                                               (1, 2049, 8, 2, 0), (3, 385, 12, 2, 0), (1, 300, 28, 4, 900), (1, 1, 4, 1, 2100)])
+def test_calls_of_one_wave_with_and_without_paired_tiles(tik, S, L, Hq, Hkv, prefix):
+    """Small calls split query tiles into pairs and single tiles by how many items fit the SMs: the rows have
+    the bits of a call whose batch is too large for that rule (the same sequences six times over)."""
+    w = synth.custom_workload([1] * S, [prefix + L - 1] * S, Hq, Hkv, 128, 64, index=61)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    many = lambda t: t.repeat(6 * (1 + 300 // (S * Hq)), 1, 1)
+    n_many = 6 * (1 + 300 // (S * Hq)) * S
+    cu_many = torch.arange(n_many + 1, device="cuda", dtype=torch.int32) * (prefix + L)
+    o = tik.tik_attn_train_fwd(q, k, v, cu, prefix + L, w.softmax_scale, ws=False)
+    o_many = tik.tik_attn_train_fwd(many(q), many(k), many(v), cu_many, prefix + L, w.softmax_scale, ws=False)
+    assert count_diff(o_many[:o.shape[0]], o) == 0
+    layout = synth.make_paged_layout(w)
+    kc, vc = synth.fill_paged_cache(w, layout, k, v)
+    bt = torch.from_numpy(layout.block_table).cuda()
+    ctx = torch.full((S,), prefix + L, dtype=torch.int32, device="cuda")
+    rows = torch.cat([torch.arange((prefix + L) * s + prefix, (prefix + L) * (s + 1), device="cuda") for s in range(S)])
+    cu_q = torch.arange(S + 1, device="cuda", dtype=torch.int32) * L
+    o_pre = tik.tik_attn_prefill(q[rows].contiguous(), cu_q, ctx, kc, vc, bt, L, prefix + L, w.softmax_scale)
+    assert count_diff(o_pre, o[rows]) == 0
