@@ -92,7 +92,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     constexpr uint32_t IDESC_QK = mma_idesc_bf16(128, 128, false);
     constexpr uint32_t IDESC_PV = mma_idesc_bf16(128, D, true);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     // Launched with programmatic stream serialization: the grid may be scheduled while the kernel
     // before it in the stream (typically the cache write or the pre-attention step of the same
     // call sequence) is still draining; nothing of this kernel's input is read before this wait.
@@ -176,6 +176,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // mode: even steps belong to B (= T0), odd steps to A (= T1 = T0 - 1), step g uses KV tile g/2;
     // A has one KV tile less, so the last step (even) is B's diagonal tile.
     const int n_steps = pair ? (2 * n_tiles - 1) : n_tiles;
+    // (the issuing warps shadow these with warp-uniform copies)
+    const int n_steps_v = n_steps, tile_first_v = tile_first;
+    const bool pair_v = pair;
     const int KS = (pair || MODE == MODE_DECODE) ? 2 : KV_STAGES;   // K stages in use
     const int q_row_first[2] = {static_cast<int>(qrow0[0]), static_cast<int>(qrow0[1])};
 
@@ -391,8 +394,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         // Two threads feed the tensor pipe (this one and the PV issuer in warp 3): whatever an
         // issuing thread executes between MMAs is time in which it queues nothing, so each
         // keeps to waits, one MMA chain and its commits per step.
-        if (lane == 0) {
-            mbar_wait(bar_q, 0, abort_word, p.dev_status);
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            const int n_steps = warp_uniform(n_steps_v);
+            const bool pair = warp_uniform(static_cast<int>(pair_v)) != 0;
+            const int KS = (pair || MODE == MODE_DECODE) ? 2 : KV_STAGES;
+            mbar_wait_warp(bar_q, 0, abort_word, p.dev_status);
             const uint64_t dq0 = smem_desc_sw128(sQ, 0, 1024);
             const uint64_t dq1 = smem_desc_sw128(sQ + L::TILE, 0, 1024);
             for (int g = 0; g < n_steps; ++g) {
@@ -400,8 +407,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 const int st = (KS == 2) ? (kt & 1) : (kt % KV_STAGES), b = g & 1;
                 const int kuse = (KS == 2) ? (kt >> 1) : (kt / KV_STAGES);
                 // the single score buffer is free once the softmax of step g-1 holds it in registers
-                mbar_wait(bar_kfull + 8 * st, kuse & 1, abort_word, p.dev_status);
-                if (g >= 1) mbar_wait(bar_sempty + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_kfull + 8 * st, kuse & 1, abort_word, p.dev_status);
+                if (g >= 1) mbar_wait_warp(bar_sempty + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 const uint64_t dq = (pair && b) ? dq1 : dq0;
                 const uint64_t dk = smem_desc_sw128(sK + st * L::TILE, 0, 1024);
@@ -449,12 +456,21 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 }
             }
         }
-        if (lane == 0) {
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            const int n_steps = warp_uniform(n_steps_v), tile_first = warp_uniform(tile_first_v);
+            const bool pair = warp_uniform(static_cast<int>(pair_v)) != 0;
+            auto chunk_of = [&](int it) { return (tile_first + it) / TILES_PER_CHUNK; };
+            auto is_chunk_start = [&](int it) { return ((tile_first + it) % TILES_PER_CHUNK) == 0; };
+            auto col_o_of = [&](int it) -> uint32_t {
+                if (MODE == MODE_DECODE) return (chunk_of(it) & 1) ? COL_OB : COL_OA;
+                return chunk_of(it) == 0 ? COL_OA : COL_OB;
+            };
             for (int g = 0; g < n_steps; ++g) {
                 const int vt = pair ? (g >> 1) : g;
                 const int st = vt % KV_STAGES, b = g & 1;
-                mbar_wait(bar_vfull + 8 * st, (vt / KV_STAGES) & 1, abort_word, p.dev_status);
-                mbar_wait(bar_pfull + 8 * b, (g >> 1) & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_vfull + 8 * st, (vt / KV_STAGES) & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_pfull + 8 * b, (g >> 1) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 // paired mode: B accumulates in O_A, A in O_B, each from its first KV tile on
                 const uint32_t col_o = pair ? (b ? COL_OB : COL_OA) : col_o_of(g);

@@ -62,7 +62,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     constexpr uint32_t IDESC_SC = mma_idesc_bf16(128, 64, false);       // one half: 64 streamed rows
     constexpr uint32_t IDESC_SC128 = mma_idesc_bf16(128, 128, false);   // DQ: all 128 streamed rows at once
     constexpr uint32_t IDESC_OUT = mma_idesc_bf16(128, D, true);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
 
     // Launch order and dependencies: delta kernel, dK/dV grid, dQ grid, each with a programmatic
     // dependency.  The dK/dV grid waits for the delta kernel here.  The dQ grid starts once every CTA
@@ -100,6 +100,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         kvh = blockIdx.y;
         n_steps = p.G * (nq - own);                        // (g, query tile i >= own), g outermost
     }
+    const int n_steps_v = n_steps;       // (the issuing warps shadow it with a warp-uniform copy)
     // step t -> the streamed tile and (DKV) the query head
     auto step_tile = [&](int t) { return MODE == BWD_DQ ? t : own + t % (nq - own); };
     auto step_head = [&](int t) { return MODE == BWD_DQ ? head : kvh * p.G + t / (nq - own); };
@@ -217,8 +218,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // MMAs issued by one thread execute in order: the score MMAs of half h of step t+1 overwrite
         // the columns that hold the weights of half h of step t only after the gradient MMAs that
         // read them.  Issue order per step: gradient(a,t), score(a,t+1), gradient(b,t), score(b,t+1).
-        if (lane == 0) {
-            mbar_wait(bar_r, 0, abort_word, p.dev_status);
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            const int n_steps = warp_uniform(n_steps_v);
+            mbar_wait_warp(bar_r, 0, abort_word, p.dev_status);
             const uint64_t dr1 = smem_desc_sw128(sR1, 0, 1024), dr2 = smem_desc_sw128(sR2, 0, 1024);
             auto stage_c1 = [&](int t) { return sbase + L::OFF_C + (t % BWD_STAGES) * 2 * L::TILE; };
             auto score = [&](int t, int h) {      // T1h = R1 C1h^T, T2h = R2 C2h^T (64 streamed rows = 8 KiB)
@@ -251,12 +254,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 auto score_full = [&](int t) {
                     const uint32_t c1 = stage_k(t), c2 = sbase + L::OFF_C + (DQ_KSTAGES + t % DQ_VSTAGES) * L::TILE;
                     const uint32_t t2 = tmem + ((t & 1) ? COL_T2B : COL_T2);
-                    mbar_wait(bar_cfull + 8 * (t % DQ_KSTAGES), (t / DQ_KSTAGES) & 1, abort_word, p.dev_status);
-                    mbar_wait(bar_vfull + 8 * (t % DQ_VSTAGES), (t / DQ_VSTAGES) & 1, abort_word, p.dev_status);
-                    if (t > 0) mbar_wait(bar_tfull + 8, (t - 1) & 1, abort_word, p.dev_status);   // S of step t-1 is in registers
+                    mbar_wait_warp(bar_cfull + 8 * (t % DQ_KSTAGES), (t / DQ_KSTAGES) & 1, abort_word, p.dev_status);
+                    mbar_wait_warp(bar_vfull + 8 * (t % DQ_VSTAGES), (t / DQ_VSTAGES) & 1, abort_word, p.dev_status);
+                    if (t > 0) mbar_wait_warp(bar_tfull + 8, (t - 1) & 1, abort_word, p.dev_status);   // S of step t-1 is in registers
                     // the dP tile of this parity held dS of step t-2 (the two issuing threads have no
                     // common program order, so its gradient product is waited for)
-                    if (t > 1) mbar_wait(bar_gdone + 8 * (t & 1), ((t - 2) >> 1) & 1, abort_word, p.dev_status);
+                    if (t > 1) mbar_wait_warp(bar_gdone + 8 * (t & 1), ((t - 2) >> 1) & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     if (D == 128) {
                         mma_ss_chain8_fresh(tmem + COL_T1, dr1, smem_desc_sw128(c1, 0, 1024), IDESC_SC128);
@@ -273,17 +276,17 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     score_full(t);
                 }
             } else {
-            mbar_wait(bar_cfull, 0, abort_word, p.dev_status);
+            mbar_wait_warp(bar_cfull, 0, abort_word, p.dev_status);
             tc_fence_after();
             score(0, 0);
             score(0, 1);
             for (int t = 0; t < n_steps; ++t) {
                 if (*abort_word) break;
                 const bool more = t + 1 < n_steps;
-                if (more) mbar_wait(bar_cfull + 8 * ((t + 1) % BWD_STAGES), ((t + 1) / BWD_STAGES) & 1, abort_word,
+                if (more) mbar_wait_warp(bar_cfull + 8 * ((t + 1) % BWD_STAGES), ((t + 1) / BWD_STAGES) & 1, abort_word,
                                     p.dev_status);
                 for (int h = 0; h < 2; ++h) {
-                    mbar_wait(bar_efull + 8 * h, t & 1, abort_word, p.dev_status);
+                    mbar_wait_warp(bar_efull + 8 * h, t & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     gradient(t, h);
                     if (h == 1) mma_commit(bar_cempty + 8 * (t % BWD_STAGES));     // stage of step t consumed
@@ -298,10 +301,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // ------------------------------------------------------------ DQ: gradient-product issuer
         // A thread of its own, so that its waits and commits do not stand between two score
         // products in the other issuing thread.
-        if (MODE == BWD_DQ && lane == 0) {
+        if (MODE == BWD_DQ) {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            const int n_steps = warp_uniform(n_steps_v);
             for (int t = 0; t < n_steps; ++t) {
                 if (*abort_word) break;
-                mbar_wait(bar_efull, t & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_efull, t & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 // A = dS: every thread left its 32 columns' bf16 pairs in the first 16 columns of
                 // its own 32-column block, so the eight 16-key steps sit at 0, 8, 32, 40, ...

@@ -74,6 +74,12 @@ __device__ long long g_pa_steps[8 * 4 * 16 * 8];
         mbar_wait(__VA_ARGS__);   \
     } while (0)
 
+#define PA_WAIT_WARP(site, ...)        \
+    do {                               \
+        PA_TAG(site);                  \
+        mbar_wait_warp(__VA_ARGS__);   \
+    } while (0)
+
 __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
 }
@@ -320,7 +326,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     constexpr uint32_t IDESC_QK = mma_idesc_bf16(128, 128, false);
     constexpr uint32_t IDESC_PV = mma_idesc_bf16(128, D, true);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
 #ifdef TIK_PA_TRACE
     int pa_tag = 0, pa_aux = 0;
 #endif
@@ -391,7 +397,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const uint32_t tmem = *tmem_slot;
 
     // (plan entries are read around L1: a line of an earlier call's plan may still sit there)
-    const unsigned n_items = static_cast<unsigned>(__ldcg(&plan[0]).x) * static_cast<unsigned>(p.Hq);   // < 2^31 (host check)
+    const unsigned n_items = warp_uniform(static_cast<uint32_t>(__ldcg(&plan[0]).x)) * static_cast<unsigned>(p.Hq);   // < 2^31 (host check)
     const unsigned ncta = gridDim.x, cta = blockIdx.x;
     // list position of this CTA's k-th item (rounds alternate direction)
     auto item_index = [&](int k) -> unsigned {
@@ -502,7 +508,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ QK^T issuer
-        if (lane == 0) {
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
             uint32_t Gs = 0, kbase = 0;
             uint32_t qcnt0 = 0, qcnt1 = 0;
             int sB = 0;
@@ -511,7 +518,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (item_index(0) < n_items) e_n = load_entry(item_index(0), head_n);
             for (int k = 0;; ++k) {
                 if (item_index(k) >= n_items || *abort_word) break;
-                e = e_n;
+                e.x = warp_uniform(e_n.x), e.y = warp_uniform(e_n.y), e.z = warp_uniform(e_n.z), e.w = warp_uniform(e_n.w);
                 head = head_n;
                 if (item_index(k + 1) < n_items) e_n = load_entry(item_index(k + 1), head_n);
                 const PAItem it = pa_decode(e, head);
@@ -526,15 +533,15 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     if (g == 0) PA_STAMP(k, 0);
                     if (g == 0 || (it.pair && g == 1)) {          // first use of this query tile
                         const int slot = tileA ? (sB ^ 1) : sB;
-                        PA_WAIT(3, bar_qfull + 8 * slot, (slot ? qcnt1 : qcnt0) & 1, abort_word, p.dev_status);
+                        PA_WAIT_WARP(3, bar_qfull + 8 * slot, (slot ? qcnt1 : qcnt0) & 1, abort_word, p.dev_status);
                         if (slot) ++qcnt1; else ++qcnt0;
                     }
                     if (g == 0) PA_STAMP(k, 1);
-                    PA_WAIT(4, bar_kfull + 8 * st, (kc >> 1) & 1, abort_word, p.dev_status);
+                    PA_WAIT_WARP(4, bar_kfull + 8 * st, (kc >> 1) & 1, abort_word, p.dev_status);
                     if (g == 0) PA_STAMP(k, 2);
                     PA_SSTAMP(k, 0, g, 0);
                     // the single score buffer is free once the softmax of the previous step holds it in registers
-                    if (Gs >= 1) PA_WAIT(5, bar_sempty + 8 * ((Gs - 1) & 1), ((Gs - 1) >> 1) & 1, abort_word, p.dev_status);
+                    if (Gs >= 1) PA_WAIT_WARP(5, bar_sempty + 8 * ((Gs - 1) & 1), ((Gs - 1) >> 1) & 1, abort_word, p.dev_status);
                     if (g == 0) PA_STAMP(k, 3);
                     if (g == 1) PA_STAMP(k, 4);
                     if (g == it.n_steps - 1) PA_STAMP(k, 5);
@@ -559,7 +566,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         __syncwarp();
     } else {
         // ------------------------------------------------------------ PV issuer
-        if (lane == 0) {
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
             uint32_t Gs = 0, vbase = 0;
             uint32_t drains0 = 0, drains1 = 0;  // epilogues that have read accumulator A / B so far
             int head = 0, head_n = 0;
@@ -567,7 +575,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (item_index(0) < n_items) e_n = load_entry(item_index(0), head_n);
             for (int k = 0;; ++k) {
                 if (item_index(k) >= n_items || *abort_word) break;
-                e = e_n;
+                e.x = warp_uniform(e_n.x), e.y = warp_uniform(e_n.y), e.z = warp_uniform(e_n.z), e.w = warp_uniform(e_n.w);
                 head = head_n;
                 if (item_index(k + 1) < n_items) e_n = load_entry(item_index(k + 1), head_n);
                 const PAItem it = pa_decode(e, head);
@@ -577,10 +585,10 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     const uint32_t vc = vbase + vt;
                     const int st = vc & 1, b = Gs & 1;
                     if (g == 0) PA_STAMP(k, 6);
-                    PA_WAIT(6, bar_vfull + 8 * st, (vc >> 1) & 1, abort_word, p.dev_status);
+                    PA_WAIT_WARP(6, bar_vfull + 8 * st, (vc >> 1) & 1, abort_word, p.dev_status);
                     if (g == 0) PA_STAMP(k, 7);
                     PA_SSTAMP(k, 1, g, 0);
-                    PA_WAIT(7, bar_pfull + 8 * b, (Gs >> 1) & 1, abort_word, p.dev_status);
+                    PA_WAIT_WARP(7, bar_pfull + 8 * b, (Gs >> 1) & 1, abort_word, p.dev_status);
                     if (g == 0) PA_STAMP(k, 8);
                     if (g == it.n_steps - 1) PA_STAMP(k, 9);
                     // paired: the warpgroup of this step's parity accumulates its tile in its own accumulator;
@@ -589,7 +597,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     const bool fresh = it.pair ? (vt == 0) : ((g % TILES_PER_CHUNK) == 0);
                     const uint32_t drained = acc ? drains1 : drains0;
                     if ((it.pair ? (g < 2) : (g == 0)) && drained > 0)
-                        PA_WAIT(8, bar_odrain + 8 * acc, (drained - 1) & 1, abort_word, p.dev_status);
+                        PA_WAIT_WARP(8, bar_odrain + 8 * acc, (drained - 1) & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     PA_SSTAMP(k, 1, g, 1);
                     mma_ts_chain8(tmem + (acc ? COL_OB : COL_OA), tmem + COL_P + 64 * b,

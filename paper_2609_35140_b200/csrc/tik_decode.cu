@@ -43,9 +43,9 @@ struct DCSmem {
 // QK^T chain for the compact query tile: A atoms are 1 KiB (64 descriptor units) apart, B atoms 16 KiB.
 __device__ __forceinline__ void mma_ss_chain8_fresh_qcompact(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 da, db;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
         "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
         TIK_MMA_SS_STEP(2, 2) TIK_MMA_SS_STEP(4, 4) TIK_MMA_SS_STEP(6, 6)
         TIK_MMA_SS_STEP(64, 1024) TIK_MMA_SS_STEP(66, 1026) TIK_MMA_SS_STEP(68, 1028)
         TIK_MMA_SS_STEP(70, 1030)
@@ -65,7 +65,7 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     constexpr uint32_t IDESC_QK = mma_idesc_bf16(128, 128, false);
     constexpr uint32_t IDESC_PV = mma_idesc_bf16(128, D, true);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     pdl_wait();
     pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid's last wave
 
@@ -78,9 +78,9 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
     const int chunk0 = blockIdx.x * p.cpc;                      // a CTA streams cpc consecutive chunks
     if (ctx <= 0 || chunk0 * CHUNK >= ctx) return;
-    const int tile_first = chunk0 * TILES_PER_CHUNK;
+    const int tile_first = chunk0 * TILES_PER_CHUNK, tile_first_v = tile_first;
     const int tile_last = min(tile_first + p.cpc * TILES_PER_CHUNK - 1, (ctx - 1) / 128);
-    const int n_tiles = tile_last - tile_first + 1;
+    const int n_tiles = tile_last - tile_first + 1, n_tiles_v = n_tiles;
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw;
@@ -180,8 +180,10 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            mbar_wait(bar_q, 0, abort_word, p.dev_status);
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            const int n_tiles = warp_uniform(n_tiles_v), tile_first = warp_uniform(tile_first_v);
+            mbar_wait_warp(bar_q, 0, abort_word, p.dev_status);
             const uint64_t dq = smem_desc_sw128(sQ, 0, 0);      // stride 0 between 8-row groups: every group reads rows 0..7
             for (int it = 0; it < n_tiles; ++it) {
                 if (*abort_word) break;
@@ -189,7 +191,7 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const int sk = nk % DC_SLOTS, sv = nv % DC_SLOTS;
                 // scores: the previous tile's PV (issued by this thread, executed in order) has read
                 // the weights that these scores overwrite
-                mbar_wait(bar_full + 8 * sk, (nk / DC_SLOTS) & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_full + 8 * sk, (nk / DC_SLOTS) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 const uint64_t dk = smem_desc_sw128(sRing + sk * L::TILE, 0, 1024);
                 if (D == 128) mma_ss_chain8_fresh_qcompact(tmem + COL_S, dq, dk, IDESC_QK);
@@ -197,8 +199,8 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 mma_commit(bar_sfull);
                 mma_commit(bar_empty + 8 * sk);
                 // values
-                mbar_wait(bar_full + 8 * sv, (nv / DC_SLOTS) & 1, abort_word, p.dev_status);
-                mbar_wait(bar_pfull, it & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_full + 8 * sv, (nv / DC_SLOTS) & 1, abort_word, p.dev_status);
+                mbar_wait_warp(bar_pfull, it & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 const bool fresh = ((tile_first + it) % TILES_PER_CHUNK) == 0;
                 mma_ts_chain8(tmem + COL_O, tmem + COL_S, smem_desc_sw128(sRing + sv * L::TILE, L::ATOM, 1024),

@@ -43,7 +43,7 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, OFF_STG = C::OFF_STG, OFF_BAR = C::OFF_BAR;
     constexpr uint32_t TMEM_COLS = 512;      // two 256-column accumulators
     constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : 128, NB, false);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;     // 0 = the CTA that issues the pair's MMAs
 
     // raster: bands of BAND row tiles; within a band the row tile varies fastest so the CTAs in
@@ -155,17 +155,18 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
             uint32_t it = 0;
             for (int nt = 0; nt < n_nt; ++nt) {
                 const int buf = nt & 1;
                 const uint32_t use = nt >> 1;
-                if (use > 0) mbar_wait(bar_acc_empty + 8 * buf, (use - 1) & 1, abort_word, p.dev_status);
+                if (use > 0) mbar_wait_warp(bar_acc_empty + 8 * buf, (use - 1) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 for (int kb = 0; kb < n_kb; ++kb, ++it) {
                     if (*abort_word) break;
                     const int s = it % STAGES;
-                    mbar_wait(bar_full + 8 * s, (it / STAGES) & 1, abort_word, p.dev_status);
+                    mbar_wait_warp(bar_full + 8 * s, (it / STAGES) & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     const uint32_t a0 = sbase + s * STAGE_BYTES, b0 = a0 + A_BYTES;
                     if (PAIR) {
@@ -276,7 +277,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                    const __grid_constant__ CUtensorMap tmY, const LinearParams p) {
     using namespace linu;
     constexpr uint32_t TMEM_COLS = 512;      // two accumulators, 256 columns apart
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int nu = p.nu;
     const uint32_t a_bytes = static_cast<uint32_t>(p.a_rows) * 128u;
     const uint32_t slice_bytes = a_bytes + static_cast<uint32_t>(nu) * 128u;      // a multiple of 1 KiB
@@ -360,17 +361,18 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
             int s = 0;
             uint32_t use = 0;
             for (int i = 0; i < n_my; ++i) {
                 const int buf = i & 1;
                 const uint32_t acc_use = i >> 1;
-                if (acc_use > 0) mbar_wait(bar_acc_empty + 8 * buf, (acc_use - 1) & 1, abort_word, p.dev_status);
+                if (acc_use > 0) mbar_wait_warp(bar_acc_empty + 8 * buf, (acc_use - 1) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 for (int kb = 0; kb < n_kb; kb += kps) {
                     if (*abort_word) break;
-                    mbar_wait(bar_full + 8 * s, use & 1, abort_word, p.dev_status);
+                    mbar_wait_warp(bar_full + 8 * s, use & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     const uint32_t a0 = sbase + s * stage_bytes, b0 = a0 + a_bytes;
                     const int ns = min(kps, n_kb - kb);

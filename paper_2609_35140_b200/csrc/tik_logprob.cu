@@ -46,7 +46,7 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, OFF_BAR = C::OFF_BAR;
     constexpr uint32_t TMEM_COLS = 512;      // two 256-column accumulators
     constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : 128, NB, false);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;     // 0 = the CTA that issues the pair's MMAs
 
     // raster: bands of BAND token tiles; within a band the token tile varies fastest so the
@@ -175,19 +175,20 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
             uint32_t it = 0, acc = 0;              // acc counts accumulator steps across super-chunks
             const int n_sp_loop = unit_mode ? n_my_units : n_sp;
             for (int sp = 0; sp < n_sp_loop; ++sp)
             for (int nt = 0; nt < (unit_mode ? 1 : n_nt_of(sp)); ++nt, ++acc) {
                 const int buf = acc & 1;
                 const uint32_t use = acc >> 1;
-                if (use > 0) mbar_wait(bar_acc_empty + 8 * buf, (use - 1) & 1, abort_word, p.dev_status);
+                if (use > 0) mbar_wait_warp(bar_acc_empty + 8 * buf, (use - 1) & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 for (int kb = 0; kb < n_kb; ++kb, ++it) {
                     if (*abort_word) break;
                     const int s = it % STAGES;
-                    mbar_wait(bar_full + 8 * s, (it / STAGES) & 1, abort_word, p.dev_status);
+                    mbar_wait_warp(bar_full + 8 * s, (it / STAGES) & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     const uint32_t a0 = sbase + s * STAGE_BYTES, b0 = a0 + A_BYTES;
                     if (PAIR) {

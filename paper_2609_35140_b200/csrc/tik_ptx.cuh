@@ -25,13 +25,6 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(pred));
-    return pred != 0;
-}
 
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -75,6 +68,16 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity,
         }
     }
 }
+
+// The same for a converged warp (the issuing warps): every lane waits, all leave together.
+__device__ __forceinline__ void mbar_wait_warp(uint32_t bar, uint32_t parity,
+                                               volatile int* abort_word, int* dev_status) {
+    mbar_wait(bar, parity, abort_word, dev_status);
+    __syncwarp();
+}
+// A value that is the same in all lanes, in a form the compiler knows to be (uniform registers).
+__device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while its
@@ -253,24 +256,6 @@ __host__ __device__ constexpr uint32_t mma_idesc_bf16(int M, int N, bool b_mn_ma
     return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) |
            (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]; accumulate != 0 keeps the existing D.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                       uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]: A is 128 lanes x 8 columns, two consecutive-K bf16 per column.
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 // Named barriers (ids 1..15; 0 is __syncthreads): producer side arrives, consumer side syncs.
 __device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -278,22 +263,27 @@ __device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t nthreads)
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-// ---- MMA chains issued from one asm block.  The issuing thread's own instruction stream
-// limits how fast MMAs enter the tensor pipe, so a chain spends two 64-bit adds per MMA on
-// descriptor stepping and nothing else.  Offsets are in descriptor units (16 bytes).
+// ---- MMA chains issued from one asm block.  The issuing warp's own instruction stream limits how fast
+// MMAs enter the tensor pipe.  tcgen05 instructions take their operands from the warp's uniform
+// registers, so the WHOLE warp, converged, executes the issue path -- waits (mbar_wait_warp), descriptor
+// arithmetic on warp-uniform values, chains, commits -- and one elected lane issues.  With the path
+// inside `if (lane == 0)` every operand of every MMA was moved over from per-thread registers:
+// stand-alone, a chain of eight M128 x N128 x K16 with two barrier waits and two commits took 1485 clk of
+// issue that way and takes 824 this way (512 clk of MMAs); a chain alone 798 -> 627.
+// Offsets are in descriptor units (16 bytes).
 #define TIK_MMA_SS_STEP(OFFA, OFFB)                                   \
     "add.u64 da, %1, " #OFFA ";\n\t"                                  \
     "add.u64 db, %2, " #OFFB ";\n\t"                                  \
-    "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, pt;\n\t"
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, pt;\n\t"
 
 // K-major A and B, 64-wide K slice inside one 128B-swizzle atom: 4 steps of 32 bytes.
 // first_accumulate == 0 makes the first MMA overwrite D.
 __device__ __forceinline__ void mma_ss_chain4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                               uint32_t idesc, uint32_t first_accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 da, db;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
         "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
         TIK_MMA_SS_STEP(2, 2) TIK_MMA_SS_STEP(4, 4) TIK_MMA_SS_STEP(6, 6)
         "}" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(first_accumulate)
         : "memory");
@@ -302,9 +292,9 @@ __device__ __forceinline__ void mma_ss_chain4(uint32_t d_tmem, uint64_t a_desc, 
 __device__ __forceinline__ void mma_ss_chain8_fresh(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                                     uint32_t idesc) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 da, db;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
         "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
         TIK_MMA_SS_STEP(2, 2) TIK_MMA_SS_STEP(4, 4) TIK_MMA_SS_STEP(6, 6)
         TIK_MMA_SS_STEP(1024, 1024) TIK_MMA_SS_STEP(1026, 1026) TIK_MMA_SS_STEP(1028, 1028)
         TIK_MMA_SS_STEP(1030, 1030)
@@ -321,13 +311,13 @@ __device__ __forceinline__ void mma_ss_chain4_fresh(uint32_t d_tmem, uint64_t a_
 #define TIK_MMA_TS_STEP(OFFA, OFFB)                                   \
     "add.u32 ta, %1, " #OFFA ";\n\t"                                  \
     "add.u64 db, %2, " #OFFB ";\n\t"                                  \
-    "tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %3, pt;\n\t"
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %3, pt;\n\t"
 __device__ __forceinline__ void mma_ts_chain8(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                               uint32_t idesc, uint32_t first_accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
         "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
         TIK_MMA_TS_STEP(8, 128) TIK_MMA_TS_STEP(16, 256) TIK_MMA_TS_STEP(24, 384)
         TIK_MMA_TS_STEP(32, 512) TIK_MMA_TS_STEP(40, 640) TIK_MMA_TS_STEP(48, 768)
         TIK_MMA_TS_STEP(56, 896)
@@ -339,9 +329,9 @@ __device__ __forceinline__ void mma_ts_chain8(uint32_t d_tmem, uint32_t a_tmem, 
 __device__ __forceinline__ void mma_ts_chain4(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                               uint32_t idesc, uint32_t first_accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
         "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
         TIK_MMA_TS_STEP(8, 128) TIK_MMA_TS_STEP(16, 256) TIK_MMA_TS_STEP(24, 384)
         "}" ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(first_accumulate)
         : "memory");
@@ -353,9 +343,9 @@ __device__ __forceinline__ void mma_ts_chain4(uint32_t d_tmem, uint32_t a_tmem, 
 __device__ __forceinline__ void mma_ts_chain8_blocks(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                                      uint32_t idesc, uint32_t first_accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
         "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
         TIK_MMA_TS_STEP(8, 128) TIK_MMA_TS_STEP(32, 256) TIK_MMA_TS_STEP(40, 384)
         TIK_MMA_TS_STEP(64, 512) TIK_MMA_TS_STEP(72, 640) TIK_MMA_TS_STEP(96, 768)
         TIK_MMA_TS_STEP(104, 896)
@@ -411,29 +401,33 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 __device__ __forceinline__ void mma_ss_chain4_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                                    uint32_t idesc, uint32_t first_accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, pt;\n\t.reg .b64 da, db;\n\t"
+        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
         "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p0;\n\t"
         "add.u64 da, %1, 2;\n\tadd.u64 db, %2, 2;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
         "add.u64 da, %1, 4;\n\tadd.u64 db, %2, 4;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
         "add.u64 da, %1, 6;\n\tadd.u64 db, %2, 6;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, pt;\n\t"
         "}" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(first_accumulate)
         : "memory");
 }
 // Arrives on one mbarrier (of either CTA: a shared::cluster address) once all pair MMAs issued so
-// far by this thread have completed.
+// far by this warp have completed.
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar_cluster_addr) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster_addr)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar_cluster_addr)
+        : "memory");
 }
 
-// Arrives on the mbarrier once all MMAs issued so far by this thread have completed.
+// Arrives on the mbarrier once all MMAs issued so far by this warp (its elected lane) have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 }  // namespace tik
