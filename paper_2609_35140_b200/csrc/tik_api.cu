@@ -613,6 +613,29 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     if (T >= (1ll << 31) - 128) return fail(ctx, TIK_ERR_UNSUPPORTED, "T must be < 2^31 - 128");
     CUtensorMap tmA, tmB;
     std::string err;
+    if (T <= 80 && N <= 64ll * ctx->sm_count) {     // see linear_narrow_kernel
+        LinearParams p{};
+        p.y = static_cast<__nv_bfloat16*>(y);
+        p.T = T;
+        p.K = K;
+        p.N = N;
+        p.dev_status = ctx->dev_status;
+        p.nu = 8 * ((N + 8 * ctx->sm_count - 1) / (8 * ctx->sm_count));     // weight rows per CTA: whole 8-row swizzle atoms
+        p.nunit = (N + p.nu - 1) / p.nu;
+        p.a_rows = 16 * ((static_cast<int>(T) + 15) / 16);
+        // as many K slices per stage (one barrier round trip of the issuing thread) as leave four stages
+        p.kps = 8;
+        while (p.kps > 1 && (p.kps > K / 64 || LINEAR_NARROW_RING / ((p.nu + p.a_rows) * 128u * p.kps) < 4)) p.kps /= 2;
+        const uint64_t st3[2] = {static_cast<uint64_t>(K) * 2, 128};
+        const uint64_t wd[3] = {64, static_cast<uint64_t>(N), static_cast<uint64_t>(K / 64)};
+        const uint64_t xd[3] = {64, static_cast<uint64_t>(T), static_cast<uint64_t>(K / 64)};
+        const uint32_t boxW[3] = {64, static_cast<uint32_t>(p.nu), static_cast<uint32_t>(p.kps)};
+        const uint32_t boxX[3] = {64, static_cast<uint32_t>(p.a_rows), static_cast<uint32_t>(p.kps)};
+        if (!make_tmap_bf16(ctx, &tmA, weight, 3, wd, st3, boxW, &err) || !make_tmap_bf16(ctx, &tmB, x, 3, xd, st3, boxX, &err))
+            return fail(ctx, TIK_ERR_CUDA, err.c_str());
+        cudaError_t e = launch_linear_narrow(tmA, tmB, p, static_cast<cudaStream_t>(stream));
+        return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_linear");
+    }
     uint64_t ad[2] = {static_cast<uint64_t>(K), static_cast<uint64_t>(T)};
     uint64_t bd[2] = {static_cast<uint64_t>(K), static_cast<uint64_t>(N)};
     uint64_t st1[1] = {static_cast<uint64_t>(K) * 2};

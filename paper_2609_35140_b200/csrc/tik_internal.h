@@ -208,6 +208,8 @@ struct LinearParams {
     int unit_mode;               // T <= 128: persistent CTAs over column units (tmA box a_rows, tmB box nu rows)
     int ntp;                     // pair unit mode: pairs of row tiles (1 .. 8)
     int nu, nunit, a_rows;       // unit width 64 / 128 / 256, ceil(N / nu), staged x rows 32 / 64 / 128
+                                 // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 16 .. 80)
+    int kps;                     // narrow outputs: K slices per ring stage
     int sm_count;
     int* dev_status;
 };
@@ -240,6 +242,9 @@ inline int linear_unit_cols(int N, int a_rows, int sm_count) {
     }
     return best;
 }
+// T <= 80 and N <= 64 sm_count; tmW / tmX: [K / 64][rows][64] views with boxes of 64 x nu x kps and 64 x a_rows x kps
+constexpr uint32_t LINEAR_NARROW_RING = 192 * 1024;
+cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX, const LinearParams& p, cudaStream_t stream);
 cudaError_t launch_linear(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,
                           const LinearParams& p, bool pair, cudaStream_t stream);
 

@@ -455,6 +455,160 @@ static cudaError_t launch_linear_unit(const CUtensorMap& tmA, const CUtensorMap&
     return launch_pdl(linear_unit_kernel, dim3(grid), lin::THREADS, linu::ALLOC, stream, 1, tmA, tmB, tmY, p);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Decode-shaped calls with a narrow output (T <= 80 and N <= 64 columns per SM: the down, q, k, v and
+// output projections of a rollout step).  linear_unit_kernel gives such a call at most N / 64 CTAs, each
+// pulling 64 weight rows and at least 32 x rows per K slice at the ~95 GB/s that one SM takes in; K is not
+// split (an element is one chain), so the way to shorten the call is fewer rows per CTA on more SMs.
+// Here the weights are the MMA's M operand -- M64, of which a CTA stages only its r = 8, 16, .. 64 rows, as
+// few as spread N over all SMs -- and x, rounded up to 16 rows, its N operand: an MMA reads 64 + T
+// shared-memory rows instead of 128 + 64.  The products of an element and the order of its sums are
+// those of the other schedules (operands exchanged), so are the bits.
+// Ring: stages of kps K slices; one TMA copy per operand and stage through a [K / 64][rows][64] view.
+// linear_unit_kernel -> this, cold L2: T = 16: K 8960, N 1536 28.5 -> 20.5 us; K 18944, N 3584 51 -> 33;
+// K 27648, N 5120 72 -> 51; T = 64: 28.6 -> 24.7, 51 -> 41, 74 -> 74.  At T = 128 x is most of what a CTA
+// takes in, on more CTAs here: 30.7 -> 34.8, 59 -> 62, 84 -> 86; at 80: 30.7 -> 26.7, 57.4 -> 53.3,
+// 82 -> 76; the line is drawn there.
+namespace linn {
+constexpr uint32_t RING_BYTES = LINEAR_NARROW_RING;
+constexpr int MAX_STAGES = 12;
+constexpr uint32_t OFF_BAR = RING_BYTES + 64 * 128;      // (a slice's M64 read may run past its r rows: never past this)
+constexpr uint32_t BYTES = OFF_BAR + 512;
+constexpr uint32_t ALLOC = BYTES + 1024;
+}  // namespace linn
+
+__global__ void __launch_bounds__(lin::THREADS, 1)
+linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const LinearParams p) {
+    using namespace linn;
+    constexpr uint32_t TMEM_COLS = 128;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    const int r = p.nu, kps = p.kps, n_kb = p.K / 64, n0 = static_cast<int>(blockIdx.x) * r;
+    const uint32_t w_slice = static_cast<uint32_t>(r) * 128u, x_slice = static_cast<uint32_t>(p.a_rows) * 128u;
+    const uint32_t w_bytes = w_slice * static_cast<uint32_t>(kps);
+    const uint32_t stage_bytes = w_bytes + x_slice * static_cast<uint32_t>(kps);
+    const int nst = min(MAX_STAGES, static_cast<int>(RING_BYTES / stage_bytes));
+    const uint32_t idesc = mma_idesc_bf16(64, p.a_rows, false);
+
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    const uint32_t pad = (1024u - (raw_addr & 1023u)) & 1023u;
+    uint8_t* smem = smem_raw + pad;
+    const uint32_t sbase = raw_addr + pad;
+    const uint32_t bar_full = sbase + OFF_BAR;                   // MAX_STAGES barriers
+    const uint32_t bar_empty = bar_full + 8 * MAX_STAGES;        // MAX_STAGES barriers
+    const uint32_t bar_acc = bar_empty + 8 * MAX_STAGES;
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + OFF_BAR + 8 * (2 * MAX_STAGES + 1));
+    volatile int* abort_word = reinterpret_cast<volatile int*>(smem + OFF_BAR + 8 * (2 * MAX_STAGES + 1) + 4);
+
+    if (tid == 0) {
+        for (int s = 0; s < MAX_STAGES; ++s) {
+            mbar_init(bar_full + 8 * s, 1);
+            mbar_init(bar_empty + 8 * s, 1);
+        }
+        mbar_init(bar_acc, 1);
+        fence_barrier_init();
+        tma_prefetch_desc(&tmW);
+        tma_prefetch_desc(&tmX);
+        // the first 256 KiB of this CTA's weights on their way to L2 while the kernel before this one drains
+        const int ahead = min(n_kb, static_cast<int>((256u * 1024u) / w_slice));
+        for (int kb = 0; kb < ahead; kb += kps) tma_prefetch_l2_3d(&tmW, 0, n0, kb);
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
+        tmem_relinquish();
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer
+        if (lane == 0) {
+            int s = 0;
+            uint32_t use = 0;                    // how often stage s has been filled before
+            for (int kb = 0; kb < n_kb; kb += kps) {
+                if (*abort_word) break;
+                if (use > 0) mbar_wait(bar_empty + 8 * s, (use - 1) & 1, abort_word, p.dev_status);
+                const uint32_t dst = sbase + s * stage_bytes;
+                // W rows past N, x rows past T and slices past K arrive as zeros
+                mbar_expect_tx(bar_full + 8 * s, stage_bytes);
+                tma_load_3d(dst, &tmW, bar_full + 8 * s, 0, n0, kb);
+                tma_load_3d(dst + w_bytes, &tmX, bar_full + 8 * s, 0, 0, kb);
+                if (++s == nst) {
+                    s = 0;
+                    ++use;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer
+        {
+            const uint32_t tmem = warp_uniform(*tmem_slot);
+            int s = 0;
+            uint32_t use = 0;
+            for (int kb = 0; kb < n_kb; kb += kps) {
+                if (*abort_word) break;
+                mbar_wait_warp(bar_full + 8 * s, use & 1, abort_word, p.dev_status);
+                tc_fence_after();
+                const uint32_t a0 = sbase + s * stage_bytes, b0 = a0 + w_bytes;
+                const int ns = min(kps, n_kb - kb);
+                for (int sl = 0; sl < ns; ++sl)
+                    mma_ss_chain4(tmem, smem_desc_sw128(a0 + sl * w_slice, 0, 1024), smem_desc_sw128(b0 + sl * x_slice, 0, 1024),
+                                  idesc, (kb + sl) ? 1u : 0u);
+                mma_commit(bar_empty + 8 * s);
+                if (++s == nst) {
+                    s = 0;
+                    ++use;
+                }
+            }
+            mma_commit(bar_acc);
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue (warps 2..5)
+        // An M64 accumulator has 16 rows (output columns) in each lane quarter; a column of it is a row of x.
+        const int quarter = warp & 3;
+        const int m = 16 * quarter + lane;
+        const bool valid = lane < 16 && m < r && n0 + m < p.N;
+        mbar_wait(bar_acc, 0, abort_word, p.dev_status);
+        tc_fence_after();
+        if (16 * quarter < r) {
+            for (int c0 = 0; c0 < static_cast<int>(p.T); c0 += 32) {
+                uint32_t v[32];
+                tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, v);
+                tmem_wait_ld();
+                __nv_bfloat16* const y = p.y + static_cast<long long>(c0) * p.N + n0 + m;
+                const int nt = min(32, static_cast<int>(p.T) - c0);
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    if (valid && i < nt) y[static_cast<long long>(i) * p.N] = __float2bfloat16_rn(__uint_as_float(v[i]));
+            }
+        }
+    }
+
+    if (*abort_word) {   // let copies and MMAs in flight finish before shared memory and TMEM are released
+        const unsigned long long t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 1000000ull) {
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+}
+
+cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX, const LinearParams& p, cudaStream_t stream) {
+    static DeviceOnce configured;
+    cudaError_t e = configured.run([&]() {
+        return cudaFuncSetAttribute(linear_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(linn::ALLOC));
+    });
+    if (e != cudaSuccess) return e;
+    return launch_pdl(linear_narrow_kernel, dim3(static_cast<unsigned>(p.nunit)), lin::THREADS, linn::ALLOC, stream, 1, tmW, tmX, p);
+}
+
 template <bool PAIR>
 static cudaError_t launch_linear_t(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,
                                    const LinearParams& p, cudaStream_t stream) {

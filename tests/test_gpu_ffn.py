@@ -162,3 +162,22 @@ def test_ffn_invalid_arguments(tik):
     with pytest.raises(tik.TikError):
         tik.tik_swiglu(_randn((4, 24), 1))                                    # I % 8
     assert tik.tik_linear(x[:0], _randn((8, 64), 2)).shape == (0, 8)
+
+
+@pytest.mark.parametrize("K,N", [(64, 8), (576, 1184), (576, 1192), (4096, 1536), (1024, 3584), (320, 9472), (256, 9480)])
+def test_narrow_linear_equals_rows_of_a_batched_call(tik, K, N):
+    """T <= 80 and N <= 64 columns per SM: weights as the M operand, 8 .. 64 rows of them per CTA.  Row counts
+    around the multiples of 16 that are staged, K tails of a ring stage, outputs of one CTA, of whole and ragged
+    last CTAs, and the first N beyond the range: the bits of a batched call, nothing written outside y."""
+    x = _randn((300, K), 3100 + K)
+    W = _randn((N, K), 3200 + N % 977, 0.02)
+    y = tik.tik_linear(x, W)
+    ref = oracle.linear(x[:3].float().cpu().numpy(), W.float().cpu().numpy())
+    g = y[:3].float().cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(g - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4 * 0.02 * np.sqrt(K))
+    for a, T in [(0, 1), (5, 15), (7, 16), (9, 17), (100, 32), (3, 48), (50, 65), (171, 80), (160, 81), (172, 97)]:
+        buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
+        tik.tik_linear(x[a:a + T].contiguous(), W, y=buf[1:T + 1])
+        assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
+        assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
+    assert tik.device_status() == 0
