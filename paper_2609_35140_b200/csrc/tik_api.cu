@@ -17,7 +17,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapFloatOOBfill);
 
 bool make_tmap_bf16(tik_ctx* ctx, CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                    const uint64_t* strides_bytes, const uint32_t* box, std::string* err) {
+                    const uint64_t* strides_bytes, const uint32_t* box, std::string* err, bool swizzle64) {
     cuuint64_t gdim[5], gstr[4];
     cuuint32_t bdim[5], estr[5];
     for (int i = 0; i < rank; ++i) {
@@ -28,7 +28,7 @@ bool make_tmap_bf16(tik_ctx* ctx, CUtensorMap* out, const void* base, int rank, 
     }
     CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
         out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, static_cast<cuuint32_t>(rank), const_cast<void*>(base), gdim,
-        gstr, bdim, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        gstr, bdim, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         char buf[256];
@@ -83,6 +83,18 @@ static bool use_persistent(const void* ws, size_t ws_bytes, int S, int max_posit
     // fewer work items than two per SM: nothing to amortise, the planning launch only adds latency
     if (static_cast<long long>(S) * X * Hq <= 2ll * sm_count) return false;
     return ws_bytes >= attn_plan_bytes(S, max_positions);
+}
+
+// CTAs per chunk for decode calls that leave most SMs idle (tik_decode_cluster.cu), 0: the other kernels.
+// chunks: (sequence, KV head, chunk) items by the host's bound.  A cluster pays while all of them run at
+// once (5 x 8 chunks in clusters of four, a second wave: 16.8 -> 25 us) and the contexts are longer than
+// its set-up (1000 keys 10.4 -> 9.1 us, 500 7.6 -> 7.3, 128 5.3 -> 6.5).  Two CTAs per chunk stop at a third of
+// the SMs' number of chunks: beyond it a call whose keys are not in L2 is bound by HBM and gains nothing
+// (16 x 2000 x 4 keys, cold: 22.6 -> 24.6 us, in L2: 16.7 -> 14.9).
+static int decode_cluster_size(long long chunks, int max_ctx, int G, int d, int sm_count) {
+    if (G > DECODE2_MAX_G || max_ctx <= 512) return 0;
+    if (d == 128 && 4 * chunks <= sm_count) return 4;
+    return 3 * chunks <= sm_count ? 2 : 0;
 }
 
 static tik_status check_heads(tik_ctx* ctx, int Hq, int Hkv, int d, float scale) {
@@ -289,16 +301,18 @@ tik_status tik_kv_cache_write(tik_ctx* ctx, const void* k_new, const void* v_new
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_kv_cache_write");
 }
 
+// v_cols: columns per V copy (64, or 32 with the 64-byte swizzle)
 static tik_status make_cache_maps(tik_ctx* ctx, const void* k_cache, const void* v_cache, int Hkv, int d,
-                                  int page_size, int num_pages, CUtensorMap* tmK, CUtensorMap* tmV) {
+                                  int page_size, int num_pages, CUtensorMap* tmK, CUtensorMap* tmV, int v_cols = 64) {
     std::string err;
     const uint64_t ud = static_cast<uint64_t>(d);
     uint64_t cd[4] = {ud, static_cast<uint64_t>(page_size), static_cast<uint64_t>(Hkv),
                       static_cast<uint64_t>(num_pages)};
     uint64_t cs[3] = {ud * 2, ud * 2 * page_size, ud * 2 * page_size * Hkv};
     uint32_t box[4] = {64, static_cast<uint32_t>(page_size), 1, 1};
+    uint32_t boxv[4] = {static_cast<uint32_t>(v_cols), static_cast<uint32_t>(page_size), 1, 1};
     if (!make_tmap_bf16(ctx, tmK, k_cache, 4, cd, cs, box, &err) ||
-        !make_tmap_bf16(ctx, tmV, v_cache, 4, cd, cs, box, &err))
+        !make_tmap_bf16(ctx, tmV, v_cache, 4, cd, cs, boxv, &err, v_cols == 32))
         return fail(ctx, TIK_ERR_CUDA, err.c_str());
     return TIK_OK;
 }
@@ -413,10 +427,12 @@ tik_status tik_attn_decode(tik_ctx* ctx, const void* q, void* o, float* lse, con
     uint64_t qs[2] = {ud * 2, ud * 2 * Hq};
     uint32_t box[3] = {64, static_cast<uint32_t>(G), 1};
     if (!make_tmap_bf16(ctx, &tmQ, q, 3, qd, qs, box, &err)) return fail(ctx, TIK_ERR_CUDA, err.c_str());
-    s = make_cache_maps(ctx, k_cache, v_cache, Hkv, d, page_size, num_pages, &tmK, &tmV);
+    const int nchunk = (max_ctx_len + CHUNK - 1) / CHUNK;
+    const long long pairs = static_cast<long long>(B) * Hkv;
+    const int cluster = decode_cluster_size(pairs * nchunk, max_ctx_len, G, d, ctx->sm_count);
+    s = make_cache_maps(ctx, k_cache, v_cache, Hkv, d, page_size, num_pages, &tmK, &tmV, cluster ? d / cluster : 64);
     if (s != TIK_OK) return s;
 
-    const int nchunk = (max_ctx_len + CHUNK - 1) / CHUNK;
     AttnParams p{};
     p.o = o;
     p.lse = lse;
@@ -447,14 +463,14 @@ tik_status tik_attn_decode(tik_ctx* ctx, const void* q, void* o, float* lse, con
     // either way and the big kernel's faster per-CTA pipeline (two softmax warpgroups, five K/V
     // stages) gives the shorter latency; with many pairs of long contexts the same pipeline streams
     // faster per SM (the paper's decode grid, Sec. 6 Q3, covers both ends).
-    const long long pairs = static_cast<long long>(B) * Hkv;
     const bool small_group = G <= DECODE2_MAX_G && (pairs <= ctx->sm_count || nchunk <= 2) && 4 * pairs * nchunk >= 3ll * ctx->sm_count;
     p.cpc = decode_chunks_per_cta(B, Hkv, nchunk, ctx->sm_count, small_group ? 2 : 1);
     p.lookahead = ctx->sm_count;
     dim3 grid((nchunk + p.cpc - 1) / p.cpc, Hkv, B);
     if (grid.y > 65535 || grid.z > 65535) return fail(ctx, TIK_ERR_UNSUPPORTED, "Hkv and B must be <= 65535");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = small_group ? launch_decode2(d, grid, tmQ, tmK, tmV, p, st) : launch_attn(d, 2, grid, tmQ, tmK, tmV, p, st);
+    cudaError_t e = cluster ? launch_decode_cluster(d, cluster, nchunk, Hkv, B, tmQ, tmK, tmV, p, st)
+                    : small_group ? launch_decode2(d, grid, tmQ, tmK, tmV, p, st) : launch_attn(d, 2, grid, tmQ, tmK, tmV, p, st);
     if (e == cudaSuccess && !p.direct_out) e = launch_combine(d, p, B, st);
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_decode");
 }

@@ -5,28 +5,30 @@
 // chunk) whatever the memory system could deliver.  Here C = 2 or 4 CTAs share a chunk.  What may be
 // split without touching the contract: score columns (a key's scores are one MMA chain of their own)
 // and output columns (a column of O is one chain over the keys of its own).  What may not: the chain of an
-// output element over the chunk's tiles, and the order of the row sums.  So, per cluster:
-//   1. scores: CTA r computes S = Q K^T of the tiles r, r + C, ...; every score row goes to the shared
-//      memory of all C CTAs (distributed shared memory: G rows x 512 B per tile, a remote mbarrier
-//      counts the warps that have written);
-//   2. softmax: with all scores of the chunk at hand nothing is serial but the sixteen-step recurrence of
-//      the reference maximum, so a thread takes one row's half tile: 64 exponentials, its half row sum,
-//      its bf16 weights.  Every CTA does all of it (G x 2048 exponentials are ~0.6 us);
+// output element over the chunk's tiles, and the order of the row sums.  So, tile by tile and pipelined:
+//   1. scores: CTA r computes S = Q K^T of the tiles r, r + C, ...; four transfer warps put every score row
+//      into the shared memory of all C CTAs (distributed shared memory, a remote mbarrier per tile);
+//   2. softmax: a warp takes two tiles, a thread one row's half tile: 64 exponentials, its half row
+//      sum, its bf16 weights.  Serial across tiles is only the recurrence of the reference maximum, over tile
+//      maxima that the warps publish.  Every CTA does all of it;
 //   3. values: CTA r accumulates O over all tiles in ascending order for its own D / C columns, so a CTA
 //      loads a C-th of V; weights come from shared memory, and the rare rescale of O between
-//      two tiles is known in advance.
-// Same tiles, same MMA chains over d and keys, same row-sum shape, same rescales, so same bits as every
-// other regime.  Query rows and weights are 8-row atoms read with a zero stride between row groups (see
-// tik_decode.cu); M64 MMAs suffice for G <= 8 rows.
+//      two tiles is known when the tile's weights are.
+// Every chunk leaves its partial for combine_kernel, or its rows when it is the only one.
+// Same tiles, same MMA chains over d and keys, same row-sum shape, same rescales, so same bits as
+// every other regime.  Query rows and weights are 8-row atoms read with a zero stride between row
+// groups (see tik_decode.cu); M64 MMAs suffice for G <= 8 rows.
+// Measured in a CUDA graph of back-to-back calls (one CTA per chunk -> this): one sequence of 2000 keys, 4 KV
+// heads x 7 16.5 -> 12.1 us, 4321 keys 17.8 -> 13.6, 4 x 2000 keys x 8 KV heads 16.9 -> 13.3 (C = 4);
+// 5 x 2000 x 8 16.8 -> 15.0 (C = 2).
 #include "tik_core.cuh"
 #include "tik_internal.h"
 #include "tik_ptx.cuh"
 
 namespace tik {
 
-constexpr int DX_SOFTMAX_WARPS = 8;
-constexpr int DX_THREADS = 32 * (DX_SOFTMAX_WARPS + 2);     // + warp 8 TMA, warp 9 MMA
-constexpr int DX_MAX_STAGES = 8;
+// warps 0-7 softmax, 8-11 transfer, 12 TMA, 13 MMA
+constexpr int DX_THREADS = 32 * 14;
 
 template <int D>
 struct DXSmem {
@@ -35,18 +37,19 @@ struct DXSmem {
     static constexpr uint32_t NU = (D == 128) ? 4 : 8;           // ring units (128 KiB)
     static constexpr uint32_t OFF_RING = 0;
     static constexpr uint32_t OFF_Q = NU * UNIT;                 // D / 64 atoms of 8 rows x 128 bytes
-    // scores: 8 rows of 2048 fp32, a row's pitch 16 bytes longer so that eight rows' 16-byte reads meet
-    // all banks; the weights (16 tiles x 2 atoms of 8 rows x 128 bytes) overlay them
-    static constexpr uint32_t S_PITCH = CHUNK * 4 + 16;
+    // scores of a tile: 8 rows of 128 fp32, the row pitch 16 bytes longer so that eight rows' 16-byte
+    // reads meet all banks; the tile's weights (2 atoms of 8 rows x 128 bytes) overlay them
+    static constexpr uint32_t S_PITCH = 128 * 4 + 16;
+    static constexpr uint32_t S_TILE = 5 * 1024;
     static constexpr uint32_t OFF_S = OFF_Q + (D / 64) * 1024;
-    static constexpr uint32_t OFF_TM = OFF_S + ((8 * S_PITCH + 1023) / 1024) * 1024;     // [16 tiles][8 rows] tile maxima
+    static constexpr uint32_t OFF_TM = OFF_S + TILES_PER_CHUNK * S_TILE;     // [16 tiles][8 rows] tile maxima
     static constexpr uint32_t OFF_AL = OFF_TM + 16 * 8 * 4;      // [16][8] rescale factors
     static constexpr uint32_t OFF_RS = OFF_AL + 16 * 8 * 4;      // [16][2][8] half row sums
     static constexpr uint32_t OFF_M = OFF_RS + 2 * 16 * 8 * 4;   // [8] last reference maximum
     static constexpr uint32_t OFF_FLAG = OFF_M + 8 * 4;          // [16] tiles before which O is rescaled
     static constexpr uint32_t OFF_TAB = OFF_FLAG + 16 * 4;       // [128] physical pages of the chunk
     static constexpr uint32_t OFF_BAR = OFF_TAB + 128 * 4;
-    static constexpr uint32_t BYTES = OFF_BAR + 256;
+    static constexpr uint32_t BYTES = OFF_BAR + 512;
 };
 
 __device__ __forceinline__ void st_cluster_f4(uint32_t addr, float a, float b, float c, float d) {
@@ -154,45 +157,56 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t bar_q = bar0 + 128;
     const uint32_t bar_sfull = bar0 + 136;       // [3] scores of an own tile in a score buffer
     const uint32_t bar_sfree = bar0 + 160;       // [3] ... and read from it (4 warps)
-    const uint32_t bar_all = bar0 + 184;         // score rows of all tiles of the chunk are in this CTA's shared memory
-    const uint32_t bar_p = bar0 + 192;           // weights written (8 warps)
-    const uint32_t bar_pv = bar0 + 200;          // PV up to a rescale, or the last one, done
-    const uint32_t bar_resc = bar0 + 208;        // O rescaled
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_BAR + 216);
-    volatile int* abort_word = reinterpret_cast<volatile int*>(smem + L::OFF_BAR + 220);
+    const uint32_t bar_tile = bar0 + 184;        // [16] score rows of a tile are in this CTA's shared memory (4 warps)
+    const uint32_t bar_tm = bar0 + 312;          // [8] maxima of a softmax warp's two tiles published
+    const uint32_t bar_p = bar0 + 376;           // [8] weights of a softmax warp's two tiles written
+    const uint32_t bar_pv = bar0 + 440;          // PV up to a rescale, or the last one, done
+    const uint32_t bar_resc = bar0 + 448;        // O rescaled
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_BAR + 456);
+    volatile int* abort_word = reinterpret_cast<volatile int*>(smem + L::OFF_BAR + 460);
     int* const tab = reinterpret_cast<int*>(smem + L::OFF_TAB);
 
     // ---------------------------------------------------------------- set-up that needs no input
-    if (warp == 8) {
+    if (warp == 12) {
         if (lane == 0) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmK);
             tma_prefetch_desc(&tmV);
-            for (int i = 0; i < 2 * DX_MAX_STAGES + 1; ++i) mbar_init(bar_full + 8 * i, 1);     // full, empty, q
-            for (int i = 0; i < NSB; ++i) {
-                mbar_init(bar_sfull + 8 * i, 1);
-                mbar_init(bar_sfree + 8 * i, 4);
-            }
-            mbar_init(bar_p, DX_SOFTMAX_WARPS);
-            mbar_init(bar_pv, 1);
-            mbar_init(bar_resc, 1);
-            fence_barrier_init();
         }
+        for (int i = lane; i < 57; i += 32) {
+            const bool four = (i >= 20 && i < 23) || (i >= 23 && i < 39);     // sfree, tile: four warps
+            mbar_init(bar0 + 8 * i, four ? 4 : 1);
+        }
+        fence_barrier_init();
         // rows >= G of the query atoms are never loaded
         for (uint32_t i = lane; i < NATOM * 1024 / 16; i += 32)
             reinterpret_cast<uint4*>(smem + L::OFF_Q)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
         __syncwarp();
-    } else if (warp == 9) {
+    } else if (warp == 13) {
         tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
         tmem_relinquish();
     }
     pdl_wait();
     pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid
+    if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
 
     const int seq = blockIdx.z, kvh = blockIdx.y, chunk = static_cast<int>(blockIdx.x) / C;
     const int rank = static_cast<int>(cluster_ctarank());
     const int head = kvh * p.G;
+    const int tile0 = chunk * TILES_PER_CHUNK;
+    if (warp == 12) {
+        // the query rows and the chunk's block-table entries do not wait for the context length
+        if (lane == 0) {
+            mbar_expect_tx(bar_q, static_cast<uint32_t>(p.G) * 128u * NATOM);
+            for (int a = 0; a < NATOM; ++a) tma_load_3d(sQ + a * 1024, &tmQ, bar_q, a * 64, head, seq);
+        }
+        for (int i = lane; i < (CHUNK >> p.page_shift); i += 32) {
+            const int lp = ((128 * tile0) >> p.page_shift) + i;
+            tab[i] = (lp < p.max_blocks) ? p.block_table[static_cast<long long>(seq) * p.max_blocks + lp] : -1;
+        }
+        __syncwarp();
+    }
     int ctx = warp_uniform(p.ctx_lens[seq]);
     if (ctx > p.max_ctx) {
         if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) atomicOr(p.dev_status, TIK_DEV_BAD_CONTEXT);
@@ -202,43 +216,42 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     if (idle) {
         if ((sbase & 1023u) != 0 && tid == 0) atomicOr(p.dev_status, TIK_DEV_WAIT_EXPIRED);
         __syncthreads();
-        if (warp == 9) tmem_dealloc(*tmem_slot, TMEM_COLS);
+        if (warp == 12) {
+            mbar_wait(bar_q, 0, abort_word, p.dev_status);     // its copy is in flight
+            if (*abort_word) {
+                const unsigned long long t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < 1000000ull) {
+                }
+            }
+        }
+        __syncthreads();
+        if (warp == 13) tmem_dealloc(*tmem_slot, TMEM_COLS);
         return;
     }
-    const int tile0 = chunk * TILES_PER_CHUNK;
     const int n_tiles = min(TILES_PER_CHUNK, (ctx - 1) / 128 - tile0 + 1);
     const int nk = (n_tiles - rank + C - 1) / C;               // own score tiles rank, rank + C, ... (0 when n_tiles <= rank)
     const int nv = (n_tiles + C - 1) / C;                      // V units of C tiles
-    if (tid == 0) {
-        mbar_init(bar_all, static_cast<uint32_t>(4 * n_tiles));
-        *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
-        fence_barrier_init();
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    cluster_arrive();                                          // this CTA's barriers exist
+    // Two cluster barriers: the first says that every CTA's mbarriers exist, the second that nobody
+    // writes to another CTA any more (a thread arrives there after its last remote write, all wait at the end).
+    cluster_arrive();
     const uint32_t tmem = warp_uniform(*tmem_slot);
 
-    if (warp == 8) {
-        // ------------------------------------------------------------ TMA: pages, query rows, K tiles, V columns
+    if (warp == 12) {
+        // ------------------------------------------------------------ TMA: K tiles, V columns
         for (int i = lane; i < (CHUNK >> p.page_shift); i += 32) {
-            const int lp = ((128 * tile0) >> p.page_shift) + i;
-            int ph = p.num_pages;       // out of range: the box is filled with zeros
-            if ((lp << p.page_shift) < ctx) {
-                ph = (lp < p.max_blocks) ? p.block_table[static_cast<long long>(seq) * p.max_blocks + lp] : -1;
-                if (ph < 0 || ph >= p.num_pages) {
-                    atomicOr(p.dev_status, TIK_DEV_BAD_BLOCK);
-                    ph = p.num_pages;
-                }
+            int ph = tab[i];
+            if ((((128 * tile0) >> p.page_shift) + i) << p.page_shift >= ctx) {
+                ph = p.num_pages;       // out of range: the box is filled with zeros
+            } else if (ph < 0 || ph >= p.num_pages) {
+                atomicOr(p.dev_status, TIK_DEV_BAD_BLOCK);
+                ph = p.num_pages;
             }
             tab[i] = ph;
         }
         __syncwarp();
-        if (lane == 0) {
-            mbar_expect_tx(bar_q, static_cast<uint32_t>(p.G) * 128u * NATOM);
-            for (int a = 0; a < NATOM; ++a) tma_load_3d(sQ + a * 1024, &tmQ, bar_q, a * 64, head, seq);
-        }
         const int my = lane & (p.pages_per_tile - 1);
         const uint32_t page_row = static_cast<uint32_t>(my << p.page_shift);
         for (int n = 0; n < nk + nv; ++n) {
@@ -267,7 +280,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         __syncwarp();
         cluster_wait();
         cluster_arrive();
-    } else if (warp == 9) {
+    } else if (warp == 13) {
         // ------------------------------------------------------------ MMA issuer (whole warp)
         cluster_wait();
         cluster_arrive();
@@ -285,13 +298,13 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             mma_commit(bar_sfull + 8 * b);
             mma_commit(bar_empty + 8 * u);
         }
-        mbar_wait_warp(bar_p, 0, abort_word, p.dev_status);
         const volatile int* flag = reinterpret_cast<const volatile int*>(smem + L::OFF_FLAG);
         int resc = 0;
         for (int t = 0; t < n_tiles; ++t) {
             if (*abort_word) break;
             const int n = nk + t / C, u = n % NU;
             if (t % C == 0) mbar_wait_warp(bar_full + 8 * u, (n / NU) & 1, abort_word, p.dev_status);
+            if (t % 2 == 0) mbar_wait_warp(bar_p + 8 * (t / 2), 0, abort_word, p.dev_status);
             if (warp_uniform(flag[t]) != 0) {
                 // O of the tiles before this one is complete, then rescaled by warp 0
                 mma_commit(bar_pv);
@@ -299,30 +312,29 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 ++resc;
             }
             tc_fence_after();
-            const uint64_t dp = smem_desc_sw128(sS + t * 2048, 0, 0);
+            const uint64_t dp = smem_desc_sw128(sS + t * L::S_TILE, 0, 0);
             const uint32_t v = sRing + u * L::UNIT + (t % C) * VBYTES;
             if (VC == 64) mma_ss_chain8_compact_v64(tmem + COL_O, dp, smem_desc_sw128(v, L::ATOM, 1024), IDESC_PV, t > 0 ? 1u : 0u);
             else mma_ss_chain8_compact_v32(tmem + COL_O, dp, smem_desc_sw64(v, 8192, 512), IDESC_PV, t > 0 ? 1u : 0u);
             if (t % C == C - 1 || t == n_tiles - 1) mma_commit(bar_empty + 8 * u);
         }
         mma_commit(bar_pv);
-    } else {
-        // ------------------------------------------------------------ scores of the own tiles to all CTAs
+    } else if (warp >= 8) {
+        // ------------------------------------------------------------ transfer: scores of the own tiles to all CTAs
         // M64 accumulator: row i of the query group on lanes i and i + 8 of every quarter (row groups
-        // repeat).  Warp `quarter` of group g reads 32 columns of the own tiles g, g + 2, ...; lanes 0-7 write
-        // columns 0..15 of them, lanes 8-15 columns 16..31, to the same place in every CTA.
-        const int quarter = warp & 3, grp = warp >> 2;
+        // repeat).  Warp `quarter` reads 32 columns; lanes 0-7 write columns 0..15 of them, lanes 8-15
+        // columns 16..31, to the same place in every CTA.
+        const int quarter = warp & 3;
         const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const int row = lane & 7, hi = (lane >> 3) & 1;
         const bool writer = lane < 16 && row < p.G;
-        uint32_t dst[C], all[C];
+        uint32_t dst[C];
 #pragma unroll
-        for (int k = 0; k < C; ++k) {
+        for (int k = 0; k < C; ++k)
             dst[k] = mapa_cluster(sS, static_cast<uint32_t>(k)) + row * L::S_PITCH + quarter * 128u + hi * 64u;
-            all[k] = mapa_cluster(bar_all, static_cast<uint32_t>(k));
-        }
+        const uint32_t my_bar = mapa_cluster(bar_tile, static_cast<uint32_t>(lane < C ? lane : 0));
         cluster_wait();                                        // the other CTAs' barriers exist
-        for (int i = grp; i < nk; i += 2) {
+        for (int i = 0; i < nk; ++i) {
             const int b = i % NSB, t = rank + i * C;
             mbar_wait_warp(bar_sfull + 8 * b, (i / NSB) & 1, abort_word, p.dev_status);
             tc_fence_after();
@@ -343,84 +355,90 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
                 for (int k = 0; k < C; ++k)
 #pragma unroll
-                    for (int j = 0; j < 16; j += 4) st_cluster_f4(dst[k] + t * 512u + 4u * j, x[j], x[j + 1], x[j + 2], x[j + 3]);
+                    for (int j = 0; j < 16; j += 4)
+                        st_cluster_f4(dst[k] + t * L::S_TILE + 4u * j, x[j], x[j + 1], x[j + 2], x[j + 3]);
             }
             __syncwarp();
-            if (lane < C) {
-                uint32_t bar = all[0];
-#pragma unroll
-                for (int k = 1; k < C; ++k)
-                    if (lane == k) bar = all[k];
-                mbar_arrive_cluster(bar);
-            }
+            if (lane < C) mbar_arrive_cluster(my_bar + 8 * t);
         }
-        // ------------------------------------------------------------ softmax of the whole chunk
-        mbar_wait_cluster(bar_all, 0, abort_word, p.dev_status);
         __syncwarp();
-        cluster_arrive();                                      // (see the teardown)
+        cluster_arrive();
+    } else {
+        // ------------------------------------------------------------ softmax: two tiles per warp
+        const int row = lane & 7, half = (lane >> 3) & 1, t = 2 * warp + (lane >> 4);
         float* const tmax = reinterpret_cast<float*>(smem + L::OFF_TM);
         float* const alphas = reinterpret_cast<float*>(smem + L::OFF_AL);
         float* const sums = reinterpret_cast<float*>(smem + L::OFF_RS);
         float* const m_last = reinterpret_cast<float*>(smem + L::OFF_M);
         volatile int* const flag = reinterpret_cast<volatile int*>(smem + L::OFF_FLAG);
         const float c = p.c;
-        const int t = tid >> 4, half = (tid >> 3) & 1;         // this thread: row, tile t of the chunk, columns 64 half ..
-        const bool live = t < n_tiles && row < p.G;
-        uint32_t s[64];
-        float mt = -CUDART_INF_F;
-        if (live) {
-            const float4* src = reinterpret_cast<const float4*>(smem + L::OFF_S + row * L::S_PITCH + t * 512 + half * 256);
-            float mx[4];
+        cluster_wait();
+        if (2 * warp < n_tiles) {
+            const bool live = t < n_tiles && row < p.G;
+            mbar_wait_cluster(bar_tile + 8 * (2 * warp), 0, abort_word, p.dev_status);
+            if (2 * warp + 1 < n_tiles) mbar_wait_cluster(bar_tile + 8 * (2 * warp + 1), 0, abort_word, p.dev_status);
+            __syncwarp();
+            uint32_t s[64];
+            float mt = -CUDART_INF_F;
+            if (live) {
+                const float4* src = reinterpret_cast<const float4*>(smem + L::OFF_S + t * L::S_TILE + row * L::S_PITCH + half * 256);
+                float mx[4];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float4 v = src[i];
-                s[4 * i] = __float_as_uint(v.x), s[4 * i + 1] = __float_as_uint(v.y);
-                s[4 * i + 2] = __float_as_uint(v.z), s[4 * i + 3] = __float_as_uint(v.w);
-                const float m2 = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
-                mx[i & 3] = i < 4 ? m2 : fmaxf(mx[i & 3], m2);
+                for (int i = 0; i < 16; ++i) {
+                    const float4 v = src[i];
+                    s[4 * i] = __float_as_uint(v.x), s[4 * i + 1] = __float_as_uint(v.y);
+                    s[4 * i + 2] = __float_as_uint(v.z), s[4 * i + 3] = __float_as_uint(v.w);
+                    const float m2 = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
+                    mx[i & 3] = i < 4 ? m2 : fmaxf(mx[i & 3], m2);
+                }
+                mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
             }
-            mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-        }
-        mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 8));   // the other half of the row's tile
-        if (half == 0) tmax[t * 8 + row] = mt;
-        named_bar_sync(1, 32 * DX_SOFTMAX_WARPS);              // maxima there; all scores are in registers
-        float m_old = -CUDART_INF_F, m_new = -CUDART_INF_F;
+            mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 8));   // the other half of the row's tile
+            if (half == 0) tmax[t * 8 + row] = mt;
+            __syncwarp();                                          // (all scores of the two tiles are in registers)
+            if (lane == 0) mbar_arrive(bar_tm + 8 * warp);
+            float m_old = -CUDART_INF_F, m_new = -CUDART_INF_F;
+            for (int w = 0; w <= warp; ++w) {
+                if (w < warp) mbar_wait_warp(bar_tm + 8 * w, 0, abort_word, p.dev_status);
 #pragma unroll
-        for (int j = 0; j < TILES_PER_CHUNK; ++j) {
-            const float mj = tmax[j * 8 + row];
-            if (j <= t) {
-                m_old = m_new;
-                m_new = softmax_next_max(m_old, mj, c);
+                for (int j = 0; j < 2; ++j) {
+                    const float mj = tmax[(2 * w + j) * 8 + row];
+                    if (2 * w + j <= t) {
+                        m_old = m_new;
+                        m_new = softmax_next_max(m_old, mj, c);
+                    }
+                }
             }
-        }
-        const float alpha = softmax_alpha(m_old, m_new, c);    // 0 on the chunk's first tile
-        const unsigned moved = __ballot_sync(0xffffffffu, live && t > 0 && alpha != 1.0f);
-        if (live) {
-            const float neg_mc = -__fmul_rn(m_new, c);
-            RowSum4 rs;
-            rs.reset();
+            const float alpha = softmax_alpha(m_old, m_new, c);    // 0 on the chunk's first tile
+            const unsigned moved = __ballot_sync(0xffffffffu, live && t > 0 && alpha != 1.0f);
+            if (live) {
+                const float neg_mc = -__fmul_rn(m_new, c);
+                RowSum4 rs;
+                rs.reset();
 #pragma unroll
-            for (int i = 0; i < 64; i += 8) softmax_p8(&s[i], c, neg_mc, rs, &s[i >> 1]);
-            uint8_t* const atom = smem + L::OFF_S + (2 * t + half) * 1024 + row * 128;
+                for (int i = 0; i < 64; i += 8) softmax_p8(&s[i], c, neg_mc, rs, &s[i >> 1]);
+                uint8_t* const atom = smem + L::OFF_S + t * L::S_TILE + half * 1024 + row * 128;
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                *reinterpret_cast<uint4*>(atom + ((i ^ row) << 4)) = make_uint4(s[4 * i], s[4 * i + 1], s[4 * i + 2], s[4 * i + 3]);
-            sums[(2 * t + half) * 8 + row] = rs.total();
-            if (half == 0) {
-                alphas[t * 8 + row] = alpha;
-                if (t == n_tiles - 1) m_last[row] = m_new;
+                for (int i = 0; i < 8; ++i)
+                    *reinterpret_cast<uint4*>(atom + ((i ^ row) << 4)) = make_uint4(s[4 * i], s[4 * i + 1], s[4 * i + 2], s[4 * i + 3]);
+                sums[(2 * t + half) * 8 + row] = rs.total();
+                if (half == 0) {
+                    alphas[t * 8 + row] = alpha;
+                    if (t == n_tiles - 1) m_last[row] = m_new;
+                }
             }
+            if ((lane & 15) == 0) flag[t] = (moved & (0xffffu << (lane & 16))) ? 1 : 0;
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_p + 8 * warp);
         }
-        if ((lane & 15) == 0) flag[t] = (moved & (0xffffu << (lane & 16))) ? 1 : 0;     // a warp holds two tiles
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_p);
         if (warp == 0) {
             // -------------------------------------------------------- rescales of O, then the chunk's result
-            mbar_wait_warp(bar_p, 0, abort_word, p.dev_status);
+            const uint32_t tlane = tmem;                           // lane quarter 0: rows 0 .. 7 on lanes 0 .. 7
             int phase = 0;
             float l_lo = 0.0f, l_hi = 0.0f;
             for (int j = 0; j < n_tiles; ++j) {
+                if (j % 2 == 0) mbar_wait_warp(bar_p + 8 * (j / 2), 0, abort_word, p.dev_status);
                 const float a = row < p.G ? alphas[j * 8 + row] : 1.0f;
                 l_lo = __fmaf_rn(l_lo, a, row < p.G ? sums[(2 * j) * 8 + row] : 0.0f);
                 l_hi = __fmaf_rn(l_hi, a, row < p.G ? sums[(2 * j + 1) * 8 + row] : 0.0f);
@@ -445,12 +463,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             }
             mbar_wait_warp(bar_pv, phase & 1, abort_word, p.dev_status);
             tc_fence_after();
-            const bool out = lane < p.G && !*abort_word;       // (lanes 0 .. 7: G <= 8)
             const float m = row < p.G ? m_last[row] : 0.0f;
+            const float Ltot = finalize_l(l_lo, l_hi), inv = finalize_inv(Ltot);
             const long long orow = static_cast<long long>(seq) * p.Hq + head + lane;
             const long long slot = orow * p.nchunk_max + chunk;
-            const float Ltot = finalize_l(l_lo, l_hi), inv = finalize_inv(Ltot);
-            if (out && rank == 0) {
+            const bool store = lane < p.G && !*abort_word;         // (lanes 0 .. 7: G <= 8)
+            if (store && rank == 0) {
                 if (p.direct_out) {
                     if (p.lse) p.lse[orow] = finalize_lse(m, Ltot, c);
                 } else {
@@ -464,7 +482,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 uint32_t v[32];
                 tmem_ld32(tlane + COL_O + 32 * cc, v);
                 tmem_wait_ld();
-                if (!out) continue;
+                if (!store) continue;
                 if (p.direct_out) {
                     // one chunk per sequence: the partial is the result (see the decode mode of attn_kernel)
                     uint4* d4 = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.o) + orow * D + rank * VC + 32 * cc);
@@ -484,21 +502,21 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 }
             }
         }
+        __syncwarp();
+        cluster_arrive();
     }
 
     // ---------------------------------------------------------------- teardown
-    if (*abort_word) {   // let copies, MMAs and the peers' writes in flight finish before shared memory and TMEM are released
+    if (*abort_word) {   // let copies and MMAs in flight finish before shared memory and TMEM are released
         const unsigned long long t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 1000000ull) {
         }
     }
-    // No CTA leaves while another may still write to it.  Normally bar_all has seen to that and every
-    // CTA has arrived here long ago; after an expired wait this is what keeps the cluster together.
     __syncwarp();
     cluster_wait();
     tc_fence_before();
     __syncthreads();
-    if (warp == 9) tmem_dealloc(tmem, TMEM_COLS);
+    if (warp == 13) tmem_dealloc(tmem, TMEM_COLS);
 }
 
 template <int D, int C>

@@ -77,10 +77,10 @@ struct DeviceOnce {
 };
 
 // Builds a bf16 tiled tensor map with 128-byte swizzle; dims/box innermost first, strides
-// in bytes for dims 1..rank-1.  Returns false (and fills err) on failure.
+// in bytes for dims 1..rank-1.  Returns false (and fills err) on failure.  swizzle64: 64-byte swizzle instead.
 bool make_tmap_bf16(tik_ctx* ctx, CUtensorMap* out, const void* base, int rank,
                     const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box,
-                    std::string* err);
+                    std::string* err, bool swizzle64 = false);
 
 struct AttnParams {
     alignas(64) CUtensorMap tmO; // train / prefill: tiled map of the output (same shape and box as Q)
@@ -118,6 +118,11 @@ cudaError_t launch_combine(int d, const AttnParams& p, int B, cudaStream_t strea
 constexpr int DECODE2_MAX_G = 8;
 cudaError_t launch_decode2(int d, dim3 grid, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                            const AttnParams& p, cudaStream_t stream);
+
+// Decode of small calls (tik_decode_cluster.cu): clusters of C = 2 or 4 CTAs (d = 64: 2) per chunk.  tmV has a
+// box of d / C columns, with the 64-byte swizzle when that is 32.  Same scratch layout and output bits.
+cudaError_t launch_decode_cluster(int d, int C, int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
+                                  const CUtensorMap& tmV, const AttnParams& p, cudaStream_t stream);
 
 // Persistent full-sequence attention (tik_attn_persist.cu): a planning kernel writes the list of
 // work items of the call into `plan` (attn_plan_bytes bytes, 16-byte aligned), then one CTA per SM
