@@ -454,17 +454,20 @@ tik_status tik_attn_decode(tik_ctx* ctx, const void* q, void* o, float* lse, con
     p.part_o = static_cast<float*>(ws);
     p.part_ml = p.part_o + static_cast<size_t>(B) * Hq * nchunk * d;
     p.dev_status = ctx->dev_status;
-    // Two kernels give the same bits.  The small CTA of tik_decode.cu (two per SM) wins where CTAs
-    // are short or few per SM: at most one (sequence, KV head) pair per SM but about as many chunks
-    // as SMs or more (the one-CTA-per-SM kernel runs a ragged second wave there), and any number of
-    // pairs with contexts of at most two chunks (a CTA streams <= 32 tiles; two co-resident CTAs hide
-    // each other's set-up and tail: 64 x 4096 keys 103 -> 93 us, 256 x 2048 395 -> 313 us, also
-    // right after a seconds-long GEMM).  With fewer chunks than SMs every CTA has an SM to itself
-    // either way and the big kernel's faster per-CTA pipeline (two softmax warpgroups, five K/V
-    // stages) gives the shorter latency; with many pairs of long contexts the same pipeline streams
-    // faster per SM (the paper's decode grid, Sec. 6 Q3, covers both ends).
-    const bool small_group = G <= DECODE2_MAX_G && (pairs <= ctx->sm_count || nchunk <= 2) && 4 * pairs * nchunk >= 3ll * ctx->sm_count;
-    p.cpc = decode_chunks_per_cta(B, Hkv, nchunk, ctx->sm_count, small_group ? 2 : 1);
+    // Calls without clusters: two kernels give the same bits.  The small CTA of tik_decode.cu (two per SM, one
+    // chunk each: the hardware deals them out dynamically) wins with more (sequence, KV head, chunk)
+    // items than SMs, where CTAs are short or few per SM -- at most one (sequence, KV head) pair per SM
+    // (32 x 6000 keys x 4 KV heads 58 -> 56 us, 16 x 16000 x 8 140 -> 130) or contexts of at most two chunks
+    // (64 x 1000 x 4 30.6 -> 26.7, 256 x 1000 x 8 143 -> 121) -- and with eight items per SM or more (64 x 5000
+    // x 8 165 -> 150, 128 x 6000 x 4 187 -> 177, 256 x 8000 x 4 466 -> 439).  In between the kernels are within
+    // 5 % of each other, the big one ahead where sequences share prompt pages (64 x 1280..5120 x 4, groups of
+    // eight: 79 against 83 us).  With an SM for every item the big kernel's faster pipeline (two softmax
+    // warpgroups, five K/V stages) is shorter: 16 x 2000 x 8 26.7 against 32.8 us, 32 x 1500 x 4 22.6 against
+    // 26.7 -- except for contexts of one tile, where set-up is all there is: 128 keys 5.3 -> 4.4 us, 250 5.7 = 5.9.
+    const long long items = pairs * nchunk;
+    const bool small_group = G <= DECODE2_MAX_G && (max_ctx_len <= 128 || (items > ctx->sm_count &&
+                             (pairs <= ctx->sm_count || nchunk <= 2 || items >= 8ll * ctx->sm_count)));
+    p.cpc = small_group ? 1 : decode_chunks_per_cta(B, Hkv, nchunk, ctx->sm_count);
     p.lookahead = ctx->sm_count;
     dim3 grid((nchunk + p.cpc - 1) / p.cpc, Hkv, B);
     if (grid.y > 65535 || grid.z > 65535) return fail(ctx, TIK_ERR_UNSUPPORTED, "Hkv and B must be <= 65535");

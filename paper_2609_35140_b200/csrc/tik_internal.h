@@ -154,16 +154,11 @@ struct PrepParams {
 };
 cudaError_t launch_prep(int d, const PrepParams& p, int64_t total_new, cudaStream_t stream);
 
-// Decode: how many consecutive chunks one CTA streams.  A CTA's set-up and drain cost about a
-// third of one chunk's streaming time, so several chunks per CTA pay as long as the grid still
-// covers every CTA slot several times over.  Chunk partials do not depend on this choice.
-// With two resident CTAs per SM (tik_decode.cu) a CTA's rate is bound by its own serial chain and
-// short ring (measured ~22 GB/s per CTA), so what counts is that all slots stay busy and that no
-// CTA is long: many one-chunk CTAs that the hardware deals out dynamically do that better than few
-// long ones (a batch of ragged contexts is as slow as its longest CTA).  Chunks are grouped only
-// when the grid stays above four waves.
-inline int decode_chunks_per_cta(long long B, int Hkv, int nchunk, int sm_count, int ctas_per_sm = 1) {
-    const long long slots = static_cast<long long>(ctas_per_sm) * (sm_count > 0 ? sm_count : 148);
+// Decode with one CTA per SM: how many consecutive chunks a CTA streams.  A CTA's set-up and drain cost about
+// a third of one chunk's streaming time, so several chunks per CTA pay as long as the grid still covers
+// the SMs four times.  Chunk partials do not depend on this choice.
+inline int decode_chunks_per_cta(long long B, int Hkv, int nchunk, int sm_count) {
+    const long long slots = sm_count > 0 ? sm_count : 148;
     for (int c = 4; c > 1; --c)
         if (c <= nchunk && B * Hkv * ((nchunk + c - 1) / c) >= 4 * slots) return c;
     return 1;

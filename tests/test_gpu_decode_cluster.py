@@ -55,3 +55,21 @@ def test_cluster_decode_equals_train_rows(tik, lens, Hkv, G, d, page, ramp):
     o = torch.full((S, w.Hq, d), 7.0, dtype=torch.bfloat16, device="cuda")
     tik.tik_attn_decode(q[rows2].contiguous(), ctx2, kc, vc, bt, max(lens), w.softmax_scale, o=o)
     assert bool((o[0] == 7.0).all()) and count_diff(o[1:], o_train[rows2][1:]) == 0
+
+
+@pytest.mark.parametrize("S,Hkv,G,lo,hi", [(3, 2, 4, 1, 128), (3, 2, 4, 100, 129), (37, 4, 2, 1500, 2048), (38, 4, 2, 1500, 2048),
+                                           (150, 8, 1, 4097, 4300)])
+def test_decode_at_the_edges_of_the_kernel_choice(tik, S, Hkv, G, lo, hi):
+    """Contexts of one tile and one key more, as many chunks as SMs and a few more, and many pairs of three
+    chunks: the rows equal those of the packed train-forward."""
+    rng = np.random.default_rng(S + hi)
+    lens = [hi] + [int(x) for x in rng.integers(lo, hi + 1, S - 1)]
+    w = synth.custom_workload([1] * S, [L - 1 for L in lens], G * Hkv, Hkv, 128, 64, index=71)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    o_train = tik.tik_attn_train_fwd(q, k, v, cu, hi, w.softmax_scale)
+    layout = synth.make_paged_layout(w)
+    kc, vc = synth.fill_paged_cache(w, layout, k, v)
+    ctx = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    rows = torch.tensor([int(w.cu_seqlens()[s]) + L - 1 for s, L in enumerate(lens)], device="cuda")
+    o = tik.tik_attn_decode(q[rows].contiguous(), ctx, kc, vc, torch.from_numpy(layout.block_table).cuda(), hi, w.softmax_scale)
+    assert count_diff(o, o_train[rows]) == 0
