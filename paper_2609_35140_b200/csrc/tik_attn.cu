@@ -1035,8 +1035,7 @@ __global__ void __launch_bounds__(D) combine_kernel(const AttnParams p) {
 
 // ------------------------------------------------------------------ KV-cache write
 // A block copies KVW_TOK (8 or 1) consecutive new tokens (K and V rows of all KV heads: 16-byte vectors).
-// Threads 0 .. KVW_TOK-1 find their token's sequence (binary search over cu_new), position and
-// physical page; then all threads copy, every thread's loads issued before its stores.  (One token
+// Warps 0 .. KVW_TOK-1 find their token's sequence, position and physical page; then all threads copy, every thread's loads issued before its stores.  (One token
 // per 128-thread block, each doing its own search before 32 bytes of copying per thread, reached
 // 0.76 of the copy bandwidth.)
 constexpr int KVW_THREADS = 256;
@@ -1051,26 +1050,22 @@ kv_write_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new
     pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid
     __shared__ long long dst_base[KVW_TOK];     // vector index of (page, head 0, row, 0), or -1
     const long long tok0 = static_cast<long long>(blockIdx.x) * KVW_TOK;
-    if (threadIdx.x < KVW_TOK) {
-        const long long token = tok0 + threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < KVW_TOK) {                              // warp w looks up token w
+        const long long token = tok0 + warp;
         long long base = -1;
         if (token < total_new) {
-            int lo = 0, hi = S;            // find s with cu_new[s] <= token < cu_new[s+1]
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (cu_new[mid] <= token) lo = mid; else hi = mid;
-            }
-            const int s = lo;
-            const int n_s = cu_new[s + 1] - cu_new[s];
-            const int pos = ctx_lens[s] - n_s + static_cast<int>(token - cu_new[s]);
-            if (token < cu_new[s + 1] && pos >= 0) {
+            const int s = warp_find_sequence(cu_new, S, token, lane);
+            const int first = cu_new[s], end = cu_new[s + 1];
+            const int pos = ctx_lens[s] - (end - first) + static_cast<int>(token - first);
+            if (token < end && pos >= 0) {
                 const int lp = pos / page_size, row = pos % page_size;
                 const int phys = (lp < max_blocks) ? block_table[static_cast<long long>(s) * max_blocks + lp] : -1;
-                if (phys < 0 || phys >= num_pages) atomicOr(dev_status, TIK_DEV_BAD_BLOCK);
-                else base = (static_cast<long long>(phys) * Hkv * page_size + row) * vec_per_head;
+                if (phys >= 0 && phys < num_pages) base = (static_cast<long long>(phys) * Hkv * page_size + row) * vec_per_head;
+                else if (lane == 0) atomicOr(dev_status, TIK_DEV_BAD_BLOCK);
             }
         }
-        dst_base[threadIdx.x] = base;
+        if (lane == 0) dst_base[warp] = base;
     }
     __syncthreads();
     const int nvec = Hkv * vec_per_head;                 // vectors per token and tensor

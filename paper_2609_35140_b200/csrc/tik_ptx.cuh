@@ -79,6 +79,21 @@ __device__ __forceinline__ void mbar_wait_warp(uint32_t bar, uint32_t parity,
 __device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
+// The sequence s with cu[s] <= token < cu[s + 1] (empty sequences skipped), found by a whole warp: 32 probes
+// per round, so one or two rounds of global latency instead of the log2(S) dependent loads of a binary
+// search.  0 <= token; S >= 1.
+__device__ __forceinline__ int warp_find_sequence(const int32_t* cu, int S, long long token, int lane) {
+    int lo = 0, hi = S;                  // cu[lo] <= token, and cu[hi] > token if the token exists
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32, probe = lo + step * (lane + 1);
+        const unsigned below = __ballot_sync(0xffffffffu, probe < hi && cu[probe] <= token);
+        const int n = __popc(below);     // cu is ascending: the first n probes
+        lo += step * n;
+        hi = min(hi, lo + step);
+    }
+    return lo;
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while its
 // predecessor in the stream still runs: its CTAs are scheduled once every CTA of the predecessor

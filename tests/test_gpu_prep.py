@@ -162,3 +162,34 @@ def test_bad_position_and_bad_block_are_flagged_and_skipped(tik):
         tik.tik_qk_norm_rope_kv_write(q0.clone(), k0.clone(), None, None, None, float("nan"), tab, cu)
     with pytest.raises(tik.TikError):        # a cache without V
         tik.tik_qk_norm_rope_kv_write(q0.clone(), k0.clone(), None, None, None, EPS, tab, cu, ctx, kc, vc, bt)
+
+
+@pytest.mark.parametrize("S,Hq,Hkv,d", [(1, 64, 8, 128), (33, 28, 4, 128), (455, 64, 8, 128), (456, 64, 8, 128), (1100, 5, 1, 64)])
+def test_steps_of_one_token_per_sequence_equal_a_packed_call(tik, S, Hq, Hkv, d):
+    """A decode step's call -- one new token per sequence, sequence search over 1 .. 1100 of them with empty
+    ones in between, one warp per batch of heads below 4096 batches and per token above -- gives the bits and
+    cache rows of one call that packs the same tokens as a single sequence at the same positions."""
+    g = torch.Generator(device="cuda").manual_seed(S)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    page, pos0 = 64, 37
+    n = S - S // 3                                               # every third sequence has no new token
+    has = torch.tensor([1 if s % 3 != 1 or s // 3 >= S // 3 else 0 for s in range(S)])
+    assert int(has.sum()) == n
+    q, k, v, wq, wk = rnd(n, Hq, d), rnd(n, Hkv, d), rnd(n, Hkv, d), rnd(d), rnd(d)
+    rope = synth.make_rope_table(pos0 + n, d, device="cuda")
+    cu = torch.cat([torch.zeros(1, dtype=torch.int64), has.cumsum(0)]).to(torch.int32).cuda()
+    ctx = torch.zeros(S, dtype=torch.int32)
+    ctx[has == 1] = pos0 + 1 + torch.arange(n, dtype=torch.int32)     # token i of the call at position pos0 + i
+    blocks = (pos0 + n + page - 1) // page
+    table = torch.arange(blocks, dtype=torch.int32, device="cuda")[None].repeat(S, 1).contiguous()   # all in the same pages
+    out = []
+    for cu_, ctx_, table_ in ((cu, ctx.cuda(), table), (torch.tensor([0, n], dtype=torch.int32, device="cuda"),
+                                                        torch.tensor([pos0 + n], dtype=torch.int32, device="cuda"), table[:1])):
+        kc = torch.zeros(blocks, Hkv, page, d, dtype=torch.bfloat16, device="cuda")
+        vc, q_, k_ = torch.zeros_like(kc), q.clone(), k.clone()
+        tik.tik_qk_norm_rope_kv_write(q_, k_, v, wq, wk, 1e-6, rope, cu_, ctx_, kc, vc, table_)
+        kc2, vc2 = torch.zeros_like(kc), torch.zeros_like(kc)
+        tik.tik_kv_cache_write(k_, v, cu_, ctx_, kc2, vc2, table_)
+        assert count_diff(kc2, kc) == 0 and count_diff(vc2, vc) == 0
+        out.append((q_, k_, kc, vc))
+    assert all(count_diff(a, b) == 0 for a, b in zip(*out))
