@@ -316,20 +316,33 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
-// One thread per token: fold the super-chunk pairs in ascending order, write the result.
-__global__ void __launch_bounds__(256) logprob_finish_kernel(const LogprobParams p) {
-    pdl_wait();                        // the super-chunk pairs and target logits are complete and visible
-    pdl_launch_dependents();
-    const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (t >= p.T) return;
-    const float* ml = p.part_ml + 2 * t * p.nsuper;
-    float M = ml[0], Lsum = ml[1];
-    for (int s = 1; s < p.nsuper; ++s) {
-        const FoldCoef f = fold_coef(M, ml[2 * s], LOG2E_F);
-        Lsum = fold_value(Lsum, ml[2 * s + 1], f);
-        M = f.M_new;
+// Folds n <= 32 consecutive (max, sum) pairs, lane i holding the i-th, into the running pair (M, L) of a warp, in
+// ascending order with the arithmetic of fold_coef / fold_value.  A fold's factors depend on the maxima only,
+// and a running maximum is exact in any order: so the 32 factor pairs are computed side by side from a
+// prefix maximum, and what stays serial is one fused multiply-add per pair.  `start`: lane 0's pair is
+// the first of all and is copied.
+__device__ __forceinline__ void lp_fold_warp(float& M, float& L, float m, float l, int n, bool start, int lane) {
+    const bool valid = lane < n;
+    float run = valid ? m : -CUDART_INF_F;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float o = __shfl_up_sync(0xffffffffu, run, off);
+        if (lane >= off) run = fmaxf(run, o);
     }
-    const float lse = lp_lse(M, Lsum);
+    float before = __shfl_up_sync(0xffffffffu, run, 1);                   // maximum of the pairs before this one ...
+    before = lane == 0 ? M : (start ? before : fmaxf(M, before));         // ... and of everything folded earlier
+    const FoldCoef f = fold_coef(before, m, LOG2E_F);
+    float A = f.A, b = __fmul_rn(l, f.B);
+    if (start && lane == 0) {
+        A = 0.0f;
+        b = l;
+    }
+    for (int i = 0; i < n; ++i) L = __fmaf_rn(L, __shfl_sync(0xffffffffu, A, i), __shfl_sync(0xffffffffu, b, i));
+    const float top = __shfl_sync(0xffffffffu, run, 31);
+    M = start ? top : fmaxf(M, top);
+}
+__device__ __forceinline__ void lp_write(const LogprobParams& p, long long t, float M, float L) {
+    const float lse = lp_lse(M, L);
     if (p.lse) p.lse[t] = lse;
     const int target = p.target[t];
     if (target < 0 || target >= p.V) {
@@ -340,65 +353,67 @@ __global__ void __launch_bounds__(256) logprob_finish_kernel(const LogprobParams
     }
 }
 
+// One warp per token: fold the super-chunk pairs in ascending order, write the result.  (One thread per
+// token was a chain of 149 dependent folds on T / 256 blocks.  64 rows, H 3584: whole call
+// 183.8 -> 182.2 us; 4001 rows, H 1536: 1216 -> 1211.)
+__global__ void __launch_bounds__(256) logprob_finish_kernel(const LogprobParams p) {
+    pdl_wait();                        // the super-chunk pairs and target logits are complete and visible
+    pdl_launch_dependents();
+    const long long t = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= p.T) return;
+    const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + t * p.nsuper;
+    float M = -CUDART_INF_F, L = 0.0f;
+    float2 next = lane < p.nsuper ? ml[lane] : make_float2(0.0f, 0.0f);
+    for (int s0 = 0; s0 < p.nsuper; s0 += 32) {
+        const float2 x = next;
+        if (s0 + 32 + lane < p.nsuper) next = ml[s0 + 32 + lane];
+        lp_fold_warp(M, L, x.x, x.y, min(32, p.nsuper - s0), s0 == 0, lane);
+    }
+    if (lane == 0) lp_write(p, t, M, L);
+}
+
 // Unit mode: one block per token.  Thread s folds the tiles of super-chunk s in ascending order
-// (first tile copied, the others folded: the main kernel's in-CTA sequence), then thread 0 folds
+// (first tile copied, the others folded: the main kernel's in-CTA sequence), then a warp folds
 // the super-chunks in ascending order as logprob_finish_kernel does.
 __global__ void __launch_bounds__(256) logprob_finish_tiles_kernel(const LogprobParams p) {
     pdl_wait();
     pdl_launch_dependents();
     __shared__ float sm[256], sl[256];
     const long long t = blockIdx.x;
-    const float* ml = p.part_ml + 2 * t * p.ntile128;
+    const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + t * p.ntile128;
     constexpr int TPS = LP_SUPER / LP_TILE;        // tiles per super-chunk
+    const int lane = threadIdx.x & 31;
+    float Mt = -CUDART_INF_F, Lt = 0.0f;           // warp 0: everything folded so far
     for (int s0 = 0; s0 < p.nsuper; s0 += 256) {
         const int s = s0 + threadIdx.x;
         float M = 0.0f, Lsum = 0.0f;
         if (s < p.nsuper) {
-            const int t0 = s * TPS, t1 = min(p.ntile128, t0 + TPS);
-            M = ml[2 * t0];
-            Lsum = ml[2 * t0 + 1];
-            for (int j = t0 + 1; j < t1; ++j) {
-                const FoldCoef f = fold_coef(M, ml[2 * j], LOG2E_F);
-                Lsum = fold_value(Lsum, ml[2 * j + 1], f);
-                M = f.M_new;
+            const int t0 = s * TPS, n = min(TPS, p.ntile128 - t0);
+            float2 x[TPS];
+#pragma unroll
+            for (int j = 0; j < TPS; ++j)
+                if (j < n) x[j] = ml[t0 + j];
+            M = x[0].x;
+            Lsum = x[0].y;
+#pragma unroll
+            for (int j = 1; j < TPS; ++j) {
+                if (j < n) {
+                    const FoldCoef f = fold_coef(M, x[j].x, LOG2E_F);
+                    Lsum = fold_value(Lsum, x[j].y, f);
+                    M = f.M_new;
+                }
             }
         }
         __syncthreads();                            // (the previous batch of super-chunks has been consumed)
         sm[threadIdx.x] = M;
         sl[threadIdx.x] = Lsum;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            // running total kept in sm[0] / sl[0] across batches of 256 super-chunks
-            float Mt = sm[0], Lt = sl[0];
-            if (s0 > 0) {
-                // restore the running total saved below, then fold this batch's first entry
-                const float Mr = p.part_ml[2 * t * p.ntile128], Lr = p.part_ml[2 * t * p.ntile128 + 1];
-                const FoldCoef f = fold_coef(Mr, Mt, LOG2E_F);
-                Lt = fold_value(Lr, Lt, f);
-                Mt = f.M_new;
-            }
-            const int n = min(256, p.nsuper - s0);
-            for (int i = 1; i < n; ++i) {
-                const FoldCoef f = fold_coef(Mt, sm[i], LOG2E_F);
-                Lt = fold_value(Lt, sl[i], f);
-                Mt = f.M_new;
-            }
-            if (s0 + 256 < p.nsuper) {              // more batches follow: park the running total
-                p.part_ml[2 * t * p.ntile128] = Mt;
-                p.part_ml[2 * t * p.ntile128 + 1] = Lt;
-            } else {
-                const float lse = lp_lse(Mt, Lt);
-                if (p.lse) p.lse[t] = lse;
-                const int target = p.target[t];
-                if (target < 0 || target >= p.V) {
-                    atomicOr(p.dev_status, TIK_DEV_BAD_TARGET);
-                    p.logprob[t] = CUDART_NAN_F;
-                } else {
-                    p.logprob[t] = __fsub_rn(p.z_target[t], lse);
-                }
-            }
-        }
+        if (threadIdx.x < 32)
+            for (int i0 = 0; i0 < 256 && s0 + i0 < p.nsuper; i0 += 32)
+                lp_fold_warp(Mt, Lt, sm[i0 + lane], sl[i0 + lane], min(32, p.nsuper - s0 - i0), s0 + i0 == 0, lane);
     }
+    if (threadIdx.x == 0) lp_write(p, t, Mt, Lt);
 }
 
 template <bool PAIR>
@@ -431,7 +446,7 @@ cudaError_t launch_logprob(const CUtensorMap& tmA, const CUtensorMap& tmB, const
     cudaError_t e = pair ? launch_logprob_main<true>(tmA, tmB, p, stream) : launch_logprob_main<false>(tmA, tmB, p, stream);
     if (e != cudaSuccess) return e;
     return launch_pdl(p.unit_mode ? logprob_finish_tiles_kernel : logprob_finish_kernel,
-                      dim3(static_cast<unsigned>(p.unit_mode ? p.T : (p.T + 255) / 256)), 256, 0, stream, 1, p);
+                      dim3(static_cast<unsigned>(p.unit_mode ? p.T : (p.T + 7) / 8)), 256, 0, stream, 1, p);
 }
 
 }  // namespace tik

@@ -123,3 +123,19 @@ def test_bad_target_is_nan_and_flagged(tik):
     ref, _ = _oracle(hidden, W, target)
     assert np.abs(lp[good] - ref[good]).max() <= LOGPROB_TOL
     assert tik.device_status() & tik.DEV_BAD_TARGET
+
+
+@pytest.mark.parametrize("T,V", [(5, 1), (3, 1024), (9, 1025), (2, 33000), (2050, 33000), (2049, 1030), (3, 300001)])
+def test_any_number_of_super_chunks(tik, T, V):
+    """1 to 293 super-chunks of 1024 columns, ragged last ones, with the per-tile partials of small calls and
+    the per-super-chunk ones of large calls: against torch in fp64, and rows of a small call equal those of a large one."""
+    H = 64
+    g = torch.Generator(device="cuda").manual_seed(V)
+    x = torch.randn(T, H, generator=g, device="cuda").to(torch.bfloat16)
+    W = (torch.randn(V, H, generator=g, device="cuda") * 0.3).to(torch.bfloat16)
+    ids = torch.randint(0, V, (T,), generator=g, device="cuda").to(torch.int32)
+    got = tik.tik_token_logprob(x, W, ids)
+    want = torch.log_softmax(x.double() @ W.double().t(), -1).gather(1, ids.long()[:, None])[:, 0]
+    assert float((got.double() - want).abs().max()) <= 1e-4          # fp32 sums of up to 3e5 terms, |z| < 20
+    big = tik.tik_token_logprob(x.repeat(1 + 2048 // T, 1), W, ids.repeat(1 + 2048 // T))
+    assert torch.equal(big[:T], got)
