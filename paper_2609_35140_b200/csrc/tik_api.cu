@@ -642,9 +642,11 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
         p.nu = 8 * ((N + 8 * ctx->sm_count - 1) / (8 * ctx->sm_count));     // weight rows per CTA: whole 8-row swizzle atoms
         p.nunit = (N + p.nu - 1) / p.nu;
         p.a_rows = 16 * ((static_cast<int>(T) + 15) / 16);
-        // as many K slices per stage (one barrier round trip of the issuing thread) as leave four stages
-        p.kps = 8;
-        while (p.kps > 1 && (p.kps > K / 64 || LINEAR_NARROW_RING / ((p.nu + p.a_rows) * 128u * p.kps) < 4)) p.kps /= 2;
+        // as many K slices per stage (a barrier round trip and a commit of the issuing warp, ~280 clk against 25
+        // per MMA) as leave four stages, or 16 of them and three (16 rows, K 8960, N 1536: 20.5 -> 18.5 us)
+        p.kps = 16;
+        while (p.kps > 1 && (p.kps > K / 64 || LINEAR_NARROW_RING / ((p.nu + p.a_rows) * 128u * p.kps) < (p.kps == 16 ? 3u : 4u)))
+            p.kps /= 2;
         const uint64_t st3[2] = {static_cast<uint64_t>(K) * 2, 128};
         const uint64_t wd[3] = {64, static_cast<uint64_t>(N), static_cast<uint64_t>(K / 64)};
         const uint64_t xd[3] = {64, static_cast<uint64_t>(T), static_cast<uint64_t>(K / 64)};
