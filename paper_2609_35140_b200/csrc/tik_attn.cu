@@ -89,8 +89,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     constexpr uint32_t COL_S = 0;                          // one score buffer of 128 columns
     constexpr uint32_t COL_P = 128;                        // two weight buffers of 64 columns (bf16 pairs)
     constexpr uint32_t COL_OA = 256, COL_OB = 256 + D;
-    constexpr uint32_t IDESC_QK = mma_idesc_bf16(128, 128, false);
-    constexpr uint32_t IDESC_PV = mma_idesc_bf16(128, D, true);
+    // decode of at most 16 query heads per KV head: M64, half the tensor work of M128
+    const int mma_m = (MODE == MODE_DECODE && p.G <= 16) ? 64 : 128;
+    const uint32_t IDESC_QK = mma_idesc_bf16(mma_m, 128, false);
+    const uint32_t IDESC_PV = mma_idesc_bf16(mma_m, D, true);
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     // Launched with programmatic stream serialization: the grid may be scheduled while the kernel
@@ -280,12 +282,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     };
     auto load_q = [&]() {                                   // lane 0 of warp 0
         if (MODE == MODE_DECODE) {
-            // the G query rows go to rows 0.., 32.., 64.., 96..: every lane quarter of the score
-            // tile then holds the same G rows and the four warps of a warpgroup share a row's columns
+            // the G query rows go to the first rows of every lane quarter of the score tile, which
+            // then holds the same G rows and the four warps of a warpgroup share a row's columns
+            // (an M64 MMA spreads its rows 16 per lane quarter, an M128 one 32)
             mbar_expect_tx(bar_q, 4u * static_cast<uint32_t>(p.G) * 128u * NATOM);
-            for (int q4 = 0; q4 < 4; ++q4)
+            const uint32_t quarter_rows = p.G <= 16 ? 16u : 32u;
+            for (uint32_t q4 = 0; q4 < 4; ++q4)
                 for (int a = 0; a < NATOM; ++a)
-                    tma_load_3d(sQ + a * L::ATOM + q4 * 4096, &tmQ, bar_q, a * 64, head, seq);
+                    tma_load_3d(sQ + a * L::ATOM + q4 * quarter_rows * 128u, &tmQ, bar_q, a * 64, head, seq);
         } else {
             mbar_expect_tx(bar_q, pair ? 2 * L::TILE : L::TILE);
             for (int q2 = 0; q2 < (pair ? 2 : 1); ++q2)
@@ -672,7 +676,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                         wait_pv(it - 1);
                         write_partial_ml(chunk_of(it - 1), m_prev, l_prev_lo, l_prev_hi);
                         write_partial_o(chunk_of(it - 1), 0, D);
-                    } else if (!chunk_start && !__all_sync(0xffffffffu, alpha == 1.0f)) {
+                    } else if (!chunk_start && !__all_sync(0xffffffffu, lane >= p.G || alpha == 1.0f)) {
                         wait_pv(it - 1);
                         rescale_o_tmem<D>(tlane + col_o_of(it), alpha);
                     }

@@ -8,12 +8,11 @@
 // (K tile -> QK^T -> softmax -> PV) fill each other's gaps.
 //
 // The arithmetic is attn_kernel<D, decode>'s: the same 128-key tiles at absolute positions, the
-// same M128 x N128 x K16 score MMAs and M128 x Nd x K16 value MMAs, the same column split of a
-// row over four warps with one warp summing and packing in the contract's order, the same
+// same chains of K16 MMAs, the same column split of a row over four warps with one warp summing and packing in the contract's order, the same
 // per-chunk partials for combine_kernel.  What changes is layout and schedule:
 //   * Q is 8 rows x d in shared memory (1 KiB per 64 columns).  The MMA's A descriptor has a
-//     stride of ZERO between its 8-row groups, so all sixteen groups of the 128-row operand read
-//     the same rows: row i of the group sits on TMEM lanes i, i + 8, ..., in every lane quarter.
+//     stride of ZERO between its 8-row groups, so all eight groups of the 64-row operand read
+//     the same rows: row i of the group sits on TMEM lanes i and i + 8 of every lane quarter.
 //     (attn_kernel spends a 32 KiB tile on the same effect.)
 //   * the weights P overwrite the scores S in tensor memory (columns 0..63 of the score buffer):
 //     S 128 + O d = 256 columns.  Per CTA the chain QK^T -> softmax -> PV is therefore serial;
@@ -62,8 +61,12 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     constexpr uint32_t TMEM_COLS = 256;
     constexpr uint32_t COL_S = 0;              // scores (128 columns); the packed weights overwrite columns 0..63
     constexpr uint32_t COL_O = 128;            // the chunk's accumulator (D columns)
-    constexpr uint32_t IDESC_QK = mma_idesc_bf16(128, 128, false);
-    constexpr uint32_t IDESC_PV = mma_idesc_bf16(128, D, true);
+    // M64: half the tensor work and operand reads of M128 for at most eight rows.  A long decode is bound by
+    // HBM at the power cap, where the tensor pipe's energy costs memory clock: 16 x 15000..16384 keys (32/8
+    // heads, with cache write) 187 -> 175 us at 1400 -> 1540 MHz.  Rows i and i + 8 of the (repeated) query
+    // group sit on lanes 0..15 of every quarter; lanes 16..31 hold nothing.
+    constexpr uint32_t IDESC_QK = mma_idesc_bf16(64, 128, false);
+    constexpr uint32_t IDESC_PV = mma_idesc_bf16(64, D, true);
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     pdl_wait();
@@ -351,7 +354,7 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const float alpha = softmax_alpha(m_old, m_new, c);
                 l_lo = __fmaf_rn(chunk_start ? 0.0f : l_lo, alpha, rs_lo.total());
                 l_hi = __fmaf_rn(chunk_start ? 0.0f : l_hi, alpha, rs_hi.total());
-                if (!chunk_start && !__all_sync(0xffffffffu, alpha == 1.0f)) {
+                if (!chunk_start && !__all_sync(0xffffffffu, lane >= p.G || alpha == 1.0f)) {
                     wait_pv(it - 1);             // the accumulator holds every earlier tile of the chunk
 #pragma unroll 1
                     for (int cc = 0; cc < D / 32; ++cc) {
