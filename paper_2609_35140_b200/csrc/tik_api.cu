@@ -552,6 +552,7 @@ tik_status tik_token_logprob(tik_ctx* ctx, const void* hidden, const void* lm_he
     // A log-probability has the same bits either way (same K order, same 128-column tiles).
     const bool pair = T > 128;
     uint32_t boxB[2] = {64, pair ? 128u : 256u};
+    if (T <= 64) box[1] = 64;            // M64 MMAs, see logprob_kernel
     if (!make_tmap_bf16(ctx, &tmA, hidden, 2, ad, st1, box, &err) ||
         !make_tmap_bf16(ctx, &tmB, lm_head, 2, bd, st1, boxB, &err))
         return fail(ctx, TIK_ERR_CUDA, err.c_str());

@@ -258,7 +258,7 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 // schedule is built for bytes in flight and even SM load instead of tensor throughput: the grid is
 // one persistent CTA per SM walking column units u = blockIdx.x, + gridDim.x, ...; a unit is
 // `nu` = 64, 128 or 256 output columns (the host picks the width from a cost model);
-// only `a_rows` = 32, 64 or 128 rows of x are staged per K slice (the MMA still spans 128 rows: rows
+// only `a_rows` = 32, 64 or 128 rows of x are staged per K slice (the MMA spans 64 or 128 rows: rows
 // past a_rows read whatever the stage holds, their accumulator rows are never stored); the ring
 // has as many stages as fit in 192 KiB (3 .. 4) of one, two or four K slices each, and the producer runs ahead into the next unit
 // while the epilogue of the last one drains.  An output element is still one chain of K16 MMAs in
@@ -291,7 +291,10 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int nst = min(MAX_STAGES, static_cast<int>(RING_BYTES / stage_bytes));
     const int n_my = (p.nunit - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
     const int n_kb = p.K / 64;
-    const uint32_t idesc = mma_idesc_bf16(128, nu, false);
+    // At most 64 rows: M64, half the tensor work of M128 (16 rows, K 1536, N 17920, in a graph: 14 -> 11.3 us);
+    // accumulator row i then sits on lane i % 16 of lane quarter i / 16.
+    const bool m64 = p.a_rows <= 64;
+    const uint32_t idesc = mma_idesc_bf16(m64 ? 64 : 128, nu, false);
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -393,7 +396,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // As in the batched kernel: a thread per accumulator row, 64 columns at a time through a
         // swizzled staging tile and one tiled TMA store, which clips rows past T and columns past N.
         const int quarter = warp & 3;
-        const int row = quarter * 32 + lane;
+        const int row = m64 ? quarter * 16 + (lane & 15) : quarter * 32 + lane;
         uint32_t piece = 0;
         for (int i = 0; i < n_my; ++i) {
             const int buf = i & 1;
@@ -411,6 +414,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 uint8_t* stg = smem + OFF_STG + (piece & 1) * lin::STG_BYTES;
                 if (warp == 2 && lane == 0) tma_store_wait_read1();
                 named_bar_sync(1, 128);
+                if (!m64 || lane < 16)
 #pragma unroll
                 for (int c16 = 0; c16 < 8; ++c16) {
                     const uint4 val = make_uint4(

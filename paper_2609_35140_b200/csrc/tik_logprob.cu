@@ -36,7 +36,10 @@ struct Cfg {
 };
 }  // namespace lp
 
-template <bool PAIR>
+// M64 (single CTAs, one token tile of at most 64 rows): M64 MMAs and 64 staged rows, half the tensor work --
+// such a call streams lm_head at the power cap, where that work costs memory throughput: 16 rows, H 1536 92 ->
+// 84 us, 64 rows, H 5120 280 -> 267.  Accumulator row i then sits on lane i % 16 of lane quarter i / 16.
+template <bool PAIR, bool M64>
 __global__ void __launch_bounds__(lp::THREADS, 1)
 logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const LogprobParams p) {
@@ -45,7 +48,8 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr int STAGES = C::STAGES;
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, OFF_BAR = C::OFF_BAR;
     constexpr uint32_t TMEM_COLS = 512;      // two 256-column accumulators
-    constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : 128, NB, false);
+    constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : M64 ? 64 : 128, NB, false);
+    constexpr uint32_t STAGED_BYTES = (M64 ? A_BYTES / 2 : A_BYTES) + C::B_BYTES;
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;     // 0 = the CTA that issues the pair's MMAs
 
@@ -166,7 +170,7 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         tma_load_2d_pair(sbase + s * STAGE_BYTES + A_BYTES, &tmB, lead_full + 8 * s, kb * 64,
                                          col0 + 128 * static_cast<int>(rank));
                     } else {
-                        mbar_expect_tx(bar_full + 8 * s, STAGE_BYTES);
+                        mbar_expect_tx(bar_full + 8 * s, STAGED_BYTES);
                         tma_load_2d(sbase + s * STAGE_BYTES, &tmA, bar_full + 8 * s, kb * 64, tok0);
                         tma_load_2d(sbase + s * STAGE_BYTES + A_BYTES, &tmB, bar_full + 8 * s, kb * 64, col0);
                     }
@@ -213,9 +217,10 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5)
         const int quarter = warp & 3;                      // TMEM lane quarter of this warp
-        const int row = quarter * 32 + lane;
+        const int row = M64 ? quarter * 16 + (lane & 15) : quarter * 32 + lane;
+        const bool own_row = !M64 || lane < 16;
         long long t = static_cast<long long>(tok_fixed) + row;
-        bool row_valid = t < p.T;
+        bool row_valid = own_row && t < p.T;
         int target = (!unit_mode && row_valid) ? p.target[t] : -1;
         const float it_scale = p.inv_temperature;
         uint32_t acc = 0;
@@ -224,7 +229,7 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int col_base = unit_mode ? unit_col(sp) : (sup0 + sp) * LP_SUPER;
         if (unit_mode) {                                   // the unit's token tile
             t = static_cast<long long>(unit_tok(sp)) + row;
-            row_valid = t < p.T;
+            row_valid = own_row && t < p.T;
             target = row_valid ? p.target[t] : -1;
         }
         float M = -CUDART_INF_F, Lsum = 0.0f;
@@ -416,11 +421,11 @@ __global__ void __launch_bounds__(256) logprob_finish_tiles_kernel(const Logprob
     if (threadIdx.x == 0) lp_write(p, t, Mt, Lt);
 }
 
-template <bool PAIR>
+template <bool PAIR, bool M64>
 static cudaError_t launch_logprob_main(const CUtensorMap& tmA, const CUtensorMap& tmB, const LogprobParams& p,
                                        cudaStream_t stream) {
     using C = lp::Cfg<PAIR>;
-    auto kern = logprob_kernel<PAIR>;
+    auto kern = logprob_kernel<PAIR, M64>;
     static DeviceOnce configured;     // the opt-in belongs to the (function, device) pair
     {
         cudaError_t e = configured.run([&]() {
@@ -439,11 +444,13 @@ static cudaError_t launch_logprob_main(const CUtensorMap& tmA, const CUtensorMap
     return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), lp::THREADS, C::ALLOC, stream, PAIR ? 2 : 1, tmA, tmB, p);
 }
 
-// pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of the 256 columns)
+// T <= 64: tmA must have a box of 64 rows; pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of the 256 columns)
 cudaError_t launch_logprob(const CUtensorMap& tmA, const CUtensorMap& tmB, const LogprobParams& p, bool pair,
                            cudaStream_t stream) {
     if (p.T <= 0) return cudaSuccess;
-    cudaError_t e = pair ? launch_logprob_main<true>(tmA, tmB, p, stream) : launch_logprob_main<false>(tmA, tmB, p, stream);
+    cudaError_t e = pair ? launch_logprob_main<true, false>(tmA, tmB, p, stream)
+                    : p.T <= 64 ? launch_logprob_main<false, true>(tmA, tmB, p, stream)
+                                : launch_logprob_main<false, false>(tmA, tmB, p, stream);
     if (e != cudaSuccess) return e;
     return launch_pdl(p.unit_mode ? logprob_finish_tiles_kernel : logprob_finish_kernel,
                       dim3(static_cast<unsigned>(p.unit_mode ? p.T : (p.T + 7) / 8)), 256, 0, stream, 1, p);
