@@ -247,10 +247,9 @@ __device__ __forceinline__ float swiglu_value(float g, float u) {
 // is applied once per output element when dQ / dK leave their fp32 accumulators.
 __device__ __forceinline__ float bwd_p(float s, float c, float lse_log2) { return ex2_ftz(__fmaf_rn(s, c, -lse_log2)); }
 __device__ __forceinline__ float bwd_ds(float p, float dp, float delta) { return __fmul_rn(p, __fsub_rn(dp, delta)); }
-// the same for two neighbouring columns with two-wide instructions (identical roundings)
-__device__ __forceinline__ void bwd_pds_x2(float s0, float s1, float dp0, float dp1, float c, float nl2_0, float nl2_1,
-                                           float ndl0, float ndl1, float& p0, float& p1, float& ds0, float& ds1) {
-    float x0, x1, t0, t1;
+// the same for two neighbouring columns with two-wide instructions (identical roundings); the scalars come negated
+__device__ __forceinline__ void bwd_p_x2(float s0, float s1, float c, float nl2_0, float nl2_1, float& p0, float& p1) {
+    float x0, x1;
     asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
         "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\tmov.b64 rc, {%5, %6};\n\t"
         "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
@@ -258,6 +257,10 @@ __device__ __forceinline__ void bwd_pds_x2(float s0, float s1, float dp0, float 
         : "f"(s0), "f"(s1), "f"(c), "f"(nl2_0), "f"(nl2_1));
     p0 = ex2_ftz(x0);
     p1 = ex2_ftz(x1);
+}
+__device__ __forceinline__ void bwd_ds_x2(float p0, float p1, float dp0, float dp1, float ndl0, float ndl1, float& ds0,
+                                          float& ds1) {
+    float t0, t1;
     asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
         "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
         "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
@@ -268,6 +271,11 @@ __device__ __forceinline__ void bwd_pds_x2(float s0, float s1, float dp0, float 
         "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
         : "=f"(ds0), "=f"(ds1)
         : "f"(p0), "f"(p1), "f"(t0), "f"(t1));
+}
+__device__ __forceinline__ void bwd_pds_x2(float s0, float s1, float dp0, float dp1, float c, float nl2_0, float nl2_1,
+                                           float ndl0, float ndl1, float& p0, float& p1, float& ds0, float& ds1) {
+    bwd_p_x2(s0, s1, c, nl2_0, nl2_1, p0, p1);
+    bwd_ds_x2(p0, p1, dp0, dp1, ndl0, ndl1, ds0, ds1);
 }
 
 }  // namespace tik
