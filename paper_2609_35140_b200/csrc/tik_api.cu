@@ -662,14 +662,15 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     uint64_t bd[2] = {static_cast<uint64_t>(K), static_cast<uint64_t>(N)};
     uint64_t st1[1] = {static_cast<uint64_t>(K) * 2};
     uint32_t box[2] = {64, 128};
-    const bool pair = T > 128;           // CTA pairs (two-SM MMAs) as soon as there is more than one row tile
-    // one row tile: the decode-shaped schedule (persistent CTAs over column units, only the rows
-    // that exist staged); same MMA chain per output element, so the same bits
-    const bool unit_mode = !pair;
+    // More than 16 row tiles: CTA pairs in a band raster (x no longer fits L2).  Up to 16: persistent CTAs or
+    // pairs over (column step, row tiles) units -- a grid of one CTA per unit spends as long on set-up as on a
+    // unit's 56 .. 432 K slices.  Same MMA chain per output element, so the same bits.
+    const long long ntile = (T + 127) / 128;
+    const bool units = ntile <= 16;
     const int a_rows = T <= 32 ? 32 : T <= 64 ? 64 : 128;
-    const int nu = unit_mode ? linear_unit_cols(N, a_rows, ctx->sm_count) : 0;
-    uint32_t boxA[2] = {64, unit_mode ? static_cast<uint32_t>(a_rows) : 128u};
-    uint32_t boxB[2] = {64, unit_mode ? static_cast<uint32_t>(nu) : pair ? 128u : 256u};
+    const LinearChoice c = units ? linear_choose(T, K, N, a_rows, ctx->sm_count) : LinearChoice{true, 256};
+    uint32_t boxA[2] = {64, static_cast<uint32_t>(c.pair ? 128 : a_rows)};
+    uint32_t boxB[2] = {64, static_cast<uint32_t>(c.pair ? 128 : c.nu)};
     CUtensorMap tmY;
     uint64_t yd[2] = {static_cast<uint64_t>(N), static_cast<uint64_t>(T)};
     uint64_t ys[1] = {static_cast<uint64_t>(N) * 2};
@@ -687,25 +688,20 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     // steps are then dealt evenly (N = 5120: two super-chunks of 10 steps, not 16 + 4, whose short
     // CTAs left a quarter of the last wave idle).  An output element is one 256-column accumulator's
     // chain over K either way: its bits do not depend on this choice.
-    const long long ntile = (T + 127) / 128;
     const int steps = (N + 255) / 256;
     int nsup = (steps + 15) / 16;
     while (nsup < steps && ntile * nsup < 4ll * ctx->sm_count) nsup = nsup * 2 < steps ? nsup * 2 : steps;
     const int per = (steps + nsup - 1) / nsup;
     p.super_cols = per * 256;
     p.nsuper = (steps + per - 1) / per;
-    // two to sixteen row tiles (decode batches up to 256, prefill-sized calls up to 2048 rows): the pair
-    // kernel, persistent over (256-column step, pair of row tiles) units -- a grid of one CTA pair per
-    // unit spends as long on set-up as on a unit's 56 .. 432 K slices, and x fits L2
-    const bool pair_units = pair && ntile <= 16;
-    p.unit_mode = (unit_mode || pair_units) ? 1 : 0;
-    p.nu = nu;
-    p.ntp = static_cast<int>((ntile + 1) / 2);
-    p.nunit = unit_mode ? (N + nu - 1) / nu : pair_units ? steps * p.ntp : 0;
+    p.unit_mode = units ? 1 : 0;
+    p.nu = c.nu;
+    p.ntp = static_cast<int>(c.pair ? (ntile + 1) / 2 : ntile);
+    p.nunit = units ? (N + c.nu - 1) / c.nu * p.ntp : 0;
     p.a_rows = a_rows;
     p.sm_count = ctx->sm_count;
     p.dev_status = ctx->dev_status;
-    cudaError_t e = launch_linear(tmA, tmB, tmY, p, pair, static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_linear(tmA, tmB, tmY, p, c.pair, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_linear");
 }
 

@@ -204,42 +204,46 @@ struct LinearParams {
     __nv_bfloat16* y;            // [T][N]
     int64_t T;
     int K, N, nsuper;
-    int super_cols;              // output columns per CTA: a multiple of 256, at most 4096
-    int unit_mode;               // T <= 128: persistent CTAs over column units (tmA box a_rows, tmB box nu rows)
-    int ntp;                     // pair unit mode: pairs of row tiles (1 .. 8)
-    int nu, nunit, a_rows;       // unit width 64 / 128 / 256, ceil(N / nu), staged x rows 32 / 64 / 128
+    int super_cols;              // pairs, band raster: output columns per CTA, a multiple of 256, at most 4096
+    int unit_mode;               // persistent CTAs (pairs) over nunit units
+    int ntp;                     // units per column step: row tiles (pairs: pairs of row tiles)
+    int nu, nunit, a_rows;       // columns per unit 64 / 128 / 256 (pairs: 256), units, staged x rows 32 / 64 / 128
                                  // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 16 .. 80)
     int kps;                     // narrow outputs: K slices per ring stage
     int sm_count;
     int* dev_status;
 };
-// Unit width of the decode-shaped linear kernel, from a cost model of one 64-wide K slice of one
-// unit on a B200: its four MMAs (N = 256: 270 ns, 128: 135 ns, 64: 100 ns -- shared-memory bound) plus
-// the issuing thread's ~170 ns per stage spread over the stage's slices; or the slice's bytes (x
-// rows and W rows) into one SM at ~95 GB/s; or its W bytes at the CTA's share of ~6.5 TB/s -- whichever
-// is longest; a CTA runs `waves` units one after the other.  The cheapest width wins, the wider one
-// on ties (x is staged once per unit).
-inline int linear_unit_cols(int N, int a_rows, int sm_count) {
-    int best = 256;
-    double best_cost = -1.0;
-    for (int nu = 256; nu >= 64; nu /= 2) {
-        const long long units = (N + nu - 1) / nu;
-        const long long waves = (units + sm_count - 1) / sm_count;
-        const double active = static_cast<double>(units < sm_count ? units : sm_count);
-        const double mma_ns = nu == 256 ? 270.0 : nu == 128 ? 135.0 : 100.0;
-        int kps = 256 / nu;
-        while (kps > 1 && (192 * 1024) / ((a_rows + nu) * 128 * kps) < 3) kps >>= 1;
-        double slice_ns = mma_ns + 170.0 / kps;
-        const double fill_ns = (a_rows + nu) * 128.0 / 95.0;
-        const double hbm_ns = nu * 128.0 / (6500.0 / active);
-        if (fill_ns > slice_ns) slice_ns = fill_ns;
-        if (hbm_ns > slice_ns) slice_ns = hbm_ns;
-        const double cost = waves * slice_ns;
-        if (best_cost < 0.0 || cost < best_cost * 0.999) {
-            best_cost = cost;
-            best = nu;
+// Schedule of a call of at most 16 row tiles, from a cost model: rounds of units x K slices x the time of one
+// 64-wide K slice, as measured on a B200 with W out of HBM.  A single CTA takes in x and W rows at ~130 GB/s
+// (128 rows: N = 64 190 ns, 128 235 ns, 256 370 ns); a pair's slice (256 x 256) is its MMAs, ~300 ns, and a
+// pair costs ~2 us more to set up and to drain.  Ties go to pairs and the wider unit (fewer bytes out of L2).
+// Before, every call of 129 .. 2048 rows ran as pairs; us, pairs -> the choice, W out of HBM:
+//   K 8960,  N 1536:   129 rows 44.2 -> 29.8 (64 columns), 1024 rows 44.6 -> 34.3 (128), 2000 rows 47 (pairs)
+//   K 18944, N 3584:   129 rows 88.5 -> 61.0 (64), 512 rows 89.1 -> 73.6 (128), 741 rows 91.1 (pairs; 128: 140)
+//   K 3584,  N 3584:   129 rows 21.0 -> 14.6 (64), 512 rows 21.2 -> 16.1 (128)
+//   K 1536,  N 256:    129 .. 2000 rows 11.7 -> 7.5 (64)
+//   K 3584,  N 37888:  278 rows 89.1 -> 82.6 (256), 512 rows 98 (pairs; 256: 109)
+struct LinearChoice {
+    bool pair;
+    int nu;
+};
+inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_count) {
+    const long long ntile = (T + 127) / 128;
+    LinearChoice best = {false, 256};
+    double best_us = -1.0;
+    auto consider = [&](bool pair, int nu) {
+        const long long slots = pair ? sm_count / 2 : sm_count;
+        const long long units = static_cast<long long>((N + nu - 1) / nu) * (pair ? (ntile + 1) / 2 : ntile);
+        const long long rounds = (units + slots - 1) / slots;
+        const double slice_ns = pair ? 300.0 : (a_rows + nu) * 128.0 / 130.0;
+        const double us = rounds * (K / 64) * slice_ns * 1e-3 + (pair ? 2.0 : 0.0);
+        if (best_us < 0.0 || us < best_us * 0.98) {
+            best_us = us;
+            best = {pair, nu};
         }
-    }
+    };
+    if (ntile > 1) consider(true, 256);
+    for (int nu = 256; nu >= 64; nu /= 2) consider(false, nu);
     return best;
 }
 // T <= 80 and N <= 64 sm_count; tmW / tmX: [K / 64][rows][64] views with boxes of 64 x nu x kps and 64 x a_rows x kps

@@ -1,12 +1,14 @@
 // Dense linear layer y = x W^T (bf16 in, fp32 accumulation in TMEM, bf16 out) for sm_100a: the
-// FFN projections of the unified operator set.  Same machinery as the log-probability GEMM: one
-// CTA = (128-row tile, super-chunk of 256 to 4096 output columns); a TMA warp streams 64-wide K slices of x and W
-// through a four-stage shared-memory ring, an MMA warp accumulates the whole K range in ascending
-// order into one of two 256-column TMEM accumulators (M128 x N256 x K16, no split-K), and four
-// epilogue warps (one thread per row) round the accumulator to bf16 and send it out through
-// shared memory and tiled TMA stores while the next 256 columns are being accumulated.  An output element is one fixed chain of MMAs over K, so it
-// depends on its x row and its W row only: a row gives the same bits whether it is computed alone
-// (decode) or inside a long batch (prefill, policy update).
+// FFN projections of the unified operator set.  An output element is one fixed chain of K16 MMAs in
+// ascending K into one fp32 accumulator (no split-K), so it depends on its x row and its W row only: a
+// row gives the same bits whether it is computed alone (decode) or inside a long batch (prefill, policy
+// update), and whichever of the three kernels below computes it:
+//   linear_kernel         CTA pairs (two-SM M256 MMAs), for calls that fill the chip: band raster, or
+//                         persistent over (column step, pair of row tiles) units
+//   linear_unit_kernel    persistent single CTAs over (column unit, row tile) units, for calls of few rows or
+//                         narrow outputs that pairs of 256 x 256 would leave idle SMs
+//   linear_narrow_kernel  weights as the M operand, for decode-sized calls with a narrow output
+// linear_choose (tik_internal.h) picks by a cost model.
 #include "tik_core.cuh"
 #include "tik_internal.h"
 #include "tik_ptx.cuh"
@@ -19,32 +21,28 @@ constexpr uint32_t A_BYTES = 128 * 128;      // 128 rows x 64 bf16
 constexpr uint32_t STG_BYTES = 128 * 128;    // output staging: 128 rows x 64 bf16, two buffers
 constexpr int BAND = 32;                     // row tiles per L2 band (even: CTA pairs stay inside a band)
 constexpr int THREADS = 192;                 // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
-// PAIR: two CTAs on neighbouring SMs share every MMA (M = 256 rows); each stages its own 128 rows of
-// x and 128 of the 256 weight rows of a step, as in the log-probability kernel.
-template <bool PAIR>
-struct Cfg {
-    static constexpr int STAGES = PAIR ? 6 : 4;
-    static constexpr uint32_t B_BYTES = (PAIR ? NB / 2 : NB) * 128;
-    static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr uint32_t OFF_STG = STAGES * STAGE_BYTES;
-    static constexpr uint32_t OFF_BAR = OFF_STG + 2 * STG_BYTES;
-    static constexpr uint32_t BYTES = OFF_BAR + 256;
-    static constexpr uint32_t ALLOC = BYTES + 1024;
-};
+// Two CTAs on neighbouring SMs share every MMA (M = 256 rows); each stages its own 128 rows of
+// x and half of a step's weight rows, as in the log-probability kernel.
+constexpr int STAGES = 6;
+constexpr uint32_t STAGE_BYTES = A_BYTES + (NB / 2) * 128;
+constexpr uint32_t OFF_STG = STAGES * STAGE_BYTES;
+constexpr uint32_t OFF_BAR = OFF_STG + 2 * STG_BYTES;
+constexpr uint32_t BYTES = OFF_BAR + 256;
+constexpr uint32_t ALLOC = BYTES + 1024;
 }  // namespace lin
 
-template <bool PAIR>
+// A TMA warp streams 64-wide K slices of x and W through a shared-memory ring, an MMA warp accumulates the
+// whole K range into one of two 256-column TMEM accumulators, and four epilogue warps (one thread per row)
+// round the accumulator to bf16 and send it out through shared memory and tiled TMA stores while the next
+// step is being accumulated.
 __global__ void __launch_bounds__(lin::THREADS, 1)
 linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               const __grid_constant__ CUtensorMap tmY, const LinearParams p) {
     using namespace lin;
-    using C = Cfg<PAIR>;
-    constexpr int STAGES = C::STAGES;
-    constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES, OFF_STG = C::OFF_STG, OFF_BAR = C::OFF_BAR;
     constexpr uint32_t TMEM_COLS = 512;      // two 256-column accumulators
-    constexpr uint32_t IDESC = mma_idesc_bf16(PAIR ? 256 : 128, NB, false);
+    constexpr uint32_t IDESC = mma_idesc_bf16(256, NB, false);
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
-    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;     // 0 = the CTA that issues the pair's MMAs
+    const uint32_t rank = cluster_ctarank();     // 0 = the CTA that issues the pair's MMAs
 
     // raster: bands of BAND row tiles; within a band the row tile varies fastest so the CTAs in
     // flight share one super-chunk of W in L2 and W is streamed from HBM once per band
@@ -55,13 +53,13 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     const long long rem = blockIdx.x - band * per_band;
     const int sup = static_cast<int>(rem / BAND);
     const int tile_in_band = static_cast<int>(rem % BAND);
-    // unit mode (up to 16 row tiles, CTA pairs only): one persistent pair per two SMs walks the
-    // units q = pair index, + number of pairs, ...; unit q = (256-column step q / ntp, pair of row
+    // unit mode (up to 16 row tiles): one persistent pair per two SMs walks the
+    // units q = pair index, + number of pairs, ...; unit q = (column step q / ntp, pair of row
     // tiles q % ntp): the pairs running at one time share a few steps of W in L2, and x (at most
     // 2048 rows) stays there throughout.  Same MMA chain per element.
-    const bool unit_mode = PAIR && p.unit_mode != 0;
+    const bool unit_mode = p.unit_mode != 0;
     const int u_first = static_cast<int>(blockIdx.x >> 1), u_stride = static_cast<int>(gridDim.x >> 1);
-    if (!unit_mode && (PAIR ? (tile_in_band & ~1) : tile_in_band) >= band_tiles) {   // a pair leaves only together
+    if (!unit_mode && (tile_in_band & ~1) >= band_tiles) {   // a pair leaves only together
         pdl_wait();
         return;
     }
@@ -95,38 +93,33 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_acc_full + 8 * b, 1);
-            mbar_init(bar_acc_empty + 8 * b, PAIR ? 256 : 128);
+            mbar_init(bar_acc_empty + 8 * b, 256);
         }
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         tma_prefetch_desc(&tmY);
         // this CTA's first weight tiles on their way to L2 while the kernel before this one drains
-        const int first_col = col_of(0) + (PAIR ? 128 * static_cast<int>(rank) : 0);
+        const int first_col = col_of(0) + (NB / 2) * static_cast<int>(rank);
         if (static_cast<int>(blockIdx.x) < p.sm_count && first_col < p.N)
             for (int kb = 0; kb < min(n_kb, STAGES); ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, first_col);
     }
     if (warp == 1) {
-        if (PAIR) {
-            tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
-            tmem_relinquish_pair();
-        } else {
-            tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
-            tmem_relinquish();
-        }
+        tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
+        tmem_relinquish_pair();
     }
     pdl_wait();
     pdl_launch_dependents();
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
-    if (PAIR) cluster_sync_all();            // the peer's barriers exist before anything signals them
+    cluster_sync_all();            // the peer's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const uint32_t lead_full = PAIR ? mapa_cluster(bar_full, 0) : bar_full;
-    const uint32_t lead_acc_empty = PAIR ? mapa_cluster(bar_acc_empty, 0) : bar_acc_empty;
-    const uint32_t peer_empty = PAIR ? mapa_cluster(bar_empty, 1) : bar_empty;
-    const uint32_t peer_acc_full = PAIR ? mapa_cluster(bar_acc_full, 1) : bar_acc_full;
+    const uint32_t lead_full = mapa_cluster(bar_full, 0);
+    const uint32_t lead_acc_empty = mapa_cluster(bar_acc_empty, 0);
+    const uint32_t peer_empty = mapa_cluster(bar_empty, 1);
+    const uint32_t peer_acc_full = mapa_cluster(bar_acc_full, 1);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -140,16 +133,10 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     const uint32_t use = it / STAGES;
                     if (use > 0) mbar_wait(bar_empty + 8 * s, (use - 1) & 1, abort_word, p.dev_status);
                     // rows past T and W rows past N are outside the tensor maps and arrive as zeros
-                    if (PAIR) {
-                        if (rank == 0) mbar_expect_tx(bar_full + 8 * s, 2 * STAGE_BYTES);   // both CTAs' bytes
-                        tma_load_2d_pair(sbase + s * STAGE_BYTES, &tmA, lead_full + 8 * s, kb * 64, row0);
-                        tma_load_2d_pair(sbase + s * STAGE_BYTES + A_BYTES, &tmB, lead_full + 8 * s, kb * 64,
-                                         col0 + 128 * static_cast<int>(rank));
-                    } else {
-                        mbar_expect_tx(bar_full + 8 * s, STAGE_BYTES);
-                        tma_load_2d(sbase + s * STAGE_BYTES, &tmA, bar_full + 8 * s, kb * 64, row0);
-                        tma_load_2d(sbase + s * STAGE_BYTES + A_BYTES, &tmB, bar_full + 8 * s, kb * 64, col0);
-                    }
+                    if (rank == 0) mbar_expect_tx(bar_full + 8 * s, 2 * STAGE_BYTES);   // both CTAs' bytes
+                    tma_load_2d_pair(sbase + s * STAGE_BYTES, &tmA, lead_full + 8 * s, kb * 64, row0);
+                    tma_load_2d_pair(sbase + s * STAGE_BYTES + A_BYTES, &tmB, lead_full + 8 * s, kb * 64,
+                                     col0 + (NB / 2) * static_cast<int>(rank));
                 }
             }
         }
@@ -169,23 +156,12 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     mbar_wait_warp(bar_full + 8 * s, (it / STAGES) & 1, abort_word, p.dev_status);
                     tc_fence_after();
                     const uint32_t a0 = sbase + s * STAGE_BYTES, b0 = a0 + A_BYTES;
-                    if (PAIR) {
-                        mma_ss_chain4_pair(tmem + buf * NB, smem_desc_sw128(a0, 0, 1024), smem_desc_sw128(b0, 0, 1024),
-                                           IDESC, kb ? 1u : 0u);
-                        mma_commit_pair(bar_empty + 8 * s);
-                        mma_commit_pair(peer_empty + 8 * s);
-                    } else {
-                        mma_ss_chain4(tmem + buf * NB, smem_desc_sw128(a0, 0, 1024), smem_desc_sw128(b0, 0, 1024),
-                                      IDESC, kb ? 1u : 0u);
-                        mma_commit(bar_empty + 8 * s);
-                    }
+                    mma_ss_chain4_pair(tmem + buf * NB, smem_desc_sw128(a0, 0, 1024), smem_desc_sw128(b0, 0, 1024), IDESC, kb ? 1u : 0u);
+                    mma_commit_pair(bar_empty + 8 * s);
+                    mma_commit_pair(peer_empty + 8 * s);
                 }
-                if (PAIR) {
-                    mma_commit_pair(bar_acc_full + 8 * buf);
-                    mma_commit_pair(peer_acc_full + 8 * buf);
-                } else {
-                    mma_commit(bar_acc_full + 8 * buf);
-                }
+                mma_commit_pair(bar_acc_full + 8 * buf);
+                mma_commit_pair(peer_acc_full + 8 * buf);
             }
         }
     } else {
@@ -233,8 +209,7 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             }
             // all TMEM reads of this accumulator are done: hand it back to the MMA warp
             tc_fence_before();
-            if (PAIR) mbar_arrive_cluster(lead_acc_empty + 8 * buf);
-            else mbar_arrive(bar_acc_empty + 8 * buf);
+            mbar_arrive_cluster(lead_acc_empty + 8 * buf);
         }
         if (warp == 2 && lane == 0) tma_store_wait_read();     // shared memory stays valid until the last read
     }
@@ -246,23 +221,20 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
     tc_fence_before();
     __syncthreads();
-    if (PAIR) cluster_sync_all();            // neither CTA leaves while the other may still touch it
-    if (warp == 1) {
-        if (PAIR) tmem_dealloc_pair(tmem, TMEM_COLS);
-        else tmem_dealloc(tmem, TMEM_COLS);
-    }
+    cluster_sync_all();            // neither CTA leaves while the other may still touch it
+    if (warp == 1) tmem_dealloc_pair(tmem, TMEM_COLS);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Decode-shaped calls (one row tile: T <= 128).  The work is one pass over W at HBM rate, so the
-// schedule is built for bytes in flight and even SM load instead of tensor throughput: the grid is
-// one persistent CTA per SM walking column units u = blockIdx.x, + gridDim.x, ...; a unit is
-// `nu` = 64, 128 or 256 output columns (the host picks the width from a cost model);
+// Calls of few rows (one row tile: a decode step) and of up to 16 row tiles whose output is too narrow for
+// the pair kernel's 256 x 256 units to occupy the SMs.  A call of one row tile is one pass over W at HBM
+// rate, so the schedule is built for bytes in flight and even SM load: the grid is one persistent
+// CTA per SM walking units u = blockIdx.x, + gridDim.x, ...; a unit is `nu` = 64, 128 or 256 output columns of
+// one row tile (row tile fastest: the CTAs running at one time share W columns in L2);
 // only `a_rows` = 32, 64 or 128 rows of x are staged per K slice (the MMA spans 64 or 128 rows: rows
 // past a_rows read whatever the stage holds, their accumulator rows are never stored); the ring
-// has as many stages as fit in 192 KiB (3 .. 4) of one, two or four K slices each, and the producer runs ahead into the next unit
-// while the epilogue of the last one drains.  An output element is still one chain of K16 MMAs in
-// ascending K into one fp32 accumulator, so its bits equal those of the batched kernel.
+// has as many stages as fit in 192 KiB (3 .. 12) of one, two or four K slices each, and the producer runs ahead
+// into the next unit while the epilogue of the last one drains.
 namespace linu {
 constexpr uint32_t RING_BYTES = 192 * 1024;
 constexpr int MAX_STAGES = 12;
@@ -295,6 +267,10 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     // accumulator row i then sits on lane i % 16 of lane quarter i / 16.
     const bool m64 = p.a_rows <= 64;
     const uint32_t idesc = mma_idesc_bf16(m64 ? 64 : 128, nu, false);
+    // (the divisions, for calls of one row tile, cost 0.2 us of 6)
+    auto unit_of = [&](int i) { return static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x); };
+    auto unit_col = [&](int i) { return (p.ntp == 1 ? unit_of(i) : unit_of(i) / p.ntp) * nu; };
+    auto unit_row = [&](int i) { return p.ntp == 1 ? 0 : unit_of(i) % p.ntp * 128; };
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -324,7 +300,8 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // the first 256 KiB of this CTA's weights are requested into L2 while the kernel before this
         // one drains (an HBM-bound call whose x is a few KiB has nothing else to wait for)
         const int ahead = min(n_kb, static_cast<int>((256u * 1024u) / (static_cast<uint32_t>(nu) * 128u)));
-        for (int kb = 0; kb < ahead; ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, static_cast<int>(blockIdx.x) * nu);
+        const int first_col = unit_col(0);
+        for (int kb = 0; kb < ahead; ++kb) tma_prefetch_l2_2d(&tmB, kb * 64, first_col);
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), TMEM_COLS);
@@ -344,7 +321,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             int s = 0;
             uint32_t use = 0;                    // how often stage s has been filled before
             for (int i = 0; i < n_my; ++i) {
-                const int col0 = (static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x)) * nu;
+                const int col0 = unit_col(i), row0 = unit_row(i);
                 for (int kb = 0; kb < n_kb; kb += kps) {
                     if (*abort_word) break;
                     if (use > 0) mbar_wait(bar_empty + 8 * s, (use - 1) & 1, abort_word, p.dev_status);
@@ -353,7 +330,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     for (int sl = 0; sl < ns; ++sl) {
                         const uint32_t dst = sbase + s * stage_bytes + sl * slice_bytes;
                         tma_load_2d(dst + a_bytes, &tmB, bar_full + 8 * s, (kb + sl) * 64, col0);   // W rows past N: zeros
-                        tma_load_2d(dst, &tmA, bar_full + 8 * s, (kb + sl) * 64, 0);                // x rows past T: zeros
+                        tma_load_2d(dst, &tmA, bar_full + 8 * s, (kb + sl) * 64, row0);             // x rows past T: zeros
                     }
                     if (++s == nst) {
                         s = 0;
@@ -402,7 +379,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             const int buf = i & 1;
             mbar_wait(bar_acc_full + 8 * buf, (i >> 1) & 1, abort_word, p.dev_status);
             tc_fence_after();
-            const int col0 = (static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x)) * nu;
+            const int col0 = unit_col(i), row0 = unit_row(i);
             const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + buf * 256;
 #pragma unroll 1
             for (int q = 0; q < nu / 64; ++q, ++piece) {
@@ -427,7 +404,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 fence_proxy_async_smem();
                 named_bar_sync(1, 128);
                 if (warp == 2 && lane == 0) {
-                    tma_store_2d(&tmY, smem_u32(stg), col0 + 64 * q, 0);
+                    tma_store_2d(&tmY, smem_u32(stg), col0 + 64 * q, row0);
                     tma_store_commit();
                 }
             }
@@ -613,35 +590,24 @@ cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX,
     return launch_pdl(linear_narrow_kernel, dim3(static_cast<unsigned>(p.nunit)), lin::THREADS, linn::ALLOC, stream, 1, tmW, tmX, p);
 }
 
-template <bool PAIR>
-static cudaError_t launch_linear_t(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,
-                                   const LinearParams& p, cudaStream_t stream) {
-    using C = lin::Cfg<PAIR>;
-    auto kern = linear_kernel<PAIR>;
-    static DeviceOnce configured;     // the opt-in belongs to the (function, device) pair
-    {
-        cudaError_t e = configured.run([&]() {
-            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        static_cast<int>(C::ALLOC));
-        });
-        if (e != cudaSuccess) return e;
-    }
-    const long long ntile = (p.T + 127) / 128;
-    const long long nband = (ntile + lin::BAND - 1) / lin::BAND;
-    long long grid = nband * lin::BAND * p.nsuper;               // even: BAND is
-    if (PAIR && p.unit_mode) {
-        const int slots = p.sm_count / 2;
-        grid = 2ll * (slots < p.nunit ? slots : p.nunit);
-    }
-    return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), lin::THREADS, C::ALLOC, stream, PAIR ? 2 : 1, tmA, tmB, tmY, p);
-}
-
-// pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of a step's 256)
+// pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of a step's)
 cudaError_t launch_linear(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,
                           const LinearParams& p, bool pair, cudaStream_t stream) {
     if (p.T <= 0) return cudaSuccess;
-    if (p.unit_mode && !pair) return launch_linear_unit(tmA, tmB, tmY, p, stream);
-    return pair ? launch_linear_t<true>(tmA, tmB, tmY, p, stream) : launch_linear_t<false>(tmA, tmB, tmY, p, stream);
+    if (!pair) return launch_linear_unit(tmA, tmB, tmY, p, stream);
+    static DeviceOnce configured;     // the opt-in belongs to the (function, device) pair
+    cudaError_t e = configured.run([&]() {
+        return cudaFuncSetAttribute(linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(lin::ALLOC));
+    });
+    if (e != cudaSuccess) return e;
+    const long long ntile = (p.T + 127) / 128;
+    const long long nband = (ntile + lin::BAND - 1) / lin::BAND;
+    long long grid = nband * lin::BAND * p.nsuper;               // even: BAND is
+    if (p.unit_mode) {
+        const int slots = p.sm_count / 2;
+        grid = 2ll * (slots < p.nunit ? slots : p.nunit);
+    }
+    return launch_pdl(linear_kernel, dim3(static_cast<unsigned>(grid)), lin::THREADS, lin::ALLOC, stream, 2, tmA, tmB, tmY, p);
 }
 
 }  // namespace tik

@@ -181,3 +181,23 @@ def test_narrow_linear_equals_rows_of_a_batched_call(tik, K, N):
         assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
         assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
     assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("K,N", [(64, 8), (192, 1000), (576, 1536), (320, 9480), (128, 37888)])
+def test_mid_size_linear_equals_rows_of_a_batched_call(tik, K, N):
+    """2 .. 16 row tiles: single CTAs over units of 64, 128 or 256 columns x one row tile, or pairs, by a cost
+    model that reaches each of them at these sizes.  Row counts around the tiles and around the range's ends:
+    the bits of a longer call (band raster), nothing written outside y."""
+    x = _randn((2300, K), 3300 + K)
+    W = _randn((N, K), 3400 + N % 977, 0.02)
+    y = tik.tik_linear(x, W)
+    rows = [0, 1150, 2299]
+    ref = oracle.linear(x[rows].float().cpu().numpy(), W.float().cpu().numpy())
+    g = y[rows].float().cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(g - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4 * 0.02 * np.sqrt(K))
+    for a, T in [(0, 129), (7, 255), (130, 256), (9, 257), (3, 385), (500, 768), (77, 1025), (1, 1500), (128, 2047), (252, 2048), (5, 2049)]:
+        buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
+        tik.tik_linear(x[a:a + T].contiguous(), W, y=buf[1:T + 1])
+        assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
+        assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
+    assert tik.device_status() == 0
