@@ -633,16 +633,15 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     if (T >= (1ll << 31) - 128) return fail(ctx, TIK_ERR_UNSUPPORTED, "T must be < 2^31 - 128");
     CUtensorMap tmA, tmB;
     std::string err;
-    if (T <= 80 && N <= 64ll * ctx->sm_count) {     // see linear_narrow_kernel
-        LinearParams p{};
-        p.y = static_cast<__nv_bfloat16*>(y);
-        p.T = T;
-        p.K = K;
-        p.N = N;
-        p.dev_status = ctx->dev_status;
-        p.nu = 8 * ((N + 8 * ctx->sm_count - 1) / (8 * ctx->sm_count));     // weight rows per CTA: whole 8-row swizzle atoms
-        p.nunit = (N + p.nu - 1) / p.nu;
-        p.a_rows = 16 * ((static_cast<int>(T) + 15) / 16);
+    const long long ntile = (T + 127) / 128;
+    LinearParams p{};
+    p.y = static_cast<__nv_bfloat16*>(y);
+    p.T = T;
+    p.K = K;
+    p.N = N;
+    p.sm_count = ctx->sm_count;
+    p.dev_status = ctx->dev_status;
+    if (linear_narrow_choose(p)) {
         // as many K slices per stage (a barrier round trip and a commit of the issuing warp, ~280 clk against 25
         // per MMA) as leave four stages, or 16 of them and three (16 rows, K 8960, N 1536: 20.5 -> 18.5 us)
         p.kps = 16;
@@ -665,7 +664,6 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     // More than 16 row tiles: CTA pairs in a band raster (x no longer fits L2).  Up to 16: persistent CTAs or
     // pairs over (column step, row tiles) units -- a grid of one CTA per unit spends as long on set-up as on a
     // unit's 56 .. 432 K slices.  Same MMA chain per output element, so the same bits.
-    const long long ntile = (T + 127) / 128;
     const bool units = ntile <= 16;
     const int a_rows = T <= 32 ? 32 : T <= 64 ? 64 : 128;
     const LinearChoice c = units ? linear_choose(T, K, N, a_rows, ctx->sm_count) : LinearChoice{true, 256};
@@ -677,11 +675,6 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     if (!make_tmap_bf16(ctx, &tmA, x, 2, ad, st1, boxA, &err) || !make_tmap_bf16(ctx, &tmB, weight, 2, bd, st1, boxB, &err) ||
         !make_tmap_bf16(ctx, &tmY, y, 2, yd, ys, box, &err))
         return fail(ctx, TIK_ERR_CUDA, err.c_str());
-    LinearParams p{};
-    p.y = static_cast<__nv_bfloat16*>(y);
-    p.T = T;
-    p.K = K;
-    p.N = N;
     // Columns per CTA (a "super-chunk" of 256-column steps): up to 16 steps amortise a CTA's set-up
     // and its last epilogue, which runs after the MMAs have ended; with few row tiles that would leave
     // SMs idle, so the number of super-chunks doubles until the grid covers the SMs four times.  The
@@ -699,8 +692,6 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     p.ntp = static_cast<int>(c.pair ? (ntile + 1) / 2 : ntile);
     p.nunit = units ? (N + c.nu - 1) / c.nu * p.ntp : 0;
     p.a_rows = a_rows;
-    p.sm_count = ctx->sm_count;
-    p.dev_status = ctx->dev_status;
     cudaError_t e = launch_linear(tmA, tmB, tmY, p, c.pair, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_linear");
 }

@@ -208,8 +208,9 @@ struct LinearParams {
     int unit_mode;               // persistent CTAs (pairs) over nunit units
     int ntp;                     // units per column step: row tiles (pairs: pairs of row tiles)
     int nu, nunit, a_rows;       // columns per unit 64 / 128 / 256 (pairs: 256), units, staged x rows 32 / 64 / 128
-                                 // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 16 .. 80)
+                                 // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 8 .. 128)
     int kps;                     // narrow outputs: K slices per ring stage
+    int m;                       // narrow outputs: rows of the M operand if that is x: 64 or 128; 0: the weights
     int sm_count;
     int* dev_status;
 };
@@ -246,7 +247,29 @@ inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_
     for (int nu = 256; nu >= 64; nu /= 2) consider(false, nu);
     return best;
 }
-// T <= 80 and N <= 64 sm_count; tmW / tmX: [K / 64][rows][64] views with boxes of 64 x nu x kps and 64 x a_rows x kps
+// The narrow schedule: one unit of nu weight rows x one row tile per CTA, nu as few as spread the call over the
+// SMs (whole 8-row swizzle atoms; an MMA of 128 rows takes N = 16 i).  Its time is the MMAs' shared-memory reads,
+// 64 or 128 rows of the M operand + the N operand's, and what TMA writes there: the operand whose choice as M
+// reads fewer rows is M (x must be for more than 80 rows).  Above 48 weight rows and 80 x rows the unit
+// kernel is as fast or faster (K 18944, N 3584, 256 rows: 53.1 us, 54.5 here; K 1536, N 8960, 128 rows: 8.3, 8.5).
+inline bool linear_narrow_choose(LinearParams& p) {
+    const long long ntile = (p.T + 127) / 128;
+    const int rows = static_cast<int>(p.T < 128 ? p.T : 128), t16 = (rows + 15) / 16 * 16, m = rows > 64 ? 128 : 64;
+    auto weight_rows = [&](int atom) {
+        const long long per = static_cast<long long>(atom) * p.sm_count;
+        return atom * ((p.N * ntile + per - 1) / per);
+    };
+    const long long nw = weight_rows(8), nx = weight_rows(m == 128 ? 16 : 8);
+    const bool x_is_m = t16 > 80 || (m == 128 ? m + nx <= 64 + t16 : nx < t16);
+    if ((x_is_m ? nx : nw) > (t16 > 80 ? 48 : 64)) return false;
+    p.m = x_is_m ? m : 0;
+    p.nu = static_cast<int>(x_is_m ? nx : nw);
+    p.a_rows = x_is_m ? (rows + 7) / 8 * 8 : t16;
+    p.ntp = static_cast<int>(ntile);
+    p.nunit = (p.N + p.nu - 1) / p.nu * p.ntp;
+    return true;
+}
+// tmW / tmX: [K / 64][rows][64] views with boxes of 64 x nu x kps and 64 x a_rows x kps
 constexpr uint32_t LINEAR_NARROW_RING = 192 * 1024;
 cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX, const LinearParams& p, cudaStream_t stream);
 cudaError_t launch_linear(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,

@@ -7,8 +7,8 @@
 //                         persistent over (column step, pair of row tiles) units
 //   linear_unit_kernel    persistent single CTAs over (column unit, row tile) units, for calls of few rows or
 //                         narrow outputs that pairs of 256 x 256 would leave idle SMs
-//   linear_narrow_kernel  weights as the M operand, for decode-sized calls with a narrow output
-// linear_choose (tik_internal.h) picks by a cost model.
+//   linear_narrow_kernel  one unit of few weight rows per CTA, for narrow outputs
+// linear_narrow_choose and linear_choose (tik_internal.h) pick.
 #include "tik_core.cuh"
 #include "tik_internal.h"
 #include "tik_ptx.cuh"
@@ -437,38 +437,43 @@ static cudaError_t launch_linear_unit(const CUtensorMap& tmA, const CUtensorMap&
 }
 
 // ---------------------------------------------------------------------------------------------
-// Decode-shaped calls with a narrow output (T <= 80 and N <= 64 columns per SM: the down, q, k, v and
-// output projections of a rollout step).  linear_unit_kernel gives such a call at most N / 64 CTAs, each
-// pulling 64 weight rows and at least 32 x rows per K slice at the ~95 GB/s that one SM takes in; K is not
-// split (an element is one chain), so the way to shorten the call is fewer rows per CTA on more SMs.
-// Here the weights are the MMA's M operand -- M64, of which a CTA stages only its r = 8, 16, .. 64 rows, as
-// few as spread N over all SMs -- and x, rounded up to 16 rows, its N operand: an MMA reads 64 + T
-// shared-memory rows instead of 128 + 64.  The products of an element and the order of its sums are
-// those of the other schedules (operands exchanged), so are the bits.
+// Calls with a narrow output (the down, q, k, v and output projections of a rollout step, and calls of some row
+// tiles whose N is smaller still).  linear_unit_kernel gives such a call at most N / 64 CTAs per row tile; K is not
+// split (an element is one chain), so the way to shorten the call is fewer weight rows per CTA on more SMs: r = 8,
+// 16, .. 64 of them, as few as spread the call over all SMs, times one row tile.
+// What bounds it is the chain of K / 16 MMAs, which is a CTA's whatever its share of the work is: ~17 clk + one
+// per 128 bytes of the operands' rows in shared memory (K 18944, N 3584, 64 rows: 36.9 us, 32.9 with no copies at
+// all, 16.9 with a quarter of the MMAs).  So the operand that is M (64 or 128 rows are read, whatever is staged) is
+// the one whose choice reads fewer rows: the weights (M64) for few rows of x, x (M64, M128) for more.  The
+// products of an element and the order of its sums are the same either way, so are the bits.
 // Ring: stages of kps K slices; one TMA copy per operand and stage through a [K / 64][rows][64] view.
-// linear_unit_kernel -> this, cold L2: T = 16: K 8960, N 1536 28.5 -> 20.5 us; K 18944, N 3584 51 -> 33;
-// K 27648, N 5120 72 -> 51; T = 64: 28.6 -> 24.7, 51 -> 41, 74 -> 74.  At T = 128 x is most of what a CTA
-// takes in, on more CTAs here: 30.7 -> 34.8, 59 -> 62, 84 -> 86; at 80: 30.7 -> 26.7, 57.4 -> 53.3,
-// 82 -> 76; the line is drawn there.
+// linear_unit_kernel -> weights as M, cold L2: T = 16: K 8960, N 1536 28.5 -> 20.5 us; K 18944, N 3584 51 -> 33;
+// K 27648, N 5120 72 -> 51.  Weights as M -> x as M, W out of HBM: T = 64: K 1536, N 256 5.2 -> 4.4; K 8960,
+// N 1536 18.3 -> 15.4; K 3584, N 4608 10.4 -> 9.3; K 18944, N 3584 37.7 -> 34.8.  linear_unit_kernel -> x as M,
+// T = 100: K 8960, N 1536 24.6 -> 23.0; K 18944, N 3584 52.8 -> 49.1; T = 300: K 1536, N 256 6.5 -> 5.7.
 namespace linn {
 constexpr uint32_t RING_BYTES = LINEAR_NARROW_RING;
 constexpr int MAX_STAGES = 12;
-constexpr uint32_t OFF_BAR = RING_BYTES + 64 * 128;      // (a slice's M64 read may run past its r rows: never past this)
+constexpr uint32_t OFF_BAR = RING_BYTES + 64 * 128;      // (the M operand's read may run past its staged rows: never past this)
 constexpr uint32_t BYTES = OFF_BAR + 512;
 constexpr uint32_t ALLOC = BYTES + 1024;
 }  // namespace linn
 
+template <bool XM>     // the M operand: x (or its 128-row tiles), else the weights
 __global__ void __launch_bounds__(lin::THREADS, 1)
 linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const LinearParams p) {
     using namespace linn;
     constexpr uint32_t TMEM_COLS = 128;
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
-    const int r = p.nu, kps = p.kps, n_kb = p.K / 64, n0 = static_cast<int>(blockIdx.x) * r;
+    const int r = p.nu, kps = p.kps, n_kb = p.K / 64;
+    const int cu = !XM || p.ntp == 1 ? static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x) / p.ntp;
+    const int n0 = cu * r, row0 = XM ? (static_cast<int>(blockIdx.x) - cu * p.ntp) * 128 : 0;
+    const int m = XM ? p.m : 64;                 // rows of the M operand
     const uint32_t w_slice = static_cast<uint32_t>(r) * 128u, x_slice = static_cast<uint32_t>(p.a_rows) * 128u;
     const uint32_t w_bytes = w_slice * static_cast<uint32_t>(kps);
     const uint32_t stage_bytes = w_bytes + x_slice * static_cast<uint32_t>(kps);
     const int nst = min(MAX_STAGES, static_cast<int>(RING_BYTES / stage_bytes));
-    const uint32_t idesc = mma_idesc_bf16(64, p.a_rows, false);
+    const uint32_t idesc = mma_idesc_bf16(m, XM ? r : p.a_rows, false);
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -518,7 +523,7 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
                 // W rows past N, x rows past T and slices past K arrive as zeros
                 mbar_expect_tx(bar_full + 8 * s, stage_bytes);
                 tma_load_3d(dst, &tmW, bar_full + 8 * s, 0, n0, kb);
-                tma_load_3d(dst + w_bytes, &tmX, bar_full + 8 * s, 0, 0, kb);
+                tma_load_3d(dst + w_bytes, &tmX, bar_full + 8 * s, 0, row0, kb);
                 if (++s == nst) {
                     s = 0;
                     ++use;
@@ -535,10 +540,11 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
                 if (*abort_word) break;
                 mbar_wait_warp(bar_full + 8 * s, use & 1, abort_word, p.dev_status);
                 tc_fence_after();
-                const uint32_t a0 = sbase + s * stage_bytes, b0 = a0 + w_bytes;
+                const uint32_t w0 = sbase + s * stage_bytes, x0 = w0 + w_bytes;
+                const uint32_t a0 = XM ? x0 : w0, b0 = XM ? w0 : x0, a_step = XM ? x_slice : w_slice, b_step = XM ? w_slice : x_slice;
                 const int ns = min(kps, n_kb - kb);
                 for (int sl = 0; sl < ns; ++sl)
-                    mma_ss_chain4(tmem, smem_desc_sw128(a0 + sl * w_slice, 0, 1024), smem_desc_sw128(b0 + sl * x_slice, 0, 1024),
+                    mma_ss_chain4(tmem, smem_desc_sw128(a0 + sl * a_step, 0, 1024), smem_desc_sw128(b0 + sl * b_step, 0, 1024),
                                   idesc, (kb + sl) ? 1u : 0u);
                 mma_commit(bar_empty + 8 * s);
                 if (++s == nst) {
@@ -550,18 +556,38 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5)
-        // An M64 accumulator has 16 rows (output columns) in each lane quarter; a column of it is a row of x.
+        // An M64 accumulator has 16 rows in each lane quarter, an M128 one 32.
         const int quarter = warp & 3;
-        const int m = 16 * quarter + lane;
-        const bool valid = lane < 16 && m < r && n0 + m < p.N;
+        const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+        const int i0 = (m == 64 ? 16 : 32) * quarter, i_m = i0 + lane;      // row of the M operand
+        const bool mine = m == 128 || lane < 16;
         mbar_wait(bar_acc, 0, abort_word, p.dev_status);
         tc_fence_after();
-        if (16 * quarter < r) {
+        if (XM) {                                // thread per row of x, r columns of it
+            const long long row = row0 + i_m;
+            const bool valid = mine && i_m < p.a_rows && row < p.T;
+            __nv_bfloat16* const y = p.y + row * p.N + n0;
+            if (row0 + i0 < p.T)
+                for (int c0 = 0; c0 < r; c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(taddr + c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 32; c += 8) {
+                        const uint4 val = make_uint4(pack_bf16x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])),
+                                                     pack_bf16x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])),
+                                                     pack_bf16x2(__uint_as_float(v[c + 4]), __uint_as_float(v[c + 5])),
+                                                     pack_bf16x2(__uint_as_float(v[c + 6]), __uint_as_float(v[c + 7])));
+                        if (valid && c0 + c < r && n0 + c0 + c < p.N) *reinterpret_cast<uint4*>(y + c0 + c) = val;
+                    }
+                }
+        } else if (i0 < r) {                     // thread per output column, a column of the accumulator is a row of x
+            const bool valid = mine && i_m < r && n0 + i_m < p.N;
             for (int c0 = 0; c0 < static_cast<int>(p.T); c0 += 32) {
                 uint32_t v[32];
-                tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, v);
+                tmem_ld32(taddr + c0, v);
                 tmem_wait_ld();
-                __nv_bfloat16* const y = p.y + static_cast<long long>(c0) * p.N + n0 + m;
+                __nv_bfloat16* const y = p.y + static_cast<long long>(c0) * p.N + n0 + i_m;
                 const int nt = min(32, static_cast<int>(p.T) - c0);
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
@@ -583,11 +609,15 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX, const LinearParams& p, cudaStream_t stream) {
     static DeviceOnce configured;
     cudaError_t e = configured.run([&]() {
-        return cudaFuncSetAttribute(linear_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(linn::ALLOC));
+        for (auto k : {linear_narrow_kernel<false>, linear_narrow_kernel<true>}) {
+            const cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(linn::ALLOC));
+            if (err != cudaSuccess) return err;
+        }
+        return cudaSuccess;
     });
     if (e != cudaSuccess) return e;
-    return launch_pdl(linear_narrow_kernel, dim3(static_cast<unsigned>(p.nunit)), lin::THREADS, linn::ALLOC, stream, 1, tmW, tmX, p);
+    return launch_pdl(p.m ? linear_narrow_kernel<true> : linear_narrow_kernel<false>, dim3(static_cast<unsigned>(p.nunit)),
+                      lin::THREADS, linn::ALLOC, stream, 1, tmW, tmX, p);
 }
 
 // pair = true: tmB must have a box of 128 rows (each CTA of a pair stages half of a step's)

@@ -201,3 +201,18 @@ def test_mid_size_linear_equals_rows_of_a_batched_call(tik, K, N):
         assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
         assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
     assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("K,N", [(64, 256), (576, 1536), (640, 4608), (192, 6000)])
+def test_narrow_linear_with_x_as_the_m_operand(tik, K, N):
+    """Row counts where x becomes the M operand of the narrow schedule (M64, M128, tiles of 128 rows), around the
+    8-row atoms and the tiles: the bits of a batched call, nothing written outside y."""
+    x = _randn((2300, K), 3500 + K)
+    W = _randn((N, K), 3600 + N % 977, 0.02)
+    y = tik.tik_linear(x, W)
+    for a, T in [(0, 17), (5, 24), (9, 40), (3, 41), (100, 63), (50, 64), (172, 65), (1, 72), (7, 88), (11, 127), (64, 128), (13, 129), (700, 260)]:
+        buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
+        tik.tik_linear(x[a:a + T].contiguous(), W, y=buf[1:T + 1])
+        assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
+        assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
+    assert tik.device_status() == 0
