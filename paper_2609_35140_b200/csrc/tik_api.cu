@@ -1,4 +1,5 @@
 // C ABI of libtik: argument checks, tensor maps, grid sizing from host upper bounds, launches.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -739,6 +740,17 @@ tik_status tik_attn_train_bwd(tik_ctx* ctx, const void* q, const void* k, const 
     p.c = scale_to_c(softmax_scale);
     p.scale = softmax_scale;
     p.dev_status = ctx->dev_status;
+    // Query heads per dQ CTA: a head's set-up, first loads and epilogue run under its neighbour's steps, but longer
+    // CTAs leave a longer tail.  Backward, us, 1 / 2 / 4 heads per CTA, with items (tile, head) per SM:
+    //   (d 128, 64/8 heads) 47 x 45..238 tokens, 41: 331 / 281 / 269;  21 x 77..681, 37: 559 / 478 / 471
+    //   (32/8) 10 x 385..2369, 23: 723 / 667 / 679;  8 x 100..400, 5.0: 65.8 / 61.6 / 64.7;  2048, 3.5: 132 / 135 / 161
+    //   (28/4) 16 x 1280..5120, 73: 3940 / 3817 / 3832;  32 x 60..128, 6.1: 68.7 / 62.9 / 64.0
+    //   (d 64, 4/1) 9 x 3440..7743, 11: 717 / 714 / 762;  40 x 100..500, 3.3: 36.2 / 36.3 / 36.9
+    const long long max_tiles = (max_seqlen + 127) / 128;
+    const long long items = std::min<long long>(total_tokens / 128 + S, max_tiles * S) * Hq;
+    p.dq_heads = items < 5ll * ctx->sm_count ? 1 : items < 12ll * ctx->sm_count || max_tiles > 12 ? 2 : 4;
+    p.dq_heads = std::min(p.dq_heads, p.G);
+    p.dq_groups = (p.G + p.dq_heads - 1) / p.dq_heads;
     cudaError_t e = launch_attn_bwd(d, (max_seqlen + 127) / 128, S, tmQ, tmK, tmV, tmDO, p, o, d_o,
                                     total_tokens * Hq, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_train_bwd");

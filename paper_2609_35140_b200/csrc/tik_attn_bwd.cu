@@ -5,6 +5,8 @@
 //   DQ  mode: a CTA owns one 128-row query tile of one (sequence, head) and walks the KV tiles
 //             0..i:      S = Q_i K_j^T, dP = dO_i V_j^T, dS = P o (dP - delta),
 //             dQ_i += dS K_j                                     (accumulator in TMEM)
+//             and then the same for the CTA's next query head of that KV head: its loads start with the last
+//             score products, its first steps run under the epilogue of the head before
 //   DKV mode: a CTA owns one 128-row KV tile of one (sequence, KV head) and walks the query
 //             tiles i >= j of the G query heads of that KV head, one after the other:
 //             S^T = K_j Q_i^T, dP^T = V_j dO_i^T, dV_j += P^T dO_i, dK_j += dS^T Q_i
@@ -90,13 +92,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         return;
     }
     const int nq = (len + 127) / 128;                      // tiles of the sequence (query and KV alike)
-    int own, head = 0, kvh, n_steps;
+    int own, head = 0, kvh, n_steps, n_heads = 1;
     if (MODE == BWD_DQ) {
         own = gridDim.x - 1 - blockIdx.x;                  // query tile, heaviest first
         if (own >= nq) return;                             // (never the last block: its tile is 0)
-        head = blockIdx.y;
-        kvh = head / p.G;
-        n_steps = own + 1;                                 // KV tiles 0..own
+        kvh = blockIdx.y / p.dq_groups;
+        const int g0 = (blockIdx.y - kvh * p.dq_groups) * p.dq_heads;
+        head = kvh * p.G + g0;                             // the first of the CTA's heads, taken one after the other
+        n_heads = min(p.dq_heads, p.G - g0);
+        n_steps = own + 1;                                 // KV tiles 0..own, for each of them
     } else {
         own = blockIdx.x;                                  // KV tile, heaviest first
         if (own >= nq) return;
@@ -139,6 +143,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_BAR + 128);
     volatile int* abort_word = reinterpret_cast<volatile int*>(smem + L::OFF_BAR + 132);
     const uint32_t bar_gdone = bar0 + 136;       // [2] DQ: the gradient product that read a dS tile is done
+    const uint32_t bar_rempty = bar0 + 152;      // DQ: a head's last score products have read the row-side tiles
     float* sc_base = reinterpret_cast<float*>(smem + L::OFF_SC);
 
     if (tid == 0) {
@@ -158,6 +163,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         mbar_init(bar_acc, 1);
         mbar_init(bar_gdone, 1);
         mbar_init(bar_gdone + 8, 1);
+        mbar_init(bar_rempty, 1);
         *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmQ);
@@ -178,22 +184,22 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             const int row_own = tok0 + 128 * own;
-            mbar_expect_tx(bar_r, 2 * L::TILE);
-            for (int a = 0; a < NATOM; ++a) {
-                if (MODE == BWD_DQ) {
-                    tma_load_3d(sR1 + a * L::ATOM, &tmQ, bar_r, a * 64, head, row_own);
-                    tma_load_3d(sR2 + a * L::ATOM, &tmDO, bar_r, a * 64, head, row_own);
-                } else {
-                    tma_load_3d(sR1 + a * L::ATOM, &tmK, bar_r, a * 64, kvh, row_own);
-                    tma_load_3d(sR2 + a * L::ATOM, &tmV, bar_r, a * 64, kvh, row_own);
+            auto load_rows = [&](int h) {
+                mbar_expect_tx(bar_r, 2 * L::TILE);
+                for (int a = 0; a < NATOM; ++a) {
+                    tma_load_3d(sR1 + a * L::ATOM, MODE == BWD_DQ ? &tmQ : &tmK, bar_r, a * 64, h, row_own);
+                    tma_load_3d(sR2 + a * L::ATOM, MODE == BWD_DQ ? &tmDO : &tmV, bar_r, a * 64, h, row_own);
                 }
-            }
+            };
+            load_rows(MODE == BWD_DQ ? head : kvh);
             const CUtensorMap* tm1 = MODE == BWD_DQ ? &tmK : &tmQ;
             const CUtensorMap* tm2 = MODE == BWD_DQ ? &tmV : &tmDO;
             Walk w = walk_start;
-            for (int t = 0; t < n_steps; ++t) {
+            const int n_all = n_steps * n_heads;
+            int tile = 0, hl = 0;                // DQ: KV tile and head of the CTA
+            for (int t = 0; t < n_all; ++t) {
                 if (*abort_word) break;          // a wait expired somewhere: stop issuing copies
-                const int row = tok0 + 128 * (MODE == BWD_DQ ? t : w.tile), h = MODE == BWD_DQ ? kvh : w.head;
+                const int row = tok0 + 128 * (MODE == BWD_DQ ? tile : w.tile), h = MODE == BWD_DQ ? kvh : w.head;
                 walk_on(w);
                 const int s1 = t % C1_STAGES, s2 = t % C2_STAGES;
                 if (t >= C1_STAGES) mbar_wait(bar_c1empty + 8 * s1, (t / C1_STAGES - 1) & 1, abort_word, p.dev_status);
@@ -204,6 +210,18 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 mbar_expect_tx(bar_c2full + 8 * s2, L::TILE);
                 for (int a = 0; a < NATOM; ++a)
                     tma_load_3d(sbase + L::OFF_C2 + s2 * L::TILE + a * L::ATOM, tm2, bar_c2full + 8 * s2, a * 64, h, row);
+                // the next head's rows, behind its first KV tile (whose stages are free before the rows are)
+                if (MODE == BWD_DQ) {
+                    if (tile == 0 && hl > 0) {
+                        mbar_wait(bar_rempty, (hl - 1) & 1, abort_word, p.dev_status);
+                        if (*abort_word) break;
+                        load_rows(head + hl);
+                    }
+                    if (++tile == n_steps) {
+                        tile = 0;
+                        ++hl;
+                    }
+                }
             }
         }
         __syncwarp();
@@ -211,7 +229,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // ------------------------------------------------------------ MMA issuer
         const uint32_t tmem = warp_uniform(*tmem_slot);
         const int n_steps = warp_uniform(n_steps_v);
-        mbar_wait_warp(bar_r, 0, abort_word, p.dev_status);
+        if (MODE == BWD_DKV) mbar_wait_warp(bar_r, 0, abort_word, p.dev_status);
         const uint64_t dr1 = smem_desc_sw128(sR1, 0, 1024), dr2 = smem_desc_sw128(sR2, 0, 1024);
         auto c1_addr = [&](int t) { return sbase + L::OFF_C1 + (t % C1_STAGES) * L::TILE; };
         auto c2_addr = [&](int t) { return sbase + L::OFF_C2 + (t % C2_STAGES) * L::TILE; };
@@ -230,8 +248,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             // element-wise threads hold it in registers, and dP / dS alternate between two tiles.  Both
             // score products of step t+1 are issued while the element-wise work of step t runs, the
             // gradient product of step t right behind them.
-            for (int t = 0; t < n_steps; ++t) {
+            const int n_all = n_steps * warp_uniform(n_heads);
+            for (int t = 0, tile = 0, hl = 0; t < n_all; ++t) {
                 if (*abort_word) break;
+                if (tile == 0) mbar_wait_warp(bar_r, hl & 1, abort_word, p.dev_status);
                 wait_c1(t);
                 wait_c2(t);
                 if (t > 0) mbar_wait_warp(bar_aux, (t - 1) & 1, abort_word, p.dev_status);   // S of step t-1 is in registers
@@ -243,6 +263,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 score((t & 1) ? COL_T2B : COL_T2, dr2, c2_addr(t));
                 mma_commit(bar_s);
                 mma_commit(bar_c2empty + 8 * (t % C2_STAGES));      // the V stage is done with
+                if (++tile == n_steps) {
+                    tile = 0;
+                    if (++hl < n_heads) mma_commit(bar_rempty);
+                }
             }
         } else {
             // MMAs issued by one warp execute in order: S(t+1) overwrites P(t) only after dV(t) has read it,
@@ -285,19 +309,24 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (MODE == BWD_DQ) {
             const uint32_t tmem = warp_uniform(*tmem_slot);
             const int n_steps = warp_uniform(n_steps_v);
-            for (int t = 0; t < n_steps; ++t) {
+            const int n_all = n_steps * warp_uniform(n_heads);
+            for (int t = 0, tile = 0; t < n_all; ++t) {
                 if (*abort_word) break;
+                // (a head's first dS is there only after every warp has read the previous head's accumulator)
                 mbar_wait_warp(bar_p, t & 1, abort_word, p.dev_status);
                 tc_fence_after();
                 // A = dS: every thread left its 32 columns' bf16 pairs in the first 16 columns of
                 // its own 32-column block, so the eight 16-key steps sit at 0, 8, 32, 40, ...
                 mma_ts_chain8_blocks(tmem + COL_A1, tmem + ((t & 1) ? COL_T2B : COL_T2),
                                      smem_desc_sw128(sbase + L::OFF_C1 + (t % C1_STAGES) * L::TILE, L::ATOM, 1024),
-                                     IDESC_OUT, t > 0 ? 1u : 0u);
+                                     IDESC_OUT, tile > 0 ? 1u : 0u);
                 mma_commit(bar_c1empty + 8 * (t % C1_STAGES));
                 mma_commit(bar_gdone + 8 * (t & 1));
+                if (++tile == n_steps) {
+                    tile = 0;
+                    mma_commit(bar_acc);
+                }
             }
-            mma_commit(bar_acc);
         }
         __syncwarp();
     } else {
@@ -309,12 +338,15 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const int row_abs = 128 * own + r;                 // position of this row in the sequence
         const float c = p.c;                               // scale * log2(e)
-        float row_l2 = 0.0f, row_dl = 0.0f;
-        if (MODE == BWD_DQ && row_abs < len) {
-            const long long idx = (static_cast<long long>(tok0) + row_abs) * p.Hq + head;
-            row_l2 = __fmul_rn(p.lse[idx], LOG2E_F);
-            row_dl = __ldcg(&p.delta[idx]);     // (around L1: no wait of this grid's own precedes the read)
-        }
+        auto fetch_row = [&](int h, float& l2, float& dl) {
+            l2 = 0.0f;
+            dl = 0.0f;
+            if (row_abs < len) {
+                const long long idx = (static_cast<long long>(tok0) + row_abs) * p.Hq + h;
+                l2 = __fmul_rn(p.lse[idx], LOG2E_F);
+                dl = __ldcg(&p.delta[idx]);     // (around L1: no wait of this grid's own precedes the read)
+            }
+        };
         // DKV: the scalars belong to the columns (query rows of the streamed tile).  Threads 0..127 fetch
         // those of the next step's columns; they reach the others through shared memory
         // (double-buffered, stored negated and as two arrays, so that neighbouring columns' values load
@@ -336,48 +368,86 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
             named_bar_sync(1, 512);
         };
-        if (MODE == BWD_DQ) {
-            const float nl2 = -row_l2, ndl = -row_dl;
-            for (int t = 0; t < n_steps; ++t) {
-                mbar_wait(bar_s, t & 1, abort_word, p.dev_status);
-                tc_fence_after();
-                const uint32_t t2 = tlane + ((t & 1) ? COL_T2B : COL_T2) + 32 * cq;
-                uint32_t s_[32], d_[32];
-                tmem_ld32(tlane + COL_T1 + 32 * cq, s_);
-                tmem_ld32(t2, d_);
+        // fp32 accumulators -> bf16 rows
+        auto epilogue = [&](int hd, uint32_t phase) {
+            mbar_wait(bar_acc, phase, abort_word, p.dev_status);
+            tc_fence_after();
+            const bool valid = row_abs < len;
+            const long long tok = static_cast<long long>(tok0) + row_abs;
+            __nv_bfloat16* out1 = (MODE == BWD_DQ) ? p.dq + (tok * p.Hq + hd) * D : p.dk + (tok * p.Hkv + kvh) * D;
+            __nv_bfloat16* out2 = p.dv + (tok * p.Hkv + kvh) * D;
+            // blocks of 32 columns of dQ (DKV: of dK, then dV) over the four threads of a row
+#pragma unroll 1
+            for (int u = cq; u < (MODE == BWD_DKV ? 2 : 1) * (D / 32); u += 4) {
+                const bool second = u >= D / 32;
+                const int col = 32 * (second ? u - D / 32 : u);
+                __nv_bfloat16* out = (second ? out2 : out1) + col;
+                const float osc = second ? 1.0f : p.scale;             // dQ, dK carry the softmax scale; dV does not
+                uint32_t v[32];
+                tmem_ld32(tlane + (second ? COL_A2 : COL_A1) + col, v);
                 tmem_wait_ld();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_aux);            // S is in registers: the next QK^T may overwrite it
-                uint32_t dk_[16];
-                if (t != own) {               // off the diagonal nothing is masked: two-wide, no compares
+                if (valid) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        float p0, p1, ds0, ds1;
-                        bwd_pds_x2(__uint_as_float(s_[i]), __uint_as_float(s_[i + 1]), __uint_as_float(d_[i]),
-                                   __uint_as_float(d_[i + 1]), c, nl2, nl2, ndl, ndl, p0, p1, ds0, ds1);
-                        dk_[i >> 1] = pack_bf16x2(ds0, ds1);
-                    }
-                } else {
-                    const int col0_abs = 128 * t + 32 * cq;
-#pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        float dsv[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const bool masked = col0_abs + i + e > row_abs;      // key after query
-                            const float pe = bwd_p(__uint_as_float(s_[i + e]), c, row_l2);
-                            dsv[e] = masked ? 0.0f : bwd_ds(pe, __uint_as_float(d_[i + e]), row_dl);
-                        }
-                        dk_[i >> 1] = pack_bf16x2(dsv[0], dsv[1]);
-                    }
+                    for (int i = 0; i < 4; ++i)
+                        reinterpret_cast<uint4*>(out)[i] = make_uint4(
+                            pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i]), osc), __fmul_rn(__uint_as_float(v[8 * i + 1]), osc)),
+                            pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 2]), osc), __fmul_rn(__uint_as_float(v[8 * i + 3]), osc)),
+                            pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 4]), osc), __fmul_rn(__uint_as_float(v[8 * i + 5]), osc)),
+                            pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 6]), osc), __fmul_rn(__uint_as_float(v[8 * i + 7]), osc)));
                 }
-                // dS goes over the first 16 of this thread's own 32 dP columns: no other thread reads them
-                tmem_st16(t2, dk_);
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_p);
+            }
+        };
+        if (MODE == BWD_DQ) {
+            float row_l2, row_dl, next_l2 = 0.0f, next_dl = 0.0f;
+            fetch_row(head, row_l2, row_dl);
+            int t = 0;                           // steps so far, of all heads
+            for (int hl = 0; hl < n_heads; ++hl) {
+                if (hl + 1 < n_heads) fetch_row(head + hl + 1, next_l2, next_dl);
+                const float nl2 = -row_l2, ndl = -row_dl;
+                for (int tile = 0; tile < n_steps; ++tile, ++t) {
+                    mbar_wait(bar_s, t & 1, abort_word, p.dev_status);
+                    tc_fence_after();
+                    const uint32_t t2 = tlane + ((t & 1) ? COL_T2B : COL_T2) + 32 * cq;
+                    uint32_t s_[32], d_[32];
+                    tmem_ld32(tlane + COL_T1 + 32 * cq, s_);
+                    tmem_ld32(t2, d_);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_aux);            // S is in registers: the next QK^T may overwrite it
+                    uint32_t dk_[16];
+                    if (tile != own) {               // off the diagonal nothing is masked: two-wide, no compares
+#pragma unroll
+                        for (int i = 0; i < 32; i += 2) {
+                            float p0, p1, ds0, ds1;
+                            bwd_pds_x2(__uint_as_float(s_[i]), __uint_as_float(s_[i + 1]), __uint_as_float(d_[i]),
+                                       __uint_as_float(d_[i + 1]), c, nl2, nl2, ndl, ndl, p0, p1, ds0, ds1);
+                            dk_[i >> 1] = pack_bf16x2(ds0, ds1);
+                        }
+                    } else {
+                        const int col0_abs = 128 * tile + 32 * cq;
+#pragma unroll
+                        for (int i = 0; i < 32; i += 2) {
+                            float dsv[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const bool masked = col0_abs + i + e > row_abs;      // key after query
+                                const float pe = bwd_p(__uint_as_float(s_[i + e]), c, row_l2);
+                                dsv[e] = masked ? 0.0f : bwd_ds(pe, __uint_as_float(d_[i + e]), row_dl);
+                            }
+                            dk_[i >> 1] = pack_bf16x2(dsv[0], dsv[1]);
+                        }
+                    }
+                    // dS goes over the first 16 of this thread's own 32 dP columns: no other thread reads them
+                    tmem_st16(t2, dk_);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_p);
+                }
+                epilogue(head + hl, hl & 1);
+                row_l2 = next_l2;
+                row_dl = next_dl;
             }
         } else {
             float l2, dl;
@@ -452,33 +522,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 if (lane == 0) mbar_arrive(bar_ds);
                 pass_col(t + 1, l2, dl);       // (the buffer was last read a step ago, before the previous barrier)
             }
-        }
-        // ---- epilogue: fp32 accumulators -> bf16 rows
-        mbar_wait(bar_acc, 0, abort_word, p.dev_status);
-        tc_fence_after();
-        const bool valid = row_abs < len;
-        const long long tok = static_cast<long long>(tok0) + row_abs;
-        __nv_bfloat16* out1 = (MODE == BWD_DQ) ? p.dq + (tok * p.Hq + head) * D : p.dk + (tok * p.Hkv + kvh) * D;
-        __nv_bfloat16* out2 = p.dv + (tok * p.Hkv + kvh) * D;
-        // blocks of 32 columns of dQ (DKV: of dK, then dV) over the four threads of a row
-#pragma unroll 1
-        for (int u = cq; u < (MODE == BWD_DKV ? 2 : 1) * (D / 32); u += 4) {
-            const bool second = u >= D / 32;
-            const int col = 32 * (second ? u - D / 32 : u);
-            __nv_bfloat16* out = (second ? out2 : out1) + col;
-            const float osc = second ? 1.0f : p.scale;             // dQ, dK carry the softmax scale; dV does not
-            uint32_t v[32];
-            tmem_ld32(tlane + (second ? COL_A2 : COL_A1) + col, v);
-            tmem_wait_ld();
-            if (valid) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    reinterpret_cast<uint4*>(out)[i] = make_uint4(
-                        pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i]), osc), __fmul_rn(__uint_as_float(v[8 * i + 1]), osc)),
-                        pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 2]), osc), __fmul_rn(__uint_as_float(v[8 * i + 3]), osc)),
-                        pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 4]), osc), __fmul_rn(__uint_as_float(v[8 * i + 5]), osc)),
-                        pack_bf16x2(__fmul_rn(__uint_as_float(v[8 * i + 6]), osc), __fmul_rn(__uint_as_float(v[8 * i + 7]), osc)));
-            }
+            epilogue(0, 0);
         }
     }
 
@@ -561,7 +605,7 @@ cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ,
     cudaError_t e = launch_pdl(d == 128 ? bwd_delta_kernel<128> : bwd_delta_kernel<64>, dim3(dgrid), 256, 0, stream, 1,
                                static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(dout), p.delta, n_vec);
     if (e != cudaSuccess) return e;
-    const dim3 gq(max_tiles, p.Hq, S), gkv(max_tiles, p.Hkv, S);
+    const dim3 gq(max_tiles, p.Hkv * p.dq_groups, S), gkv(max_tiles, p.Hkv, S);
     if (d == 128) {
         e = launch_bwd_t<128, BWD_DKV>(gkv, tmQ, tmK, tmV, tmDO, p, stream);
         if (e == cudaSuccess) e = launch_bwd_t<128, BWD_DQ>(gq, tmQ, tmK, tmV, tmDO, p, stream);

@@ -285,6 +285,7 @@ struct BwdParams {
     int Hq, Hkv, G;
     float c;                     // softmax_scale * log2(e)
     float scale;
+    int dq_heads, dq_groups;     // query heads per dQ CTA, CTAs per KV head: ceil(G / dq_heads)
     int* dev_status;
 };
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,

@@ -105,3 +105,23 @@ def test_backward_of_a_few_rows(tik, lens, Hq, Hkv, d):
                                   do.float().cpu().numpy(), w.cu_seqlens(), w.softmax_scale)
     for name, a, b in zip(("dq", "dk", "dv"), got, want):
         _check(a, b, name)
+
+
+@pytest.mark.parametrize("S,Hq,Hkv,d", [(14, 28, 4, 128), (40, 28, 4, 128), (60, 16, 2, 64), (40, 40, 20, 128)])
+def test_backward_of_many_short_sequences_equals_each_alone(tik, S, Hq, Hkv, d):
+    """Enough query tiles per SM that a dQ CTA takes two or four heads (a last group of fewer: 7 = 2 + 2 + 2 + 1 =
+    4 + 3, 2): the bits of a sequence alone, whose CTAs take one each."""
+    lens = [1 + (67 * i + 128) % 300 for i in range(S)]
+    w = synth.custom_workload([1] * S, [n - 1 for n in lens], Hq, Hkv, d, 64, index=58)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    do, _, _, _ = synth.make_qkv(w, "cuda", seed_offset=9)
+    got = _fwd_bwd(tik, w, q, k, v, cu, do)
+    cu_h = w.cu_seqlens()
+    for s in (0, 1, S // 2, S - 2, S - 1):
+        sl = slice(int(cu_h[s]), int(cu_h[s + 1]))
+        w1 = synth.custom_workload([1], [lens[s] - 1], Hq, Hkv, d, 64)
+        cu1 = torch.tensor([0, lens[s]], dtype=torch.int32, device="cuda")
+        alone = _fwd_bwd(tik, w1, q[sl].contiguous(), k[sl].contiguous(), v[sl].contiguous(), cu1, do[sl].contiguous())
+        for a, b in zip(alone, got):
+            assert count_diff(a, b[sl]) == 0, (s, lens[s])
+    assert tik.device_status() == 0
