@@ -1038,10 +1038,11 @@ __global__ void __launch_bounds__(D) combine_kernel(const AttnParams p) {
 }
 
 // ------------------------------------------------------------------ KV-cache write
-// A block copies KVW_TOK (8 or 1) consecutive new tokens (K and V rows of all KV heads: 16-byte vectors).
-// Warps 0 .. KVW_TOK-1 find their token's sequence, position and physical page; then all threads copy, every thread's loads issued before its stores.  (One token
-// per 128-thread block, each doing its own search before 32 bytes of copying per thread, reached
-// 0.76 of the copy bandwidth.)
+// A block copies KVW_TOK (8 or 1) consecutive new tokens (K and V rows of all KV heads: 16-byte vectors).  The
+// look-up of a token's page is a chain of four or five dependent loads, so the block's first loads of K and V are
+// issued before it (their addresses do not depend on it), warps 0 .. KVW_TOK-1 look up a token each, and as many
+// tokens per block as keep a prompt's blocks in one wave share that latency (8 heads x 128: 3 600 tokens one per
+// block 10.0 us, eight 5.2; 1 000 tokens 3.6, 2.8; a decode step's 256 2.5, 3.1).  32 000 tokens: 42 us, 6.2 TB/s.
 constexpr int KVW_THREADS = 256;
 template <int KVW_TOK>       // 8 for prompts, 1 for a decode step's handful of tokens (more blocks, shorter chains)
 __global__ void __launch_bounds__(KVW_THREADS)
@@ -1055,51 +1056,50 @@ kv_write_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new
     __shared__ long long dst_base[KVW_TOK];     // vector index of (page, head 0, row, 0), or -1
     const long long tok0 = static_cast<long long>(blockIdx.x) * KVW_TOK;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < KVW_TOK) {                              // warp w looks up token w
-        const long long token = tok0 + warp;
-        long long base = -1;
-        if (token < total_new) {
-            const int s = warp_find_sequence(cu_new, S, token, lane);
-            const int first = cu_new[s], end = cu_new[s + 1];
-            const int pos = ctx_lens[s] - (end - first) + static_cast<int>(token - first);
-            if (token < end && pos >= 0) {
-                const int lp = pos / page_size, row = pos % page_size;
-                const int phys = (lp < max_blocks) ? block_table[static_cast<long long>(s) * max_blocks + lp] : -1;
-                if (phys >= 0 && phys < num_pages) base = (static_cast<long long>(phys) * Hkv * page_size + row) * vec_per_head;
-                else if (lane == 0) atomicOr(dev_status, TIK_DEV_BAD_BLOCK);
-            }
-        }
-        if (lane == 0) dst_base[warp] = base;
-    }
-    __syncthreads();
     const int nvec = Hkv * vec_per_head;                 // vectors per token and tensor
-    const int per_block = KVW_TOK * nvec;
-    const long long head_pitch = static_cast<long long>(page_size) * vec_per_head;
-    for (int i0 = threadIdx.x; i0 < per_block; i0 += 4 * KVW_THREADS) {
+    const int per_block = static_cast<int>(min(static_cast<long long>(KVW_TOK), total_new - tok0)) * nvec;
+    for (int i0 = threadIdx.x; i0 - static_cast<int>(threadIdx.x) < per_block; i0 += 4 * KVW_THREADS) {
         uint4 kv[4], vv[4];
-        long long dst[4];
+        int tok[4], off[4];                              // token of the block, offset from its dst_base
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int i = i0 + u * KVW_THREADS;
-            dst[u] = -1;
             if (i < per_block) {
-                const int j = i / nvec, r = i - j * nvec;          // token of the block, vector of the token
-                const long long base = dst_base[j];
+                kv[u] = k_new[tok0 * nvec + i];
+                vv[u] = v_new[tok0 * nvec + i];
+                tok[u] = i / nvec;
+                const int v = i - tok[u] * nvec, head = v / vec_per_head;
+                off[u] = head * page_size * vec_per_head + v - head * vec_per_head;
+            }
+        }
+        if (i0 == static_cast<int>(threadIdx.x)) {       // the first loads are in flight: warp w looks up token w
+            const long long token = tok0 + warp;
+            if (warp < KVW_TOK && token < total_new) {
+                long long base = -1;
+                const int s = warp_find_sequence(cu_new, S, token, lane);
+                const int first = cu_new[s], end = cu_new[s + 1];
+                const int pos = ctx_lens[s] - (end - first) + static_cast<int>(token - first);
+                if (token < end && pos >= 0) {
+                    const int lp = pos / page_size, row = pos % page_size;
+                    const int phys = (lp < max_blocks) ? block_table[static_cast<long long>(s) * max_blocks + lp] : -1;
+                    if (phys >= 0 && phys < num_pages) base = (static_cast<long long>(phys) * Hkv * page_size + row) * vec_per_head;
+                    else if (lane == 0) atomicOr(dev_status, TIK_DEV_BAD_BLOCK);
+                }
+                if (lane == 0) dst_base[warp] = base;
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * KVW_THREADS;
+            if (i < per_block) {
+                const long long base = dst_base[tok[u]];
                 if (base >= 0) {
-                    const int hh = r / vec_per_head, e = r - hh * vec_per_head;
-                    dst[u] = base + hh * head_pitch + e;
-                    const long long src = (tok0 + j) * nvec + r;
-                    kv[u] = k_new[src];
-                    vv[u] = v_new[src];
+                    k_cache[base + off[u]] = kv[u];
+                    v_cache[base + off[u]] = vv[u];
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (dst[u] >= 0) {
-                k_cache[dst[u]] = kv[u];
-                v_cache[dst[u]] = vv[u];
-            }
     }
 }
 
@@ -1142,9 +1142,9 @@ cudaError_t launch_kv_write(const void* k_new, const void* v_new, const int32_t*
                             int Hkv, int d, int page_size, int num_pages, int* dev_status,
                             cudaStream_t stream) {
     if (total_new <= 0) return cudaSuccess;
-    const bool prompt = total_new >= 4096;
-    return launch_pdl(prompt ? kv_write_kernel<8> : kv_write_kernel<1>,
-                      dim3(static_cast<unsigned>(prompt ? (total_new + 7) / 8 : total_new)), KVW_THREADS, 0, stream, 1,
+    const int tok = total_new >= 512 ? 8 : 1;
+    auto kern = tok == 8 ? kv_write_kernel<8> : kv_write_kernel<1>;
+    return launch_pdl(kern, dim3(static_cast<unsigned>((total_new + tok - 1) / tok)), KVW_THREADS, 0, stream, 1,
                       static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), cu_new, ctx_lens,
                       static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), block_table, max_blocks, S, total_new, Hkv,
                       d * 2 / 16, page_size, num_pages, dev_status);

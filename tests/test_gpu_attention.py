@@ -183,3 +183,26 @@ def test_prefill_kv_equals_cache_write_then_prefill(tik):
                                     ro.bt, max(lens), max(b), w.softmax_scale)
         assert count_diff(o, o_ref) == 0
         assert torch.equal(bits(kc), bits(ro.kc)) and torch.equal(bits(vc), bits(ro.vc))
+
+
+@pytest.mark.parametrize("total", [1, 511, 512, 517, 1500])
+@pytest.mark.parametrize("Hkv,d", [(1, 64), (8, 128), (20, 128)])
+def test_kv_cache_write_block_sizes(tik, total, Hkv, d):
+    """One or eight tokens per block, a last block of fewer, fewer and more vectors than a block loads at a time:
+    every row where the table says, nothing else written."""
+    page, lens = 16, [total // 3, total - total // 3]
+    g = torch.Generator(device="cuda").manual_seed(total + Hkv)
+    k, v = (torch.randn(total, Hkv, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    cu = torch.tensor([0, lens[0], total], dtype=torch.int32, device="cuda")
+    ctx = torch.tensor([lens[0], lens[1] + 5], dtype=torch.int32, device="cuda")
+    mb = (max(lens) + 5 + page - 1) // page
+    table = torch.randperm(2 * mb, generator=g, device="cuda").to(torch.int32).view(2, mb)
+    kc, vc = (torch.full((2 * mb, Hkv, page, d), 3.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    want_k, want_v = kc.clone(), vc.clone()
+    seq = (torch.arange(total, device="cuda") >= lens[0]).long()
+    pos = torch.where(seq == 0, torch.arange(total, device="cuda"), torch.arange(total, device="cuda") - lens[0] + 5)
+    phys, row = table[seq, pos // page].long(), pos % page
+    want_k[phys, :, row], want_v[phys, :, row] = k, v
+    tik.tik_kv_cache_write(k, v, cu, ctx, kc, vc, table)
+    assert torch.equal(kc, want_k) and torch.equal(vc, want_v)
+    assert tik.device_status() == 0
