@@ -643,11 +643,17 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     p.sm_count = ctx->sm_count;
     p.dev_status = ctx->dev_status;
     if (linear_narrow_choose(p)) {
-        // as many K slices per stage (a barrier round trip and a commit of the issuing warp, ~280 clk against 25
-        // per MMA) as leave four stages, or 16 of them and three (16 rows, K 8960, N 1536: 20.5 -> 18.5 us)
-        p.kps = 16;
-        while (p.kps > 1 && (p.kps > K / 64 || LINEAR_NARROW_RING / ((p.nu + p.a_rows) * 128u * p.kps) < (p.kps == 16 ? 3u : 4u)))
-            p.kps /= 2;
+        // K slices per stage: a stage costs the issuing warp a barrier round trip and a commit, ~280 clk against 25 per
+        // MMA, so as many (16 at most) as leave three stages, or four where the chain is long and its steady state
+        // decides or W's share of a CTA is large.  Few rows with the largest shares are HBM-bound and want no more than
+        // 160 KiB in flight (16 rows, K 2048, N 9400: 8.3 us, 8.8 with 200 KiB).  Four or more stages of 4, 2 or 1
+        // slices before -> this: 98 rows, K 8960, N 1536 22.9 -> 19.5 us, K 18944, N 3584 48.7 -> 44.5 (32 rows 32.4
+        // -> 30.2); 64 rows, K 8960 15.4 -> 13.5.  128 rows: K 18944, N 3584 four stages 49.0, three 54.1; K 3584,
+        // N 4608 12.5, 12.0.
+        const uint32_t slices = LINEAR_NARROW_RING / ((p.nu + p.a_rows) * 128u), stages = K > 10240 || p.nu >= 48 ? 4 : 3;
+        p.kps = static_cast<int>(std::max(1u, std::min({16u, slices / stages, static_cast<uint32_t>(K / 64)})));
+        p.nst = static_cast<int>(std::min(12u, slices / p.kps));
+        if (p.nu > 48 && p.a_rows <= 32) p.kps = p.nst = 4;
         const uint64_t st3[2] = {static_cast<uint64_t>(K) * 2, 128};
         const uint64_t wd[3] = {64, static_cast<uint64_t>(N), static_cast<uint64_t>(K / 64)};
         const uint64_t xd[3] = {64, static_cast<uint64_t>(T), static_cast<uint64_t>(K / 64)};

@@ -209,7 +209,7 @@ struct LinearParams {
     int ntp;                     // units per column step: row tiles (pairs: pairs of row tiles)
     int nu, nunit, a_rows;       // columns per unit 64 / 128 / 256 (pairs: 256), units, staged x rows 32 / 64 / 128
                                  // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 8 .. 128)
-    int kps;                     // narrow outputs: K slices per ring stage
+    int kps, nst;                // narrow outputs: K slices per ring stage, stages (12 at most)
     int m;                       // narrow outputs: rows of the M operand if that is x: 64 or 128; 0: the weights
     int sm_count;
     int* dev_status;
@@ -270,7 +270,7 @@ inline bool linear_narrow_choose(LinearParams& p) {
     return true;
 }
 // tmW / tmX: [K / 64][rows][64] views with boxes of 64 x nu x kps and 64 x a_rows x kps
-constexpr uint32_t LINEAR_NARROW_RING = 192 * 1024;
+constexpr uint32_t LINEAR_NARROW_RING = 216 * 1024;
 cudaError_t launch_linear_narrow(const CUtensorMap& tmW, const CUtensorMap& tmX, const LinearParams& p, cudaStream_t stream);
 cudaError_t launch_linear(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmY,
                           const LinearParams& p, bool pair, cudaStream_t stream);

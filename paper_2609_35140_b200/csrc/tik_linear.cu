@@ -472,7 +472,7 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     const uint32_t w_slice = static_cast<uint32_t>(r) * 128u, x_slice = static_cast<uint32_t>(p.a_rows) * 128u;
     const uint32_t w_bytes = w_slice * static_cast<uint32_t>(kps);
     const uint32_t stage_bytes = w_bytes + x_slice * static_cast<uint32_t>(kps);
-    const int nst = min(MAX_STAGES, static_cast<int>(RING_BYTES / stage_bytes));
+    const int nst = p.nst;
     const uint32_t idesc = mma_idesc_bf16(m, XM ? r : p.a_rows, false);
 
     extern __shared__ uint8_t smem_raw[];
