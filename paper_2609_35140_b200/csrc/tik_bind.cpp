@@ -117,6 +117,10 @@ void want_rank(const at::Tensor& t, int64_t rank) {
     if (t.dim() != rank)
         raise(PyExc_ValueError, "expected a tensor with " + std::to_string(rank) + " dimensions, got " + std::to_string(t.dim()));
 }
+// an argument of which only one axis' size is read
+void want_axis(const at::Tensor& t, int64_t axis) {
+    if (t.dim() <= axis) raise(PyExc_IndexError, "axis " + std::to_string(axis) + " of a tensor with " + std::to_string(t.dim()) + " dimensions");
+}
 int dim(const at::Tensor& t, int64_t i) {
     const int64_t v = t.size(i);
     if (v > INT32_MAX) raise(PyExc_OverflowError, "tensor dimension out of range");
@@ -134,14 +138,16 @@ void check(tik_status rc, const tik_ctx* ctx) {
     if (rc != TIK_OK) raise_tik(std::string(tik_status_str(rc)) + ": " + tik_last_error(ctx));
 }
 
-// Runs a C entry point without the interpreter lock (a launch blocks while the launch queue is full).
+// Runs a C entry point without the interpreter lock (a launch blocks while the launch queue is full).  f reads
+// plain values only: whatever inspects a tensor or may raise happens before, under the lock.  An exception that
+// leaves f all the same passes with the lock taken back, so that its handler may set a Python error.
 template <class F>
 tik_status unlocked(F&& f) {
-    tik_status rc;
-    Py_BEGIN_ALLOW_THREADS;
-    rc = f();
-    Py_END_ALLOW_THREADS;
-    return rc;
+    struct Unlock {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Unlock() { PyEval_RestoreThread(state); }
+    } unlock;
+    return f();
 }
 
 struct Scratch {
@@ -202,7 +208,7 @@ PyObject* attn_train_fwd(Args a) {
     const at::Tensor *o_in = a.opt(), *lse = a.opt();
     PyObject* ws_in = a.next();
     want_rank(q, 3);
-    if (k.dim() < 2) want_rank(k, 3);
+    want_axis(k, 1);
     at::Tensor made;
     const at::Tensor& o = out_or(o_in, made, q.sizes(), q.scalar_type(), q);
     const int S = static_cast<int>(cu.numel() - 1);
@@ -211,8 +217,9 @@ PyObject* attn_train_fwd(Args a) {
     float* lp = f32(lse);
     int32_t* cp = i32(cu);
     const int Hq = dim(q, 1), Hkv = dim(k, 1), d = dim(q, 2);
-    check(unlocked([&] { return tik_attn_train_fwd(ctx, qp, kp, vp, op, lp, cp, S, q.size(0), max_seqlen, Hq, Hkv, d, scale,
-                                                   ws.p, ws.bytes, st); }), ctx);
+    const int64_t tot = q.size(0);
+    check(unlocked([&] { return tik_attn_train_fwd(ctx, qp, kp, vp, op, lp, cp, S, tot, max_seqlen, Hq, Hkv, d, scale, ws.p,
+                                                   ws.bytes, st); }), ctx);
     return wrap(o_in, made);
 }
 
@@ -225,7 +232,7 @@ PyObject* attn_train_bwd(Args a) {
     const float scale = a.real();
     const at::Tensor* ws_in = a.opt();
     want_rank(q, 3);
-    if (k.dim() < 2) want_rank(k, 3);
+    want_axis(k, 1);
     const int64_t tot = q.size(0);
     const int Hq = dim(q, 1), Hkv = dim(k, 1), d = dim(q, 2), S = static_cast<int>(cu.numel() - 1);
     const Scratch ws = sized_ws(ws_in, tik_workspace_bytes(TIK_OP_ATTN_TRAIN_BWD, tot, Hq, Hkv, d, 0, 0, 0), q);
@@ -248,7 +255,7 @@ struct Cache {
 };
 Cache cache_of(const at::Tensor& kc, const at::Tensor& vc, const at::Tensor& table) {
     want_rank(kc, 4);
-    want_rank(table, 2);
+    want_axis(table, 1);
     return {bf(kc), bf(vc), i32(table), dim(table, 1), dim(kc, 0), dim(kc, 1), dim(kc, 2), dim(kc, 3)};
 }
 
@@ -257,12 +264,14 @@ PyObject* kv_cache_write(Args a) {
     const at::Tensor& k = a.tensor();
     const at::Tensor *v = a.opt(), *cu = a.opt();
     const at::Tensor &lens = a.tensor(), &kc = a.tensor(), &vc = a.tensor(), &table = a.tensor();
+    want_axis(k, 0);
     const Cache c = cache_of(kc, vc, table);
     void *kp = bf(k), *vp = bf(v), *st = stream();
     int32_t *cp = i32(cu), *lp = i32(lens);
     const int S = static_cast<int>(lens.numel());
-    check(unlocked([&] { return tik_kv_cache_write(ctx, kp, vp, cp, lp, c.k, c.v, c.table, c.max_blocks, S, k.size(0), c.Hkv,
-                                                   c.d, c.page, c.num_pages, st); }), ctx);
+    const int64_t n = k.size(0);
+    check(unlocked([&] { return tik_kv_cache_write(ctx, kp, vp, cp, lp, c.k, c.v, c.table, c.max_blocks, S, n, c.Hkv, c.d,
+                                                   c.page, c.num_pages, st); }), ctx);
     Py_RETURN_NONE;
 }
 
@@ -274,16 +283,19 @@ PyObject* qk_norm_rope_kv_write(Args a) {
     const at::Tensor &cs = a.tensor(), &cu = a.tensor();
     const at::Tensor *lens = a.opt(), *kc = a.opt(), *vc = a.opt(), *table = a.opt();
     want_rank(q, 3);
-    if (k.dim() < 2) want_rank(k, 3);
-    if (kc) want_rank(*kc, 4);
-    if (table) want_rank(*table, 2);
+    want_axis(k, 1);
+    want_axis(cs, 0);
+    if (kc) want_axis(*kc, 2);
+    if (table) want_axis(*table, 1);
     const int Hq = dim(q, 1), Hkv = dim(k, 1), d = dim(q, 2), page = kc ? dim(*kc, 2) : 0, pages = kc ? dim(*kc, 0) : 0;
     const int max_blocks = table ? dim(*table, 1) : 0, S = static_cast<int>(cu.numel() - 1);
     void *qp = bf(q), *kp = bf(k), *vp = bf(v), *wqp = bf(wq), *wkp = bf(wk), *kcp = bf(kc), *vcp = bf(vc), *st = stream();
     const float* csp = f32(&cs);
     int32_t *cp = i32(cu), *lp = i32(lens), *tp = i32(table);
-    check(unlocked([&] { return tik_qk_norm_rope_kv_write(ctx, qp, kp, vp, wqp, wkp, eps, csp, dim(cs, 0), cp, lp, kcp, vcp, tp,
-                                                          max_blocks, S, q.size(0), Hq, Hkv, d, page, pages, st); }), ctx);
+    const int64_t n = q.size(0);
+    const int max_pos = dim(cs, 0);
+    check(unlocked([&] { return tik_qk_norm_rope_kv_write(ctx, qp, kp, vp, wqp, wkp, eps, csp, max_pos, cp, lp, kcp, vcp, tp,
+                                                          max_blocks, S, n, Hq, Hkv, d, page, pages, st); }), ctx);
     Py_RETURN_NONE;
 }
 
@@ -296,8 +308,9 @@ PyObject* rmsnorm(Args a) {
     at::Tensor made;
     const at::Tensor& y = out_or(y_in, made, x.sizes(), x.scalar_type(), x);
     void *xp = bf(x), *rp = bf(res), *wp = bf(w), *yp = bf(y), *st = stream();
+    const int64_t T = x.size(0);
     const int H = dim(x, 1);
-    check(unlocked([&] { return tik_rmsnorm(ctx, xp, rp, wp, yp, eps, x.size(0), H, st); }), ctx);
+    check(unlocked([&] { return tik_rmsnorm(ctx, xp, rp, wp, yp, eps, T, H, st); }), ctx);
     return wrap(y_in, made);
 }
 
@@ -307,10 +320,11 @@ PyObject* swiglu(Args a) {
     const at::Tensor* out_in = a.opt();
     want_rank(gu, 2);
     at::Tensor made;
+    const int64_t T = gu.size(0);
     const int inter = dim(gu, 1) / 2;
-    const at::Tensor& out = out_or(out_in, made, {gu.size(0), inter}, at::kBFloat16, gu);
+    const at::Tensor& out = out_or(out_in, made, {T, inter}, at::kBFloat16, gu);
     void *gp = bf(gu), *op = bf(out), *st = stream();
-    check(unlocked([&] { return tik_swiglu(ctx, gp, op, gu.size(0), inter, st); }), ctx);
+    check(unlocked([&] { return tik_swiglu(ctx, gp, op, T, inter, st); }), ctx);
     return wrap(out_in, made);
 }
 
@@ -319,12 +333,13 @@ PyObject* linear(Args a) {
     const at::Tensor &x = a.tensor(), &w = a.tensor();
     const at::Tensor* y_in = a.opt();
     want_rank(x, 2);
-    if (w.dim() < 1) want_rank(w, 2);
+    want_axis(w, 0);
     at::Tensor made;
+    const int64_t T = x.size(0);
     const int K = dim(x, 1), N = dim(w, 0);
-    const at::Tensor& y = out_or(y_in, made, {x.size(0), N}, at::kBFloat16, x);
+    const at::Tensor& y = out_or(y_in, made, {T, N}, at::kBFloat16, x);
     void *xp = bf(x), *wp = bf(w), *yp = bf(y), *st = stream();
-    check(unlocked([&] { return tik_linear(ctx, xp, wp, yp, x.size(0), K, N, st); }), ctx);
+    check(unlocked([&] { return tik_linear(ctx, xp, wp, yp, T, K, N, st); }), ctx);
     return wrap(y_in, made);
 }
 
@@ -341,12 +356,13 @@ PyObject* attn_prefill(Args a) {
     const Cache c = cache_of(kc, vc, table);
     at::Tensor made;
     const at::Tensor& o = out_or(o_in, made, q.sizes(), q.scalar_type(), q);
+    const int64_t tot = q.size(0);
     const int S = static_cast<int>(lens.numel()), Hq = dim(q, 1), d = dim(q, 2);
     const Scratch ws = plan_ws(ws_in, TIK_OP_ATTN_PREFILL, S, max_ctx, q);
     void *qp = bf(q), *op = bf(o), *st = stream();
     float* lp = f32(lse);
     int32_t *cp = i32(cu), *np = i32(lens);
-    check(unlocked([&] { return tik_attn_prefill(ctx, qp, op, lp, cp, np, c.k, c.v, c.table, c.max_blocks, S, q.size(0), max_q,
+    check(unlocked([&] { return tik_attn_prefill(ctx, qp, op, lp, cp, np, c.k, c.v, c.table, c.max_blocks, S, tot, max_q,
                                                  max_ctx, Hq, c.Hkv, d, c.page, c.num_pages, scale, ws.p, ws.bytes, st); }), ctx);
     return wrap(o_in, made);
 }
@@ -364,13 +380,14 @@ PyObject* attn_prefill_kv(Args a) {
     const Cache c = cache_of(kc, vc, table);
     at::Tensor made;
     const at::Tensor& o = out_or(o_in, made, q.sizes(), q.scalar_type(), q);
+    const int64_t tot = q.size(0);
     const int S = static_cast<int>(lens.numel()), Hq = dim(q, 1), d = dim(q, 2);
     const Scratch ws = plan_ws(ws_in, TIK_OP_ATTN_PREFILL, S, max_ctx, q);
     void *qp = bf(q), *kp = bf(k), *vp = bf(v), *op = bf(o), *st = stream();
     float* lp = f32(lse);
     int32_t *cp = i32(cu), *np = i32(lens);
     check(unlocked([&] { return tik_attn_prefill_kv(ctx, qp, kp, vp, op, lp, cp, np, c.k, c.v, c.table, c.max_blocks, S,
-                                                    q.size(0), max_q, max_ctx, Hq, c.Hkv, d, c.page, c.num_pages, scale, ws.p,
+                                                    tot, max_q, max_ctx, Hq, c.Hkv, d, c.page, c.num_pages, scale, ws.p,
                                                     ws.bytes, st); }), ctx);
     return wrap(o_in, made);
 }
@@ -418,7 +435,7 @@ PyObject* token_logprob(Args a) {
     const float inv_temperature = a.real();
     const at::Tensor *ws_in = a.opt(), *lp_in = a.opt(), *lse = a.opt();
     want_rank(x, 2);
-    if (w.dim() < 1) want_rank(w, 2);
+    want_axis(w, 0);
     const int64_t T = x.size(0);
     const int H = dim(x, 1), V = dim(w, 0);
     const Scratch ws = sized_ws(ws_in, tik_workspace_bytes(TIK_OP_TOKEN_LOGPROB, T, 0, 0, 0, 0, H, V), x);

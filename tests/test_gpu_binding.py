@@ -48,6 +48,25 @@ def test_refused_arguments(tik):
         tik.tik_linear(3, w)
 
 
+def test_tensors_without_the_axis_that_is_read_are_refused(tik):
+    """A size is read, and refused, before the interpreter lock is dropped for the call: an exception behind that
+    point would end the process instead of raising."""
+    i32 = lambda *v: torch.tensor(v, dtype=torch.int32, device="cuda")
+    q, k, scalar = (torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((2, 4, 64), (2, 1, 64), ()))
+    cache, table = torch.zeros(2, 1, 16, 64, dtype=torch.bfloat16, device="cuda"), i32(0, 1).view(2, 1)
+    rope, weight = torch.zeros(8, 64, device="cuda"), torch.ones(64, dtype=torch.bfloat16, device="cuda")
+    for bad in (lambda: tik.tik_kv_cache_write(scalar, scalar, i32(0, 1), i32(1), cache, cache, table),
+                lambda: tik.tik_kv_cache_write(k, k, i32(0, 1, 2), i32(1, 1), cache, cache, i32(0, 1)),
+                lambda: tik.tik_qk_norm_rope_kv_write(q, k, k, weight, weight, 1e-6, rope[0, 0].clone(), i32(0, 1, 2)),
+                lambda: tik.tik_qk_norm_rope_kv_write(q, scalar, k, weight, weight, 1e-6, rope, i32(0, 1, 2)),
+                lambda: tik.tik_qk_norm_rope_kv_write(q, k, k, weight, weight, 1e-6, rope, i32(0, 1, 2), i32(1, 1), scalar,
+                                                      cache, table),
+                lambda: tik.tik_linear(q[0], scalar), lambda: tik.tik_attn_train_fwd(q, scalar, scalar, i32(0, 2), 2, 0.1)):
+        with pytest.raises(IndexError):
+            bad()
+    assert bool((cache == 0).all())
+
+
 def test_threads_with_streams_of_their_own(tik):
     w = _x(640, 512, 5, 0.05)
     xs = [_x(40 + i, 512, 6 + i) for i in range(4)]
