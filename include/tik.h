@@ -72,6 +72,10 @@ const char* tik_contract_id(void);
  * kernels that use more than 48 KiB of shared memory are opted in once per (kernel, device), and
  * this exercises that table with stand-in ordinals.  Needs no GPU.  Returns 0 when it holds. */
 int tik_selftest_host(void);
+/* Host-only view of a dispatch rule for tests (no paper counterpart; needs no GPU): CTAs per chunk of a
+ * decode call of so many (sequence, KV head, chunk) items on a device that holds max_clusters clusters
+ * of the cluster kernel at one time, 0 when another kernel takes the call. */
+int tik_selftest_decode_cluster(int64_t chunks, int max_ctx, int G, int d, int max_clusters);
 
 /* Number of kernels the library has launched in this process so far (all contexts, all streams;
  * every launch site counts itself when it enqueues a kernel).  No paper counterpart: it lets a

@@ -87,15 +87,15 @@ static bool use_persistent(const void* ws, size_t ws_bytes, int S, int max_posit
 }
 
 // CTAs per chunk for decode calls that leave most SMs idle (tik_decode_cluster.cu), 0: the other kernels.
-// chunks: (sequence, KV head, chunk) items by the host's bound.  A cluster pays while all of them run at
-// once (5 x 8 chunks in clusters of four, a second wave: 16.8 -> 25 us) and the contexts are longer than
-// its set-up (1000 keys 10.4 -> 9.1 us, 500 7.6 -> 7.3, 128 5.3 -> 6.5).  Two CTAs per chunk stop at a third of
-// the SMs' number of chunks: beyond it a call whose keys are not in L2 is bound by HBM and gains nothing
-// (16 x 2000 x 4 keys, cold: 22.6 -> 24.6 us, in L2: 16.7 -> 14.9).
-static int decode_cluster_size(long long chunks, int max_ctx, int G, int d, int sm_count) {
-    if (G > DECODE2_MAX_G || max_ctx <= 512) return 0;
-    if (d == 128 && 4 * chunks <= sm_count) return 4;
-    return 3 * chunks <= sm_count ? 2 : 0;
+// chunks: (sequence, KV head, chunk) items by the host's bound.  Clusters of four pay while all of them run at
+// once.  How many do is up to the device: a cluster sits inside a GPC, so 148 SMs hold 33 of them, not 37, at one
+// CTA per SM (max_clusters, from the occupancy calculator), and a second wave costs more than the kernel saves: 33 x
+// 2000 keys in one wave 15.9 us against 16.7 without clusters, 34 in two 27.4 against 16.4.  Contexts have to be
+// longer than the set-up: without -> with clusters, 4 .. 33 chunks, keys out of HBM: 2000 keys 15.3 .. 16.7 ->
+// 13.6 .. 15.9 us, 1500 12.7 .. 13.8 -> 11.9 .. 13.7, 1000 9.5 .. 10.8 -> 9.7 .. 11.1, 520 7.7 .. 8.4 -> 8.3 .. 9.5.
+// (Clusters of two gained nothing at any size: d 128, 48 x 2000 keys 1.04 times the time without, d 64 1.0 .. 1.2.)
+static int decode_cluster_size(long long chunks, int max_ctx, int G, int d, int max_clusters) {
+    return d == 128 && G <= DECODE2_MAX_G && max_ctx > 1024 && chunks <= max_clusters ? DECODE_CLUSTER : 0;
 }
 
 static tik_status check_heads(tik_ctx* ctx, int Hq, int Hkv, int d, float scale) {
@@ -135,6 +135,10 @@ tik_status tik_create(tik_ctx** out, int device) {
     }
     if (e == cudaSuccess) e = cudaMalloc(&ctx->dev_status, 256);
     if (e == cudaSuccess) e = cudaMemset(ctx->dev_status, 0, 256);
+    if (e == cudaSuccess && decode_cluster_max_active(&ctx->max_clusters) != cudaSuccess) {
+        ctx->max_clusters = 0;         // the other decode kernels take every call
+        cudaGetLastError();
+    }
     if (e == cudaSuccess) {
         cudaDriverEntryPointQueryResult qres;
         e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ctx->encode_tiled, cudaEnableDefault, &qres);
@@ -186,6 +190,9 @@ int tik_selftest_host(void) {
     if (once.run(ok_step, DeviceOnce::MAX_DEVICES + 5) != cudaSuccess || runs != 4) return 7;
     if (once.run(ok_step, DeviceOnce::MAX_DEVICES + 5) != cudaSuccess || runs != 5) return 8;
     return 0;
+}
+int tik_selftest_decode_cluster(int64_t chunks, int max_ctx, int G, int d, int max_clusters) {
+    return decode_cluster_size(chunks, max_ctx, G, d, max_clusters);
 }
 const char* tik_contract_id(void) { return TIK_CONTRACT_ID; }
 
@@ -430,7 +437,7 @@ tik_status tik_attn_decode(tik_ctx* ctx, const void* q, void* o, float* lse, con
     if (!make_tmap_bf16(ctx, &tmQ, q, 3, qd, qs, box, &err)) return fail(ctx, TIK_ERR_CUDA, err.c_str());
     const int nchunk = (max_ctx_len + CHUNK - 1) / CHUNK;
     const long long pairs = static_cast<long long>(B) * Hkv;
-    const int cluster = decode_cluster_size(pairs * nchunk, max_ctx_len, G, d, ctx->sm_count);
+    const int cluster = decode_cluster_size(pairs * nchunk, max_ctx_len, G, d, ctx->max_clusters);
     s = make_cache_maps(ctx, k_cache, v_cache, Hkv, d, page_size, num_pages, &tmK, &tmV, cluster ? d / cluster : 64);
     if (s != TIK_OK) return s;
 
@@ -473,7 +480,7 @@ tik_status tik_attn_decode(tik_ctx* ctx, const void* q, void* o, float* lse, con
     dim3 grid((nchunk + p.cpc - 1) / p.cpc, Hkv, B);
     if (grid.y > 65535 || grid.z > 65535) return fail(ctx, TIK_ERR_UNSUPPORTED, "Hkv and B must be <= 65535");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cluster ? launch_decode_cluster(d, cluster, nchunk, Hkv, B, tmQ, tmK, tmV, p, st)
+    cudaError_t e = cluster ? launch_decode_cluster(nchunk, Hkv, B, tmQ, tmK, tmV, p, st)
                     : small_group ? launch_decode2(d, grid, tmQ, tmK, tmV, p, st) : launch_attn(d, 2, grid, tmQ, tmK, tmV, p, st);
     if (e == cudaSuccess && !p.direct_out) e = launch_combine(d, p, B, st);
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_decode");

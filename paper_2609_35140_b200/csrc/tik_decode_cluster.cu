@@ -2,7 +2,7 @@
 //
 // With few (sequence, KV head, chunk) items the other decode kernels take as long as one CTA needs for
 // one chunk: 64 KiB of keys and values per 128-key tile through one SM (~0.8 us per tile, ~14 us for a
-// chunk) whatever the memory system could deliver.  Here C = 2 or 4 CTAs share a chunk.  What may be
+// chunk) whatever the memory system could deliver.  Here C = 4 CTAs share a chunk.  What may be
 // split without touching the contract: score columns (a key's scores are one MMA chain of their own)
 // and output columns (a column of O is one chain over the keys of its own).  What may not: the chain of an
 // output element over the chunk's tiles, and the order of the row sums.  So, tile by tile and pipelined:
@@ -17,10 +17,9 @@
 // Every chunk leaves its partial for combine_kernel, or its rows when it is the only one.
 // Same tiles, same MMA chains over d and keys, same row-sum shape, same rescales, so same bits as
 // every other regime.  Query rows and weights are 8-row atoms read with a zero stride between row
-// groups (see tik_decode.cu); M64 MMAs suffice for G <= 8 rows.
-// Measured in a CUDA graph of back-to-back calls (one CTA per chunk -> this): one sequence of 2000 keys, 4 KV
-// heads x 7 16.5 -> 12.1 us, 4321 keys 17.8 -> 13.6, 4 x 2000 keys x 8 KV heads 16.9 -> 13.3 (C = 4);
-// 5 x 2000 x 8 16.8 -> 15.0 (C = 2).
+// groups (see tik_decode.cu); M64 MMAs suffice for G <= 8 rows.  Head size 128 only.
+// Measured in a CUDA graph of back-to-back calls, keys out of HBM (one CTA per chunk -> this): one sequence, 4 KV
+// heads x 7, 2000 keys 15.3 -> 13.4 us, 4321 16.9 -> 15.0, 16000 19.1 -> 17.7.
 #include "tik_core.cuh"
 #include "tik_internal.h"
 #include "tik_ptx.cuh"
@@ -30,11 +29,13 @@ namespace tik {
 // warps 0-7 softmax, 8-11 transfer, 12 TMA, 13 MMA
 constexpr int DX_THREADS = 32 * 14;
 
-template <int D>
+constexpr int DX_D = 128;                                       // head size
+
 struct DXSmem {
+    static constexpr int D = DX_D;
     static constexpr uint32_t ATOM = 128 * 128;                  // 128 keys x 64 bf16
-    static constexpr uint32_t UNIT = (D / 64) * ATOM;            // one K tile, or C tiles' V columns of this CTA
-    static constexpr uint32_t NU = (D == 128) ? 4 : 8;           // ring units (128 KiB)
+    static constexpr uint32_t UNIT = (D / 64) * ATOM;            // one K tile, or four tiles' V columns of this CTA
+    static constexpr uint32_t NU = 4;                              // ring units (128 KiB)
     static constexpr uint32_t OFF_RING = 0;
     static constexpr uint32_t OFF_Q = NU * UNIT;                 // D / 64 atoms of 8 rows x 128 bytes
     // scores of a tile: 8 rows of 128 fp32, the row pitch 16 bytes longer so that eight rows' 16-byte
@@ -83,7 +84,7 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // A chain over 128 contraction steps of 16: A = compact 8-row atoms (64 descriptor units per 64
-// columns).  QK: B atoms 16 KiB apart; PV: B rows of 128 (VC = 64) or 64 bytes (VC = 32).
+// columns).  QK: B atoms 16 KiB apart; PV: B rows of 64 bytes.
 __device__ __forceinline__ void mma_ss_chain8_compact_k(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
     asm volatile(
         "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
@@ -93,18 +94,6 @@ __device__ __forceinline__ void mma_ss_chain8_compact_k(uint32_t d_tmem, uint64_
         TIK_MMA_SS_STEP(64, 1024) TIK_MMA_SS_STEP(66, 1026) TIK_MMA_SS_STEP(68, 1028)
         TIK_MMA_SS_STEP(70, 1030)
         "}" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_ss_chain8_compact_v64(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                          uint32_t first_accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
-        TIK_MMA_SS_STEP(2, 128) TIK_MMA_SS_STEP(4, 256) TIK_MMA_SS_STEP(6, 384)
-        TIK_MMA_SS_STEP(64, 512) TIK_MMA_SS_STEP(66, 640) TIK_MMA_SS_STEP(68, 768)
-        TIK_MMA_SS_STEP(70, 896)
-        "}" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(first_accumulate)
         : "memory");
 }
 __device__ __forceinline__ void mma_ss_chain8_compact_v32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -130,13 +119,13 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr, uint32_t lbo,
     return d;
 }
 
-template <int D, int C>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AttnParams p) {
-    using L = DXSmem<D>;
+    using L = DXSmem;
+    constexpr int D = DX_D, C = DECODE_CLUSTER;
     constexpr int NATOM = D / 64;
-    constexpr int VC = D / C;                                  // output columns of this CTA: 64 or 32
+    constexpr int VC = D / C;                                  // output columns of this CTA
     constexpr uint32_t VBYTES = 128 * VC * 2;                  // one tile's V columns: a C-th of a unit
     constexpr int NU = static_cast<int>(L::NU);
     constexpr uint32_t TMEM_COLS = 512;
@@ -144,7 +133,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     constexpr uint32_t COL_O = 384;
     constexpr uint32_t IDESC_QK = mma_idesc_bf16(64, 128, false);
     constexpr uint32_t IDESC_PV = mma_idesc_bf16(64, VC, true);
-    static_assert(VC == 64 || VC == 32, "V columns per CTA");
+    static_assert(VC == 32, "rows of 64 bytes: mma_ss_chain8_compact_v32, the 64-byte swizzle of tmV");
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -293,8 +282,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (i >= NSB) mbar_wait_warp(bar_sfree + 8 * b, (i / NSB - 1) & 1, abort_word, p.dev_status);
             tc_fence_after();
             const uint64_t dk = smem_desc_sw128(sRing + u * L::UNIT, 0, 1024);
-            if (D == 128) mma_ss_chain8_compact_k(tmem + 128 * b, dq, dk, IDESC_QK);
-            else mma_ss_chain4_fresh(tmem + 128 * b, dq, dk, IDESC_QK);
+            mma_ss_chain8_compact_k(tmem + 128 * b, dq, dk, IDESC_QK);
             mma_commit(bar_sfull + 8 * b);
             mma_commit(bar_empty + 8 * u);
         }
@@ -314,8 +302,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             tc_fence_after();
             const uint64_t dp = smem_desc_sw128(sS + t * L::S_TILE, 0, 0);
             const uint32_t v = sRing + u * L::UNIT + (t % C) * VBYTES;
-            if (VC == 64) mma_ss_chain8_compact_v64(tmem + COL_O, dp, smem_desc_sw128(v, L::ATOM, 1024), IDESC_PV, t > 0 ? 1u : 0u);
-            else mma_ss_chain8_compact_v32(tmem + COL_O, dp, smem_desc_sw64(v, 8192, 512), IDESC_PV, t > 0 ? 1u : 0u);
+            mma_ss_chain8_compact_v32(tmem + COL_O, dp, smem_desc_sw64(v, 8192, 512), IDESC_PV, t > 0 ? 1u : 0u);
             if (t % C == C - 1 || t == n_tiles - 1) mma_commit(bar_empty + 8 * u);
         }
         mma_commit(bar_pv);
@@ -519,24 +506,37 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     if (warp == 13) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <int D, int C>
-static cudaError_t launch_decode_cluster_t(int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                                           const CUtensorMap& tmV, const AttnParams& p, cudaStream_t stream) {
-    auto kern = decode_cluster_kernel<D, C>;
+static cudaError_t configure() {
     static DeviceOnce configured;     // the shared-memory opt-in belongs to the (function, device) pair
-    cudaError_t e = configured.run([&]() {
-        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(DXSmem<D>::BYTES));
+    return configured.run([&]() {
+        return cudaFuncSetAttribute(decode_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(DXSmem::BYTES));
     });
-    if (e != cudaSuccess) return e;
-    return launch_pdl(kern, dim3(static_cast<unsigned>(nchunk) * C, static_cast<unsigned>(Hkv), static_cast<unsigned>(B)), DX_THREADS,
-                      DXSmem<D>::BYTES, stream, C, tmQ, tmK, tmV, p);
 }
 
-cudaError_t launch_decode_cluster(int d, int C, int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
+cudaError_t decode_cluster_max_active(int* clusters) {
+    const cudaError_t e = configure();
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = DECODE_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(DECODE_CLUSTER);
+    cfg.blockDim = dim3(DX_THREADS);
+    cfg.dynamicSmemBytes = DXSmem::BYTES;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(clusters, decode_cluster_kernel, &cfg);
+}
+
+cudaError_t launch_decode_cluster(int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                                   const CUtensorMap& tmV, const AttnParams& p, cudaStream_t stream) {
-    if (d == 64) return launch_decode_cluster_t<64, 2>(nchunk, Hkv, B, tmQ, tmK, tmV, p, stream);
-    return C == 4 ? launch_decode_cluster_t<128, 4>(nchunk, Hkv, B, tmQ, tmK, tmV, p, stream)
-                  : launch_decode_cluster_t<128, 2>(nchunk, Hkv, B, tmQ, tmK, tmV, p, stream);
+    const cudaError_t e = configure();
+    if (e != cudaSuccess) return e;
+    return launch_pdl(decode_cluster_kernel, dim3(static_cast<unsigned>(nchunk) * DECODE_CLUSTER, static_cast<unsigned>(Hkv), static_cast<unsigned>(B)),
+                      DX_THREADS, DXSmem::BYTES, stream, DECODE_CLUSTER, tmQ, tmK, tmV, p);
 }
 
 }  // namespace tik

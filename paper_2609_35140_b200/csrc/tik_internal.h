@@ -11,6 +11,7 @@
 struct tik_ctx {
     int device = 0;
     int sm_count = 0;
+    int max_clusters = 0;               // clusters of the cluster decode kernel that run at one time
     int* dev_status = nullptr;          // one int of device flags (TIK_DEV_*)
     void* encode_tiled = nullptr;       // cuTensorMapEncodeTiled from the driver
     std::string last_error;
@@ -119,9 +120,11 @@ constexpr int DECODE2_MAX_G = 8;
 cudaError_t launch_decode2(int d, dim3 grid, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                            const AttnParams& p, cudaStream_t stream);
 
-// Decode of small calls (tik_decode_cluster.cu): clusters of C = 2 or 4 CTAs (d = 64: 2) per chunk.  tmV has a
-// box of d / C columns, with the 64-byte swizzle when that is 32.  Same scratch layout and output bits.
-cudaError_t launch_decode_cluster(int d, int C, int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
+// Decode of small calls (tik_decode_cluster.cu), d = 128: clusters of four CTAs per chunk.  tmV has a box of
+// 32 columns, with the 64-byte swizzle.  Same scratch layout and output bits.
+constexpr int DECODE_CLUSTER = 4;
+cudaError_t decode_cluster_max_active(int* clusters);     // of the current device; launches nothing
+cudaError_t launch_decode_cluster(int nchunk, int Hkv, int B, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                                   const CUtensorMap& tmV, const AttnParams& p, cudaStream_t stream);
 
 // Persistent full-sequence attention (tik_attn_persist.cu): a planning kernel writes the list of

@@ -1,5 +1,5 @@
-"""Decode calls that leave most SMs idle run as clusters of two or four CTAs per 2048-key chunk
-(tik_decode_cluster.cu).  Rows and log-sum-exps equal those of the packed train-forward bit for bit: group
+"""Decode calls that leave most SMs idle run as clusters of four CTAs per 2048-key chunk where the head size is 128
+and contexts are long (tik_decode_cluster.cu).  Rows and log-sum-exps equal those of the packed train-forward bit for bit: group
 sizes, head sizes, page sizes, tile counts from one to sixteen (fewer tiles than CTAs among them), chunk
 boundaries, and keys that grow along the sequence, so that the reference maximum moves and O is rescaled."""
 import numpy as np
@@ -22,9 +22,9 @@ def tik():
 
 @pytest.mark.parametrize("lens,Hkv,G,d,page,ramp", [
     ([1], 1, 1, 128, 64, 0.0), ([128, 129], 1, 8, 128, 16, 0.0), ([300, 511, 640], 2, 7, 128, 64, 0.0),
-    ([2048], 4, 7, 128, 64, 3.0), ([2047, 1500, 77], 8, 8, 128, 128, 3.0),              # four CTAs per chunk
+    ([2048], 4, 7, 128, 64, 3.0), ([2047, 1500, 77], 8, 8, 128, 128, 3.0),
     ([4321], 4, 7, 128, 64, 1.0), ([2049, 4096, 4097], 4, 4, 128, 32, 2.0),             # several chunks: partials
-    ([1000] * 12, 5, 3, 128, 16, 3.0), ([2000, 30, 129, 257, 2048] * 3, 4, 8, 128, 64, 2.0),   # two CTAs per chunk
+    ([1000] * 12, 5, 3, 128, 16, 3.0), ([2000, 30, 129, 257, 2048] * 3, 4, 8, 128, 64, 2.0),
     ([160], 1, 4, 64, 16, 0.0), ([2048, 100, 900], 8, 8, 64, 64, 3.0), ([5000, 3000], 6, 5, 64, 128, 2.0)])
 def test_cluster_decode_equals_train_rows(tik, lens, Hkv, G, d, page, ramp):
     S = len(lens)
@@ -72,4 +72,21 @@ def test_decode_at_the_edges_of_the_kernel_choice(tik, S, Hkv, G, lo, hi):
     ctx = torch.tensor(lens, dtype=torch.int32, device="cuda")
     rows = torch.tensor([int(w.cu_seqlens()[s]) + L - 1 for s, L in enumerate(lens)], device="cuda")
     o = tik.tik_attn_decode(q[rows].contiguous(), ctx, kc, vc, torch.from_numpy(layout.block_table).cuda(), hi, w.softmax_scale)
+    assert count_diff(o, o_train[rows]) == 0
+
+
+@pytest.mark.parametrize("chunks,Hkv,G,page", [(32, 4, 7, 64), (33, 3, 8, 16), (34, 2, 4, 64), (37, 1, 8, 32), (38, 2, 1, 128)])
+def test_cluster_decode_up_to_the_clusters_that_fit(tik, chunks, Hkv, G, page):
+    """Calls of as many chunks as clusters fit on the device, of a few more and a few less, most contexts a tile or
+    two long under a bound of one chunk: the rows equal those of the packed train-forward."""
+    S = -(-chunks // Hkv)
+    lens = ([2048] + 8 * [1, 127, 128, 129, 300, 511, 640, 1025])[:S]
+    w = synth.custom_workload([1] * S, [L - 1 for L in lens], G * Hkv, Hkv, 128, page, index=72)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    o_train = tik.tik_attn_train_fwd(q, k, v, cu, 2048, w.softmax_scale)
+    layout = synth.make_paged_layout(w)
+    kc, vc = synth.fill_paged_cache(w, layout, k, v)
+    ctx = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    rows = torch.tensor([int(w.cu_seqlens()[s]) + L - 1 for s, L in enumerate(lens)], device="cuda")
+    o = tik.tik_attn_decode(q[rows].contiguous(), ctx, kc, vc, torch.from_numpy(layout.block_table).cuda(), 2048, w.softmax_scale)
     assert count_diff(o, o_train[rows]) == 0
