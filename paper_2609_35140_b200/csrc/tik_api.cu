@@ -92,10 +92,11 @@ static bool use_persistent(const void* ws, size_t ws_bytes, int S, int max_posit
 // CTA per SM (max_clusters, from the occupancy calculator), and a second wave costs more than the kernel saves: 33 x
 // 2000 keys in one wave 15.9 us against 16.7 without clusters, 34 in two 27.4 against 16.4.  Contexts have to be
 // longer than the set-up: without -> with clusters, 4 .. 33 chunks, keys out of HBM: 2000 keys 15.3 .. 16.7 ->
-// 13.6 .. 15.9 us, 1500 12.7 .. 13.8 -> 11.9 .. 13.7, 1000 9.5 .. 10.8 -> 9.7 .. 11.1, 520 7.7 .. 8.4 -> 8.3 .. 9.5.
+// 13.6 .. 15.9 us, 1500 12.7 .. 13.8 -> 11.9 .. 13.7, 1000 9.6 .. 10.8 -> 9.7 .. 11.1 (groups of eight; of four:
+// 9.6 .. 10.7 -> 9.2 .. 10.3), 700 8.1 .. 9.2 -> 8.7 .. 10.1 (of four: 8.2 .. 9.1 -> 8.3 .. 9.3).
 // (Clusters of two gained nothing at any size: d 128, 48 x 2000 keys 1.04 times the time without, d 64 1.0 .. 1.2.)
 static int decode_cluster_size(long long chunks, int max_ctx, int G, int d, int max_clusters) {
-    return d == 128 && G <= DECODE2_MAX_G && max_ctx > 1024 && chunks <= max_clusters ? DECODE_CLUSTER : 0;
+    return d == 128 && G <= DECODE2_MAX_G && max_ctx > 896 && chunks <= max_clusters ? DECODE_CLUSTER : 0;
 }
 
 static tik_status check_heads(tik_ctx* ctx, int Hq, int Hkv, int d, float scale) {

@@ -19,5 +19,5 @@ def test_clusters_only_while_all_of_them_run_at_once(lib, max_clusters):
     for chunks in range(1, 60):
         got = lib.tik_selftest_decode_cluster(chunks, 4000, 8, 128, max_clusters)
         assert got == (4 if chunks <= max_clusters else 0), chunks
-    for refused in ((4, 1024, 8, 128), (4, 4000, 9, 128), (4, 4000, 8, 64)):
+    for refused in ((4, 896, 8, 128), (4, 4000, 9, 128), (4, 4000, 8, 64)):
         assert lib.tik_selftest_decode_cluster(*refused, max_clusters) == 0
