@@ -192,6 +192,25 @@ int tik_selftest_host(void) {
     if (once.run(ok_step, DeviceOnce::MAX_DEVICES + 5) != cudaSuccess || runs != 5) return 8;
     return 0;
 }
+int tik_selftest_linear(int64_t T, int K, int N, int sm_count, int* ctas, int* cols) {
+    LinearParams p{};
+    p.T = T;
+    p.K = K;
+    p.N = N;
+    p.sm_count = sm_count;
+    if (linear_narrow_choose(p)) {
+        *ctas = p.nunit;
+        *cols = p.nu;
+        return TIK_LINEAR_NARROW;
+    }
+    const long long ntile = (T + 127) / 128;
+    const LinearChoice c = linear_wide_choose(p);
+    const long long units = static_cast<long long>((N + c.nu - 1) / c.nu) * (c.pair ? (ntile + 1) / 2 : ntile);
+    const long long slots = c.pair ? sm_count / 2 : sm_count;
+    *ctas = c.units ? static_cast<int>((units < slots ? units : slots) * (c.pair ? 2 : 1)) : 0;
+    *cols = c.nu;
+    return !c.units ? TIK_LINEAR_BAND : c.pair ? TIK_LINEAR_PAIR_UNITS : TIK_LINEAR_UNITS;
+}
 int tik_selftest_decode_cluster(int64_t chunks, int max_ctx, int G, int d, int max_clusters) {
     return decode_cluster_size(chunks, max_ctx, G, d, max_clusters);
 }
@@ -679,9 +698,9 @@ tik_status tik_linear(tik_ctx* ctx, const void* x, const void* weight, void* y, 
     // More than 16 row tiles: CTA pairs in a band raster (x no longer fits L2).  Up to 16: persistent CTAs or
     // pairs over (column step, row tiles) units -- a grid of one CTA per unit spends as long on set-up as on a
     // unit's 56 .. 432 K slices.  Same MMA chain per output element, so the same bits.
-    const bool units = ntile <= 16;
-    const int a_rows = T <= 32 ? 32 : T <= 64 ? 64 : 128;
-    const LinearChoice c = units ? linear_choose(T, K, N, a_rows, ctx->sm_count) : LinearChoice{true, 256};
+    const LinearChoice c = linear_wide_choose(p);
+    const bool units = c.units;
+    const int a_rows = linear_staged_rows(T);
     uint32_t boxA[2] = {64, static_cast<uint32_t>(c.pair ? 128 : a_rows)};
     uint32_t boxB[2] = {64, static_cast<uint32_t>(c.pair ? 128 : c.nu)};
     CUtensorMap tmY;

@@ -230,10 +230,12 @@ struct LinearParams {
 struct LinearChoice {
     bool pair;
     int nu;
+    bool units;                  // persistent over units, else the band raster (pairs)
 };
+inline int linear_staged_rows(long long T) { return T <= 32 ? 32 : T <= 64 ? 64 : 128; }
 inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_count) {
     const long long ntile = (T + 127) / 128;
-    LinearChoice best = {false, 256};
+    LinearChoice best = {false, 256, true};
     double best_us = -1.0;
     auto consider = [&](bool pair, int nu) {
         const long long slots = pair ? sm_count / 2 : sm_count;
@@ -243,28 +245,40 @@ inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_
         const double us = rounds * (K / 64) * slice_ns * 1e-3 + (pair ? 2.0 : 0.0);
         if (best_us < 0.0 || us < best_us * 0.98) {
             best_us = us;
-            best = {pair, nu};
+            best = {pair, nu, true};
         }
     };
     if (ntile > 1) consider(true, 256);
     for (int nu = 256; nu >= 64; nu /= 2) consider(false, nu);
     return best;
 }
-// The narrow schedule: one unit of nu weight rows x one row tile per CTA, nu as few as spread the call over the
-// SMs (whole 8-row swizzle atoms; an MMA of 128 rows takes N = 16 i).  Its time is the MMAs' shared-memory reads,
+// The kernel of a call that the narrow schedule does not take.  More than 16 row tiles: the band raster (x no longer
+// fits L2).
+inline LinearChoice linear_wide_choose(const LinearParams& p) {
+    if (p.T > 16 * 128) return {true, 256, false};
+    return linear_choose(p.T, p.K, p.N, linear_staged_rows(p.T), p.sm_count);
+}
+// The narrow schedule: one unit of nu weight rows x one row tile per CTA, nu as few as need no more CTAs than SMs
+// (whole 8-row swizzle atoms; an MMA of 128 rows takes N = 16 i), or one CTA per row tile when there are more of those.
+// A second wave repeats the whole chain over K: 768 rows x N 1184, K 8960, in 150 CTAs 49.7 us, by the unit kernel 26.4;
+// 8192 x 104, K 3584, in 192 CTAs 27.0, by pairs 20.8.  One CTA per row tile reads x once (K 3584, N 8, pairs -> this:
+// 20000 rows 45.6 -> 32.4, 100000 rows 156 -> 108).  In one wave, K 3584, pairs -> this: 2304 x 256 22.0 -> 12.1, 5000 x 128
+// 22.1 -> 13.4.  Its time is the MMAs' shared-memory reads,
 // 64 or 128 rows of the M operand + the N operand's, and what TMA writes there: the operand whose choice as M
 // reads fewer rows is M (x must be for more than 80 rows).  Above 48 weight rows and 80 x rows the unit
 // kernel is as fast or faster (K 18944, N 3584, 256 rows: 53.1 us, 54.5 here; K 1536, N 8960, 128 rows: 8.3, 8.5).
 inline bool linear_narrow_choose(LinearParams& p) {
     const long long ntile = (p.T + 127) / 128;
     const int rows = static_cast<int>(p.T < 128 ? p.T : 128), t16 = (rows + 15) / 16 * 16, m = rows > 64 ? 128 : 64;
+    const long long ctas = ntile < p.sm_count ? p.sm_count / ntile : 1;      // that a row tile may take
     auto weight_rows = [&](int atom) {
-        const long long per = static_cast<long long>(atom) * p.sm_count;
-        return atom * ((p.N * ntile + per - 1) / per);
+        const long long per = atom * ctas;
+        return atom * ((p.N + per - 1) / per);
     };
     const long long nw = weight_rows(8), nx = weight_rows(m == 128 ? 16 : 8);
     const bool x_is_m = t16 > 80 || (m == 128 ? m + nx <= 64 + t16 : nx < t16);
-    if ((x_is_m ? nx : nw) > (t16 > 80 ? 48 : 64)) return false;
+    const int most = t16 > 80 ? 48 : 64;
+    if ((x_is_m ? nx : nw) > most || p.N * ntile > static_cast<long long>(most) * p.sm_count) return false;
     p.m = x_is_m ? m : 0;
     p.nu = static_cast<int>(x_is_m ? nx : nw);
     p.a_rows = x_is_m ? (rows + 7) / 8 * 8 : t16;

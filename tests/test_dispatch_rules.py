@@ -9,8 +9,33 @@ def lib():
     from paper_2609_35140_b200 import binding
     lib = binding.load()
     lib.tik_selftest_decode_cluster.argtypes = [ctypes.c_int64] + 4 * [ctypes.c_int]
+    lib.tik_selftest_linear.argtypes = [ctypes.c_int64] + 3 * [ctypes.c_int] + 2 * [ctypes.POINTER(ctypes.c_int)]
     return lib
 
+
+NARROW, UNITS, PAIR_UNITS, BAND = range(4)
+
+
+def linear_schedule(lib, T, K, N, sms=148):
+    """(schedule, CTAs, columns per unit) of tik_linear."""
+    ctas, cols = ctypes.c_int(), ctypes.c_int()
+    return lib.tik_selftest_linear(T, K, N, sms, ctypes.byref(ctas), ctypes.byref(cols)), ctas.value, cols.value
+
+
+@pytest.mark.parametrize("sms", [148, 132])
+def test_narrow_linear_is_one_wave_or_one_cta_per_row_tile(lib, sms):
+    """A second wave of narrow CTAs repeats the whole chain over K: no shape gets one, except that row tiles beyond
+    the number of SMs take a CTA each, which then holds all columns.  No CTA has more columns than there are."""
+    taken = 0
+    for T in list(range(1, 140)) + [255, 256, 257, 384, 640, 768, 1024, 2048, 2049, 3456, 5000, 8192, 18944, 20000, 100000]:
+        for N in list(range(8, 1700, 8)) + list(range(4096, 9600, 64)):
+            schedule, ctas, cols = linear_schedule(lib, T, 1536, N, sms)
+            if schedule == NARROW:
+                taken += 1
+                tiles = -(-T // 128)
+                assert ctas == -(-N // cols) * tiles and (ctas <= sms or ctas == tiles), (T, N, ctas, cols)
+                assert cols < N + 16, (T, N, cols)
+    assert taken > 10000
 
 @pytest.mark.parametrize("max_clusters", [0, 1, 33, 37])
 def test_clusters_only_while_all_of_them_run_at_once(lib, max_clusters):
