@@ -220,7 +220,11 @@ struct LinearParams {
 // Schedule of a call of at most 16 row tiles, from a cost model: rounds of units x K slices x the time of one
 // 64-wide K slice, as measured on a B200 with W out of HBM.  A single CTA takes in x and W rows at ~130 GB/s
 // (128 rows: N = 64 190 ns, 128 235 ns, 256 370 ns); a pair's slice (256 x 256) is its MMAs, ~300 ns, and a
-// pair costs ~2 us more to set up and to drain.  Ties go to pairs and the wider unit (fewer bytes out of L2).
+// pair costs ~2 us more to set up and to drain.  Ties go to pairs and the wider unit (fewer bytes out of L2), but with
+// one row tile of more than 64 rows to the narrower one: such a call is one pass over W, and three rounds of 128
+// columns keep more SMs at it than two of 256 whose second is not full.  256 columns -> 128, us: 65 / 128 rows of K
+// 5120, N 55296 96.2 / 98.4 -> 91.6 / 94.6; K 3584, N 40960 63.9 / 65.6 -> 58.9 / 60.3; K 1536, N 46080 31.6 / 33.1 ->
+// 29.1 / 30.3.
 // Before, every call of 129 .. 2048 rows ran as pairs; us, pairs -> the choice, W out of HBM:
 //   K 8960,  N 1536:   129 rows 44.2 -> 29.8 (64 columns), 1024 rows 44.6 -> 34.3 (128), 2000 rows 47 (pairs)
 //   K 18944, N 3584:   129 rows 88.5 -> 61.0 (64), 512 rows 89.1 -> 73.6 (128), 741 rows 91.1 (pairs; 128: 140)
@@ -237,13 +241,14 @@ inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_
     const long long ntile = (T + 127) / 128;
     LinearChoice best = {false, 256, true};
     double best_us = -1.0;
+    const double tie = ntile == 1 && a_rows == 128 ? 1.02 : 0.98;
     auto consider = [&](bool pair, int nu) {
         const long long slots = pair ? sm_count / 2 : sm_count;
         const long long units = static_cast<long long>((N + nu - 1) / nu) * (pair ? (ntile + 1) / 2 : ntile);
         const long long rounds = (units + slots - 1) / slots;
         const double slice_ns = pair ? 300.0 : (a_rows + nu) * 128.0 / 130.0;
         const double us = rounds * (K / 64) * slice_ns * 1e-3 + (pair ? 2.0 : 0.0);
-        if (best_us < 0.0 || us < best_us * 0.98) {
+        if (best_us < 0.0 || us < best_us * tie) {
             best_us = us;
             best = {pair, nu, true};
         }

@@ -37,6 +37,14 @@ def test_narrow_linear_is_one_wave_or_one_cta_per_row_tile(lib, sms):
                 assert cols < N + 16, (T, N, cols)
     assert taken > 10000
 
+@pytest.mark.parametrize("N,cols", [(37888, 256), (37896, 128), (40960, 128), (55296, 128), (56832, 128), (56840, 256), (75776, 256)])
+def test_wide_linear_of_65_to_128_rows_keeps_the_sms_at_work(lib, N, cols):
+    """One pass over W: three rounds of 128 columns rather than two of 256 whose second is partly empty; 256 columns
+    where their last round is as full."""
+    for T in (65, 100, 128):
+        assert linear_schedule(lib, T, 5120, N)[::2] == (UNITS, cols)
+
+
 @pytest.mark.parametrize("max_clusters", [0, 1, 33, 37])
 def test_clusters_only_while_all_of_them_run_at_once(lib, max_clusters):
     """A cluster decode whose clusters do not all fit takes a second wave: 1.5 to 2 times the time of the kernels
