@@ -85,8 +85,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     // ---------------------------------------------------------------- work item
     const int seq = blockIdx.z;
-    const int tok0 = p.cu_seqlens[seq];
-    const int len = p.cu_seqlens[seq + 1] - tok0;
+    // (around L1 in the dQ grid, here and for lse and delta below: no wait of its own precedes the reads, and these
+    // buffers are rewritten from call to call)
+    const int tok0 = __ldcg(&p.cu_seqlens[seq]);
+    const int len = __ldcg(&p.cu_seqlens[seq + 1]) - tok0;
     if (len <= 0) {
         if (last_block) pdl_wait();
         return;
@@ -343,8 +345,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             dl = 0.0f;
             if (row_abs < len) {
                 const long long idx = (static_cast<long long>(tok0) + row_abs) * p.Hq + h;
-                l2 = __fmul_rn(p.lse[idx], LOG2E_F);
-                dl = __ldcg(&p.delta[idx]);     // (around L1: no wait of this grid's own precedes the read)
+                l2 = __fmul_rn(__ldcg(&p.lse[idx]), LOG2E_F);
+                dl = __ldcg(&p.delta[idx]);
             }
         };
         // DKV: the scalars belong to the columns (query rows of the streamed tile).  Threads 0..127 fetch

@@ -467,7 +467,8 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             const int lp = ((128 * j) >> p.page_shift) + lane;
                             int ph = p.num_pages;       // out of range: the box is filled with zeros
                             if ((lp << p.page_shift) < it.ctx) {
-                                ph = (lp < p.max_blocks) ? p.block_table[static_cast<long long>(it.seq) * p.max_blocks + lp] : -1;
+                                // (around L1, as the plan: behind the single-tile grid no wait precedes the read)
+                                ph = (lp < p.max_blocks) ? __ldcg(&p.block_table[static_cast<long long>(it.seq) * p.max_blocks + lp]) : -1;
                                 if (ph < 0 || ph >= p.num_pages) {
                                     if (kv == 0) atomicOr(p.dev_status, TIK_DEV_BAD_BLOCK);
                                     ph = p.num_pages;
