@@ -87,8 +87,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const int seq = blockIdx.z;
     // (around L1 in the dQ grid, here and for lse and delta below: no wait of its own precedes the reads, and these
     // buffers are rewritten from call to call)
-    const int tok0 = __ldcg(&p.cu_seqlens[seq]);
-    const int len = __ldcg(&p.cu_seqlens[seq + 1]) - tok0;
+    auto cu = [&](int i) { return MODE == BWD_DQ ? __ldcg(&p.cu_seqlens[i]) : p.cu_seqlens[i]; };
+    const int tok0 = cu(seq);
+    const int len = cu(seq + 1) - tok0;
     if (len <= 0) {
         if (last_block) pdl_wait();
         return;
