@@ -1046,10 +1046,8 @@ __global__ void __launch_bounds__(D) combine_kernel(const AttnParams p) {
 constexpr int KVW_THREADS = 256;
 template <int KVW_TOK>       // 8 for prompts, 1 for a decode step's handful of tokens (more blocks, shorter chains)
 __global__ void __launch_bounds__(KVW_THREADS)
-kv_write_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
-                const int32_t* __restrict__ cu_new, const int32_t* __restrict__ ctx_lens,
-                uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                const int32_t* __restrict__ block_table, int max_blocks, int S, long long total_new, int Hkv,
+kv_write_kernel(const uint4* k_new, const uint4* v_new, const int32_t* cu_new, const int32_t* ctx_lens,
+                uint4* k_cache, uint4* v_cache, const int32_t* block_table, int max_blocks, int S, long long total_new, int Hkv,
                 int vec_per_head /* d*2/16 */, int page_size, int num_pages, int* dev_status) {
     pdl_wait();
     pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid

@@ -545,9 +545,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // 28 heads x 128: 180 -> 118 us = 4.3 -> 6.5 TB/s, one vector per warp before).
 constexpr int DELTA_VPW = 8;
 template <int D>
-__global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* __restrict__ o,
-                                                       const __nv_bfloat16* __restrict__ dout,
-                                                       float* __restrict__ delta, long long n_vec) {
+__global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* dout,
+                                                       float* delta, long long n_vec) {
     pdl_wait();
     pdl_launch_dependents();
     const long long v0 = ((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * DELTA_VPW;

@@ -118,9 +118,8 @@ constexpr int PLAN_XMAX = 4096;
 // touched every sequence's K/V at once: a third slower on sixteen 16 K-token sequences), while
 // every CTA still meets every weight class, because the weights repeat sequence by sequence.
 // x_max: only candidates x <= x_max are listed (7: the paired items and partner-less tiles below 16).
-__global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* __restrict__ cu,
-                                                         const int32_t* __restrict__ ctx_lens, int S, int x_max,
-                                                         int4* __restrict__ plan) {
+__global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, const int32_t* ctx_lens, int S, int x_max,
+                                                         int4* plan) {
     pdl_wait();
     pdl_launch_dependents();
     __shared__ int warp_sums[32];
@@ -315,7 +314,7 @@ template <int D, bool PAGED>
 __global__ void __launch_bounds__(PA_THREADS, 1)
 attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AttnParams p,
-                    const int4* __restrict__ plan) {
+                    const int4* plan) {
     using L = PASmem<D>;
     constexpr int NATOM = D / 64;
     constexpr int DH = D / 2;

@@ -89,9 +89,10 @@ __global__ void __launch_bounds__(HN_THREADS) rmsnorm_kernel(const NormParams p)
 // covers 256 * SW_VPT consecutive vectors).  Large calls take four: all eight loads of a thread are
 // issued before the arithmetic, 128 bytes per thread in flight (6.3 -> 6.9 TB/s on 32 768 x 27 648);
 // small calls (decode) take one, which spreads them over more blocks.
+// Five blocks per SM: with four vectors the allocation is 48 registers then, 56 otherwise, and four blocks have fewer
+// bytes in flight (5999 x 18944: 103 us, 112).
 template <int SW_VPT>
-__global__ void __launch_bounds__(256) swiglu_kernel(const __nv_bfloat16* __restrict__ gu,
-                                                    __nv_bfloat16* __restrict__ out, long long T, int I) {
+__global__ void __launch_bounds__(256, 5) swiglu_kernel(const __nv_bfloat16* gu, __nv_bfloat16* out, long long T, int I) {
     const int vpr = I / 8;                                   // output vectors per row
     const long long nvec = T * vpr;
     const long long base = static_cast<long long>(blockIdx.x) * (256 * SW_VPT) + threadIdx.x;

@@ -107,7 +107,10 @@ __device__ __forceinline__ int warp_find_sequence(const int32_t* cu, int S, long
 //   * every CTA executes pdl_wait() on every path, early exits included, so a grid completes after
 //     its predecessor;
 //   * pdl_launch_dependents() comes after pdl_wait(): when a kernel starts, everything before its
-//     immediate predecessor has completed.
+//     immediate predecessor has completed;
+//   * no kernel parameter is __restrict__ and nothing is loaded through the read-only path (__ldg): a kernel's
+//     lifetime overlaps the one that writes its inputs, and either would let the compiler take them for constant
+//     throughout and move a load above the wait.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
