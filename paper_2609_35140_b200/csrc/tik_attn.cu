@@ -114,7 +114,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     int row_lo[2] = {0, 0}, row_hi[2] = {0, 0};   // valid tile rows [row_lo, row_hi), per query tile
     int tile_first, tile_last;
     if (MODE == MODE_TRAIN || MODE == MODE_PREFILL) {
-        pdl_launch_dependents();       // a grid launched behind this one may fill the SMs that its last wave leaves
         seq = blockIdx.z;
         head = blockIdx.y;
         kvh = head / p.G;
@@ -154,7 +153,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         tile_first = 0;
         tile_last = T0;
     } else {
-        pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid's last wave
         seq = blockIdx.z;
         kvh = blockIdx.y;
         head = kvh * p.G;
@@ -346,6 +344,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();       // the combine kernel, or a grid that fills the SMs which this one's last wave leaves
     const uint32_t tmem = *tmem_slot;
     auto chunk_of = [&](int it) { return (tile_first + it) / TILES_PER_CHUNK; };
     auto is_chunk_start = [&](int it) { return ((tile_first + it) % TILES_PER_CHUNK) == 0; };

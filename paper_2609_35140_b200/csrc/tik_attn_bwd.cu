@@ -71,15 +71,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     // Launch order and dependencies: delta kernel, dK/dV grid, dQ grid, each with a programmatic
     // dependency.  The dK/dV grid waits for the delta kernel here.  The dQ grid starts once every CTA
-    // of the dK/dV grid has passed that wait (so everything it reads is complete) and must not wait
+    // of the dK/dV grid has passed that wait and holds its tensor memory (so everything it reads is complete) and must not wait
     // for that grid: its CTAs fill the SMs that the dK/dV grid's last CTAs leave idle.  Only its last
     // block waits for the dK/dV grid, at its end, so that the dQ grid completes after it (and no dQ CTA
     // releases its dependents early).  Two sequences of 96 and 160 tokens (4/1 heads, d 64), forward and
     // backward: 32.2 -> 27.6 us.
-    if (MODE == BWD_DKV) {
-        pdl_wait();
-        pdl_launch_dependents();
-    }
+    if (MODE == BWD_DKV) pdl_wait();
     const bool last_block = MODE == BWD_DQ && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 &&
                             blockIdx.z == gridDim.z - 1;
 
@@ -181,6 +178,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (MODE == BWD_DKV) pdl_launch_dependents();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {

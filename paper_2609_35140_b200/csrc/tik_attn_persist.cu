@@ -382,10 +382,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // the plan (and every input) is complete from here on.  Launched behind the single-tile grid
     // (wait_at_end) this grid starts once every CTA of that grid has started, which is after the
     // plan completed, and must not wait for that grid here: it is there to fill its tail.
-    if (!p.wait_at_end) {
-        pdl_wait();
-        pdl_launch_dependents();
-    }
+    if (!p.wait_at_end) pdl_wait();
     if (warp == 3 && lane == 0) {
         // an earlier kernel on this context may have run out of a wait: then do nothing at all
         *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
@@ -393,6 +390,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (!p.wait_at_end) pdl_launch_dependents();
     const uint32_t tmem = *tmem_slot;
 
     // (plan entries are read around L1: a line of an earlier call's plan may still sit there)

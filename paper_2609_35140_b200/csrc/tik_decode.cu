@@ -70,7 +70,6 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     pdl_wait();
-    pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid's last wave
 
     const int seq = blockIdx.z, kvh = blockIdx.y;
     const int head = kvh * p.G;
@@ -172,6 +171,7 @@ decode2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid's last wave
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {

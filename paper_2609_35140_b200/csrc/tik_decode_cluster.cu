@@ -177,7 +177,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         tmem_relinquish();
     }
     pdl_wait();
-    pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
 
     const int seq = blockIdx.z, kvh = blockIdx.y, chunk = static_cast<int>(blockIdx.x) / C;
@@ -223,6 +222,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();       // the combine kernel may be scheduled behind this grid
     // Two cluster barriers: the first says that every CTA's mbarriers exist, the second that nobody
     // writes to another CTA any more (a thread arrives there after its last remote write, all wait at the end).
     cluster_arrive();

@@ -109,12 +109,12 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         tmem_relinquish_pair();
     }
     pdl_wait();
-    pdl_launch_dependents();
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();            // the peer's barriers exist before anything signals them
     tc_fence_after();
+    pdl_launch_dependents();
     const uint32_t tmem = *tmem_slot;
     const uint32_t lead_full = mapa_cluster(bar_full, 0);
     const uint32_t lead_acc_empty = mapa_cluster(bar_acc_empty, 0);
@@ -308,11 +308,11 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         tmem_relinquish();
     }
     pdl_wait();
-    pdl_launch_dependents();
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
@@ -504,11 +504,11 @@ linear_narrow_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         tmem_relinquish();
     }
     pdl_wait();
-    pdl_launch_dependents();
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {

@@ -134,12 +134,12 @@ logprob_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
     }
     pdl_wait();
-    pdl_launch_dependents();           // the finish kernel may be scheduled behind this grid's last wave
     if (tid == 0) *abort_word = (*reinterpret_cast<volatile int*>(p.dev_status) & TIK_DEV_WAIT_EXPIRED) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync_all();            // the peer's barriers exist before anything signals them
     tc_fence_after();
+    pdl_launch_dependents();           // the finish kernel may be scheduled behind this grid's last wave
     const uint32_t tmem = *tmem_slot;
     // the leader's copies of the barriers that both CTAs signal (shared::cluster addresses)
     const uint32_t lead_full = PAIR ? mapa_cluster(bar_full, 0) : bar_full;

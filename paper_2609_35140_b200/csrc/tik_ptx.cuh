@@ -105,9 +105,15 @@ __device__ __forceinline__ int warp_find_sequence(const int32_t* cu, int S, long
 //   * before pdl_wait() a CTA touches no global memory except kernel parameters and L2 prefetches
 //     (writes land in L2, so a prefetched line cannot go stale);
 //   * every CTA executes pdl_wait() on every path, early exits included, so a grid completes after
-//     its predecessor;
+//     its predecessor.  Two grids overlap their predecessor on purpose, which writes nothing that they read: the dQ
+//     grid of the backward and the persistent grid behind the single-tile grid.  They wait at their end (one
+//     block of dQ, every CTA of the other), never release dependents early, and read what earlier calls may have
+//     left in L1 around it (__ldcg);
 //   * pdl_launch_dependents() comes after pdl_wait(): when a kernel starts, everything before its
 //     immediate predecessor has completed;
+//   * ... and after the CTA's tensor memory is allocated (behind the barrier that publishes its address): a dependent
+//     CTA that shares the SM allocates before it waits, and must not hold columns that an earlier CTA, which it
+//     waits for, has yet to get;
 //   * no kernel parameter is __restrict__ and nothing is loaded through the read-only path (__ldg): a kernel's
 //     lifetime overlaps the one that writes its inputs, and either would let the compiler take them for constant
 //     throughout and move a load above the wait.
