@@ -1,6 +1,8 @@
 """Helpers shared by the GPU parity tests (no arithmetic of the method lives here)."""
 from __future__ import annotations
 
+import ctypes
+
 import numpy as np
 import torch
 
@@ -21,6 +23,16 @@ def bits(t: torch.Tensor) -> torch.Tensor:
 
 def count_diff(a: torch.Tensor, b: torch.Tensor) -> int:
     return int((bits(a) != bits(b)).sum().item())
+
+
+NARROW, UNITS, PAIR_UNITS, BAND = range(4)          # TIK_LINEAR_* of include/tik.h
+
+
+def linear_schedule(lib, T: int, K: int, N: int, sms: int = 148):
+    """(schedule, CTAs, columns per unit) that tik_linear takes; asks the library's host code only."""
+    lib.tik_selftest_linear.argtypes = [ctypes.c_int64] + 3 * [ctypes.c_int] + 2 * [ctypes.POINTER(ctypes.c_int)]
+    ctas, cols = ctypes.c_int(), ctypes.c_int()
+    return lib.tik_selftest_linear(T, K, N, sms, ctypes.byref(ctas), ctypes.byref(cols)), ctas.value, cols.value
 
 
 def canary_like(t: torch.Tensor, value: float = -777.0) -> torch.Tensor:

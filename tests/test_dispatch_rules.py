@@ -3,23 +3,15 @@ import ctypes
 
 import pytest
 
+from gpu_common import NARROW, UNITS, linear_schedule
+
 
 @pytest.fixture(scope="module")
 def lib():
     from paper_2609_35140_b200 import binding
     lib = binding.load()
     lib.tik_selftest_decode_cluster.argtypes = [ctypes.c_int64] + 4 * [ctypes.c_int]
-    lib.tik_selftest_linear.argtypes = [ctypes.c_int64] + 3 * [ctypes.c_int] + 2 * [ctypes.POINTER(ctypes.c_int)]
     return lib
-
-
-NARROW, UNITS, PAIR_UNITS, BAND = range(4)
-
-
-def linear_schedule(lib, T, K, N, sms=148):
-    """(schedule, CTAs, columns per unit) of tik_linear."""
-    ctas, cols = ctypes.c_int(), ctypes.c_int()
-    return lib.tik_selftest_linear(T, K, N, sms, ctypes.byref(ctas), ctypes.byref(cols)), ctas.value, cols.value
 
 
 @pytest.mark.parametrize("sms", [148, 132])

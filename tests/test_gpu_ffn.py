@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import oracle
-from gpu_common import count_diff
+from gpu_common import BAND, NARROW, PAIR_UNITS, UNITS, count_diff, linear_schedule
 
 pytestmark = pytest.mark.gpu
 
@@ -28,6 +28,20 @@ def _randn(shape, seed, std=1.0):
 def _close_bf16(got, ref, abs_tol=1e-6):
     g = got.float().cpu().numpy().astype(np.float64)
     assert np.all(np.abs(g - ref) <= 2.0 ** -8 * np.abs(ref) + abs_tol), float(np.abs(g - ref).max())
+
+
+def _schedule(tik, T, K, N):
+    return linear_schedule(tik.load(), T, K, N, torch.cuda.get_device_properties(0).multi_processor_count)[0]
+
+
+def _band_rows(tik, x, W):
+    """tik_linear(x, W) as part of a call that runs as CTA pairs in the band raster, whatever kernel a call of x and W
+    alone takes: more rows of x and more weight rows (both repeated) leave a row's and a column's result alone."""
+    (T, K), N = x.shape, W.shape[0]
+    rows, cols = max(T, 2049), max(N, 512)
+    assert _schedule(tik, rows, K, cols) == BAND
+    xs, Ws = x.repeat(-(-rows // T), 1)[:rows].contiguous(), W.repeat(-(-cols // N), 1)[:cols].contiguous()
+    return tik.tik_linear(xs, Ws)[:T, :N].contiguous()
 
 
 @pytest.mark.parametrize("H", [8, 64, 1000, 1536, 3584, 4096, 5120, 8192])
@@ -100,13 +114,13 @@ def test_linear_matches_oracle_and_is_batch_invariant(tik, T, K, N):
 @pytest.mark.parametrize("K,N", [(512, 37888), (256, 55296), (1024, 5120), (192, 1000), (128, 72), (64, 40000),
                                  (27648, 5120), (3584, 37888)])
 def test_decode_shaped_linear_equals_rows_of_a_batched_call(tik, K, N):
-    """One row tile (T <= 128) takes the persistent column-unit schedule with 64, 128 or 256 columns
-    per unit and 32, 64 or 128 staged rows; every such call returns the bits of the same rows inside a
-    300-row call (CTA pairs, 256-column steps), and writes nothing outside its [T][N] block.  Two row
-    tiles (T <= 256) run the pair kernel persistently over 256-column steps: same check."""
+    """Calls of one and two row tiles, by the narrow schedule or over units of 64, 128 or 256 columns with 32, 64 or
+    128 staged rows or over pairs' units: each returns the bits of the same rows inside a 300-row call, which are
+    those of the band raster (CTA pairs, 256-column steps), and writes nothing outside its [T][N] block."""
     x = _randn((300, K), 2100 + K)
     W = _randn((N, K), 2200 + N % 977, 0.02)
     y = tik.tik_linear(x, W)
+    assert count_diff(y, _band_rows(tik, x, W)) == 0
     ncol = min(N, 4096)                   # the oracle on three rows and the first columns (full-size K x N: seconds)
     ref = oracle.linear(x[:3].float().cpu().numpy(), W[:ncol].float().cpu().numpy())
     g = y[:3, :ncol].float().cpu().numpy().astype(np.float64)
@@ -168,10 +182,13 @@ def test_ffn_invalid_arguments(tik):
 def test_narrow_linear_equals_rows_of_a_batched_call(tik, K, N):
     """T <= 80 and N <= 64 columns per SM: weights as the M operand, 8 .. 64 rows of them per CTA.  Row counts
     around the multiples of 16 that are staged, K tails of a ring stage, outputs of one CTA, of whole and ragged
-    last CTAs, and the first N beyond the range: the bits of a batched call, nothing written outside y."""
+    last CTAs, and the first N beyond the range: the bits of a batched call, which are those of the band raster (a
+    300-row call of few columns is narrow too), nothing written outside y."""
     x = _randn((300, K), 3100 + K)
     W = _randn((N, K), 3200 + N % 977, 0.02)
     y = tik.tik_linear(x, W)
+    assert count_diff(y, _band_rows(tik, x, W)) == 0
+    assert {_schedule(tik, T, K, N) for T in (1, 16, 80)} == {NARROW if N <= 9472 else UNITS}
     ref = oracle.linear(x[:3].float().cpu().numpy(), W.float().cpu().numpy())
     g = y[:3].float().cpu().numpy().astype(np.float64)
     assert np.all(np.abs(g - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4 * 0.02 * np.sqrt(K))
@@ -185,12 +202,16 @@ def test_narrow_linear_equals_rows_of_a_batched_call(tik, K, N):
 
 @pytest.mark.parametrize("K,N", [(64, 8), (192, 1000), (576, 1536), (320, 9480), (128, 37888)])
 def test_mid_size_linear_equals_rows_of_a_batched_call(tik, K, N):
-    """2 .. 16 row tiles: single CTAs over units of 64, 128 or 256 columns x one row tile, or pairs, by a cost
-    model that reaches each of them at these sizes.  Row counts around the tiles and around the range's ends:
-    the bits of a longer call (band raster), nothing written outside y."""
+    """2 .. 16 row tiles: the narrow schedule, single CTAs over units of 64, 128 or 256 columns x one row tile, or
+    pairs, by rules that reach each of them at these sizes.  Row counts around the tiles and around the range's ends:
+    the bits of a longer call, which are those of the band raster, nothing written outside y."""
     x = _randn((2300, K), 3300 + K)
     W = _randn((N, K), 3400 + N % 977, 0.02)
     y = tik.tik_linear(x, W)
+    assert count_diff(y, _band_rows(tik, x, W)) == 0
+    kinds = {_schedule(tik, T, K, N) for T in (129, 256, 385, 768, 1500, 2048)}
+    assert kinds == {8: {NARROW}, 1000: {NARROW, UNITS}, 1536: {NARROW, UNITS}, 9480: {UNITS, PAIR_UNITS},
+                     37888: {UNITS, PAIR_UNITS}}[N]
     rows = [0, 1150, 2299]
     ref = oracle.linear(x[rows].float().cpu().numpy(), W.float().cpu().numpy())
     g = y[rows].float().cpu().numpy().astype(np.float64)
@@ -206,13 +227,36 @@ def test_mid_size_linear_equals_rows_of_a_batched_call(tik, K, N):
 @pytest.mark.parametrize("K,N", [(64, 256), (576, 1536), (640, 4608), (192, 6000)])
 def test_narrow_linear_with_x_as_the_m_operand(tik, K, N):
     """Row counts where x becomes the M operand of the narrow schedule (M64, M128, tiles of 128 rows), around the
-    8-row atoms and the tiles: the bits of a batched call, nothing written outside y."""
+    8-row atoms and the tiles: the bits of a batched call, which are those of the band raster and near the
+    oracle's, nothing written outside y."""
     x = _randn((2300, K), 3500 + K)
     W = _randn((N, K), 3600 + N % 977, 0.02)
     y = tik.tik_linear(x, W)
+    assert count_diff(y, _band_rows(tik, x, W)) == 0
+    assert _schedule(tik, 72, K, N) == NARROW and _schedule(tik, 127, K, N) == NARROW
+    rows = [0, 700, 2299]
+    ref = oracle.linear(x[rows].float().cpu().numpy(), W.float().cpu().numpy())
+    g = y[rows].float().cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(g - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4 * 0.02 * np.sqrt(K))
     for a, T in [(0, 17), (5, 24), (9, 40), (3, 41), (100, 63), (50, 64), (172, 65), (1, 72), (7, 88), (11, 127), (64, 128), (13, 129), (700, 260)]:
         buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
         tik.tik_linear(x[a:a + T].contiguous(), W, y=buf[1:T + 1])
         assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
         assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
+    assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("T,K,N", [(768, 320, 1152), (768, 320, 1184), (384, 192, 1576), (2304, 128, 256), (3456, 128, 256),
+                                   (5000, 64, 128), (18944, 64, 40), (20000, 128, 8), (20000, 64, 24)])
+def test_narrow_linear_at_the_ends_of_its_range(tik, T, K, N):
+    """As many CTAs as SMs, one more (another kernel takes the call), more than 16 row tiles, and more row tiles than
+    SMs with one CTA each: the bits of the band raster, nothing written outside y."""
+    x = _randn((T, K), 3700 + K)
+    W = _randn((N, K), 3800 + N % 977, 0.02)
+    narrow = (T, N) not in ((768, 1184), (3456, 256))
+    assert (_schedule(tik, T, K, N) == NARROW) == narrow
+    buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
+    tik.tik_linear(x, W, y=buf[1:T + 1])
+    assert count_diff(buf[1:T + 1], _band_rows(tik, x, W)) == 0
+    assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
     assert tik.device_status() == 0
