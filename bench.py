@@ -652,10 +652,8 @@ def workload_config(w: synth.Workload, n_gpus: int):
             "head_dim": w.d, "page_size": w.page_size, "total_tokens": w.total_tokens,
             "response_tokens": w.response_tokens, "hidden": w.hidden, "vocab": w.vocab,
             "decode_contexts": w.decode_contexts or "full sequence lengths",
-            "l2": "before every phase a 512 MiB buffer is overwritten (L2 flush) and a 256 MiB buffer is read (pushes the "
-                  "flush's own dirty lines out, so the phase does not pay for their write-back); excluded from the phase times",
-            "alone": "the phases timed on their own follow the steps after %.0f s of idle time (the step's "
-                     "power state has decayed); they are context for the in-step figures, not part of `value`" % ALONE_PAUSE_S,
+            # (the read pushes the flush's own dirty lines out, so a phase does not pay for their write-back)
+            "l2": "flushed before every phase (512 MiB written, 256 MiB read), outside the phase times",
             "parallelism": "replicas x%d (no collective)" % n_gpus}
 
 
@@ -758,8 +756,38 @@ def report_workload(w, nums, info, peaks, world):
     return out
 
 
+def _short(x):
+    """Five significant digits for measured numbers; whole numbers and texts as they are."""
+    if isinstance(x, float):
+        return float("%.5g" % x)
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    return [_short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def printed_line(line):
+    """What goes to standard output: the contract's keys, and of every workload and operator the figures that say
+    how fast it was.  Readers that keep only the last few KiB of a run's output get the whole line; the blocks in
+    full (times alone, fractions of every peak, bytes, notes) go to the file that --detail names."""
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                                "scaling", "vs_baseline", "dtype", "data", "config", "gpu_launches",
+                                "gpu_launches_other_configs", "device_flags", "contract")}
+    out["clocks"] = line["clocks"]
+    out["e2e"] = {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")}
+    out["phases_ms"], out["decode_tok_per_s"] = line["phases_ms"], line["decode_tok_per_s"]
+    out["roofline"] = {k: v for k, v in line["roofline"].items() if k != "traffic_source"}
+    # name -> [ms, achieved (TFLOP/s or GB/s), fraction of the peak it is held against]
+    out["rooflines"] = {n: [r["ms"], r["achieved"], r["frac"]] for n, r in line["rooflines"].items()}
+    out["cpu_baseline"] = line["cpu_baseline"]
+    out["per_config"] = {n: {"value_ms": c["value_ms"], "sm_mhz": c["clocks"].get("sm_mhz"),
+                             "tflops": [c[k]["tflops"] for k in ("train_fwd", "prefill", "logprob")],
+                             "decode_gbs": [d["gbs"] for d in c["decode"]]} for n, c in line["per_config"].items()}
+    return _short(out)
+
+
 def main():
     ap = argparse.ArgumentParser()
+    ap.add_argument("--detail", help="also write every block in full to this file (JSON)")
     ap.add_argument("--gpus", type=int, default=1)
     ap.add_argument("--steps", type=int, default=10)
     ap.add_argument("--warmup", type=int, default=3)
@@ -906,7 +934,10 @@ def main():
         "gpu_launches_other_configs": side_launches,
         "clocks": clk, "device_flags": flags, "contract": tik.contract_id(),
     }
-    print(json.dumps(line))
+    if args.detail:
+        with open(args.detail, "w") as f:
+            json.dump(line, f)
+    print(json.dumps(printed_line(line)))
     tdist.finalize()
 
 
