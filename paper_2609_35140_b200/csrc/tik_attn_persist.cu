@@ -310,6 +310,17 @@ __device__ __noinline__ void pa_store_rows(uint32_t acc, float inv, int row0, in
     }
 }
 
+// A row's log-sum-exp.  Out of line in the packed kernel, where the two copies cost the softmax warps registers (12 bytes
+// spilled, 140 bytes read back): 16 x 1280 .. 4880 tokens (28/4 heads) with lse 1325 -> 1297 us, 4 x 2248 .. 3164 (64/8)
+// 520 -> 509, without lse 1305 -> 1283; the paged kernel does not spill, and its small calls lose by the call (13 x
+// 131 .. 239 tokens 23.4 -> 26.8 us).
+__device__ __noinline__ void pa_store_lse_call(float* lse, long long i, float m, float l, float c) { lse[i] = finalize_lse(m, l, c); }
+template <bool PAGED>
+__device__ __forceinline__ void pa_store_lse(float* lse, long long i, float m, float l, float c) {
+    if (PAGED) lse[i] = finalize_lse(m, l, c);
+    else pa_store_lse_call(lse, i, m, l, c);
+}
+
 template <int D, bool PAGED>
 __global__ void __launch_bounds__(PA_THREADS, 1)
 attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -748,7 +759,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     volatile int* m = meta_pair + 8 * (k & 1) + 4 * wg;
                     const int e_row0 = m[0], e_lo = m[1], e_hi = m[2], e_head = m[3];
                     if (r >= e_lo && r < e_hi && p.lse)
-                        p.lse[(static_cast<long long>(e_row0) + r) * p.Hq + e_head] = finalize_lse(m_run, Ltot, c);
+                        pa_store_lse<PAGED>(p.lse, (static_cast<long long>(e_row0) + r) * p.Hq + e_head, m_run, Ltot, c);
 #ifdef TIK_PA_TRACE
                     long long* tr = (blockIdx.x == 0 && k < PA_TRACE_ITEMS && quarter == 0 && lane == 0)
                                         ? &g_pa_trace[k * PA_TRACE_EVENTS + 32 + 8 * wg] : nullptr;
@@ -892,7 +903,7 @@ attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         m[3] = it.head;
                     }
                     if (r >= lo && r < hi && p.lse)
-                        p.lse[(static_cast<long long>(row0) + r) * p.Hq + it.head] = finalize_lse(M_g, Ltot, c);
+                        pa_store_lse<PAGED>(p.lse, (static_cast<long long>(row0) + r) * p.Hq + it.head, M_g, Ltot, c);
                     tc_fence_before();
                 }
                 asm volatile("bar.sync 1, 256;" ::: "memory");
