@@ -1049,7 +1049,7 @@ kv_write_kernel(const uint4* k_new, const uint4* v_new, const int32_t* cu_new, c
                 uint4* k_cache, uint4* v_cache, const int32_t* block_table, int max_blocks, int S, long long total_new, int Hkv,
                 int vec_per_head /* d*2/16 */, int page_size, int num_pages, int* dev_status) {
     pdl_wait();
-    pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid
+    if (KVW_TOK == 1) pdl_launch_dependents();     // (prompts at the end: the rule in tik_ptx.cuh)
     __shared__ long long dst_base[KVW_TOK];     // vector index of (page, head 0, row, 0), or -1
     const long long tok0 = static_cast<long long>(blockIdx.x) * KVW_TOK;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1098,6 +1098,7 @@ kv_write_kernel(const uint4* k_new, const uint4* v_new, const int32_t* cu_new, c
             }
         }
     }
+    if (KVW_TOK > 1) pdl_launch_dependents();
 }
 
 // ------------------------------------------------------------------ launchers

@@ -546,7 +546,6 @@ template <int D>
 __global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* dout,
                                                        float* delta, long long n_vec) {
     pdl_wait();
-    pdl_launch_dependents();
     const long long v0 = ((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * DELTA_VPW;
     const int lane = threadIdx.x & 31;
     constexpr int W = D / 64;                               // 32-bit words per lane (4 or 2 elements)
@@ -581,6 +580,7 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const __nv_bfloat16* o, 
         if (lane == j) mine = part;
     }
     if (lane < DELTA_VPW && v0 + lane < n_vec) delta[v0 + lane] = mine;
+    pdl_launch_dependents();       // (at the end: the rule in tik_ptx.cuh)
 }
 
 template <int D, int MODE>

@@ -53,12 +53,14 @@ __device__ __forceinline__ void prep_unpack(const uint32_t* raw, float* x) {
     }
 }
 
+constexpr int64_t PREP_SPLIT_TOKENS = 2048;     // calls of at most so many tokens: a warp per batch of heads
+
 template <int D>
 __global__ void __launch_bounds__(PREP_WARPS * 32, PREP_MIN_CTAS) prep_kernel(const PrepParams p) {
     constexpr int EP = D / 32;
     constexpr int VPH = D * 2 / 16;             // 16-byte pieces of one V row
     pdl_wait();
-    pdl_launch_dependents();       // an attention kernel launched next may be scheduled behind this grid
+    if (p.total_new <= PREP_SPLIT_TOKENS) pdl_launch_dependents();     // (larger calls at the end: the rule in tik_ptx.cuh)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane >> 4, l16 = lane & 15;
     const long long token = static_cast<long long>(blockIdx.x) * PREP_WARPS + warp;   // one warp per token
@@ -181,16 +183,18 @@ __global__ void __launch_bounds__(PREP_WARPS * 32, PREP_MIN_CTAS) prep_kernel(co
             }
         }
     }
+    if (p.total_new > PREP_SPLIT_TOKENS) pdl_launch_dependents();
 }
 
 cudaError_t launch_prep(int d, const PrepParams& p, int64_t total_new, cudaStream_t stream) {
     if (total_new <= 0) return cudaSuccess;
     const unsigned grid = static_cast<unsigned>((total_new + PREP_WARPS - 1) / PREP_WARPS);
     // A token of Hq + Hkv heads is a serial chain of batches in one warp.  While the warps of one token per
-    // warp would not fill the chip, every batch gets a warp (with the warp-wide sequence search, in a graph): 64
-    // tokens of 28 + 4 heads 8.6 -> 3.6 us, 256 of 64 + 8 16.3 -> 5.5, 16 of 12 + 2 4.6 -> 3.4.
+    // warp would fill half of the chip's slots or less, every batch gets a warp (with the warp-wide sequence search, in a
+    // graph): 64 tokens of 28 + 4 heads 8.6 -> 3.6 us, 256 of 64 + 8 16.3 -> 5.5, 16 of 12 + 2 4.6 -> 3.4, 2000 tokens of
+    // 28 + 4 10.7 -> 9.6, of 64 + 8 20.9 -> 18.3; 2500 to 4000 tokens are even or, of 12 + 2 heads, slower (6.9 -> 7.3).
     const int batches = (p.Hq + p.Hkv + 2 * PREP_BATCH - 1) / (2 * PREP_BATCH);
-    const unsigned split = total_new * batches <= 4096 ? static_cast<unsigned>(batches) : 1u;
+    const unsigned split = total_new <= PREP_SPLIT_TOKENS ? static_cast<unsigned>(batches) : 1u;
     return launch_pdl(d == 128 ? prep_kernel<128> : prep_kernel<64>, dim3(grid, split), PREP_WARPS * 32, 0, stream, 1, p);
 }
 

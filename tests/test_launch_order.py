@@ -34,7 +34,7 @@ def test_dependents_are_released_after_the_wait_and_the_tensor_memory():
     for name, body in _kernels():
         releases = [m.start() for m in re.finditer(r"\bpdl_launch_dependents\(\)", body)]
         allocs = [m.start() for m in re.finditer(r"\btmem_alloc(?:_pair)?\(", body)]
-        assert len(releases) == 1 and "pdl_wait()" in body, name
+        assert releases and "pdl_wait()" in body, name
         assert body.index("pdl_wait()") < releases[0], name
         if allocs:
             assert max(allocs) < body.index("__syncthreads()", max(allocs)) < releases[0], name
