@@ -49,7 +49,7 @@ struct AttnSmem {
 };
 
 // Rarely taken paths of the softmax loops, kept out of line so that the loop bodies stay small
-// (the loops of two warpgroups, the issuing threads and the producers share one instruction cache).
+// (the loops of two warpgroups, the issuing warps and the producers share one instruction cache).
 template <int D>
 __device__ __noinline__ void rescale_o_tmem(uint32_t to, float alpha) {
 #pragma unroll 1
@@ -227,7 +227,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     auto produce_tile = [&](int it) {                       // whole warp (paged) or lane 0 (train)
         const int j = tile_first + it;
         // (no division by a run-time stage count: this code sits between a stage's release and its
-        // next request, and the issuing threads below are the pace-makers of the tensor pipe)
+        // next request, and the issuing warps below are the pace-makers of the tensor pipe)
         const bool two = !kv && KS == 2;
         const int st = two ? (it & 1) : (it % KV_STAGES);
         const uint32_t use = two ? (it >> 1) : (it / KV_STAGES);
@@ -394,8 +394,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ QK^T issuer
-        // Two threads feed the tensor pipe (this one and the PV issuer in warp 3): whatever an
-        // issuing thread executes between MMAs is time in which it queues nothing, so each
+        // Two warps feed the tensor pipe (this one and the PV issuer, warp 3): whatever an
+        // issuing warp executes between MMAs is time in which it queues nothing, so each
         // keeps to waits, one MMA chain and its commits per step.
         {
             const uint32_t tmem = warp_uniform(*tmem_slot);

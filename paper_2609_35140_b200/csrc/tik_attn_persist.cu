@@ -1,7 +1,7 @@
 // Full-sequence attention (packed train-forward, paged prefill) as a persistent kernel.
 //
 // The arithmetic, the tile and chunk structure and the roles are those of attn_kernel
-// (tik_attn.cu): one CTA per SM, two TMA warps (Q + K, V), two MMA-issuing threads (QK^T, PV),
+// (tik_attn.cu): one CTA per SM, two TMA warps (Q + K, V), two MMA-issuing warps (QK^T, PV),
 // two softmax warpgroups, S / P / O in tensor memory.  What differs is the schedule.  There a CTA
 // is one work item -- a pair of query tiles 2m, 2m+1 (tiles 0..15) or one query tile >= 16 of one
 // (sequence, head) -- and pays entry, first-data latency, epilogue and exit for each (~8 700 clk

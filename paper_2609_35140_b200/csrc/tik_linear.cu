@@ -170,7 +170,7 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         // shared memory and leave as one tiled TMA store of 128 rows x 128 bytes (row-by-row
         // 16-byte stores from 128 threads cost a third of the kernel on wide outputs).  The store
         // clips at the tensor's bounds, so rows past T and columns past N need no guard.  Two
-        // staging tiles alternate; the issuing thread lets at most one store group read behind it.
+        // staging tiles alternate; the storing thread lets at most one store group read behind it.
         const int quarter = warp & 3;                      // TMEM lane quarter of this warp
         const int row = quarter * 32 + lane;
         uint32_t piece = 0;
@@ -253,7 +253,7 @@ linear_unit_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int nu = p.nu;
     const uint32_t a_bytes = static_cast<uint32_t>(p.a_rows) * 128u;
     const uint32_t slice_bytes = a_bytes + static_cast<uint32_t>(nu) * 128u;      // a multiple of 1 KiB
-    // K slices per stage: the issuing thread spends ~300 cycles per stage on its barrier wait, fence,
+    // K slices per stage: the issuing warp spends ~300 cycles per stage on its barrier wait, fence,
     // descriptors and commit, more than four narrow MMAs run (N = 128: 256 cycles, N = 64: ~190);
     // 256 / nu slices per stage (as long as three stages fit) bring that share down (N = 256 MMAs run
     // 512 cycles per slice and hide it)

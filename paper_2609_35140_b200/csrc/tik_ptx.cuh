@@ -355,18 +355,6 @@ __device__ __forceinline__ void mma_ts_chain8(uint32_t d_tmem, uint32_t a_tmem, 
         : "memory");
 }
 
-// The first four of those steps (64 contraction rows).
-__device__ __forceinline__ void mma_ts_chain4(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                              uint32_t idesc, uint32_t first_accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p0, pt, e;\n\telect.sync _|e, 0xffffffff;\n\t.reg .b64 db;\n\t.reg .b32 ta;\n\t"
-        "setp.ne.b32 p0, %4, 0;\n\tsetp.eq.b32 pt, 0, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
-        TIK_MMA_TS_STEP(8, 128) TIK_MMA_TS_STEP(16, 256) TIK_MMA_TS_STEP(24, 384)
-        "}" ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(first_accumulate)
-        : "memory");
-}
-
 // All eight steps with A laid out as four 32-column blocks whose first 16 columns hold the two
 // steps of that block (a thread that owns 32 fp32 columns of a tile leaves the bf16 pairs of its
 // 32 contraction rows in the first 16 of them).
@@ -386,7 +374,7 @@ __device__ __forceinline__ void mma_ts_chain8_blocks(uint32_t d_tmem, uint32_t a
 // ---------------------------------------------------------------- CTA pairs (cta_group::2)
 // Two CTAs of a cluster of two, on neighbouring SMs, execute one MMA of M = 256: each holds its
 // own 128 rows of A and half of the B tile in its shared memory and its own 128 accumulator rows
-// in its tensor memory.  The MMA is issued by one thread of the leader CTA (cluster rank 0).
+// in its tensor memory.  The MMA is issued by an elected lane of the leader CTA's (cluster rank 0) issuing warp.
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));

@@ -10,7 +10,8 @@
 // device flag word.  Every GPU that loads the library holds those bytes until the process
 // exits.
 //
-// The kernels are the ones tik_attn_decode launches, so the output bits are the same.
+// The kernels are among those that tik_attn_decode launches (one CTA per chunk, never clusters), so the output
+// bits are the same.
 #include <cmath>
 #include <mutex>
 
