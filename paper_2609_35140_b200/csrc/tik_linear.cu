@@ -447,8 +447,8 @@ static cudaError_t launch_linear_unit(const CUtensorMap& tmA, const CUtensorMap&
 // the one whose choice reads fewer rows: the weights (M64) for few rows of x, x (M64, M128) for more.  The
 // products of an element and the order of its sums are the same either way, so are the bits.
 // Ring: stages of kps K slices; one TMA copy per operand and stage through a [K / 64][rows][64] view.
-// linear_unit_kernel -> weights as M, cold L2: T = 16: K 8960, N 1536 28.5 -> 20.5 us; K 18944, N 3584 51 -> 33;
-// K 27648, N 5120 72 -> 51.  Weights as M -> x as M, W out of HBM: T = 64: K 1536, N 256 5.2 -> 4.4; K 8960,
+// linear_unit_kernel -> weights as M, W out of HBM, in a graph: T = 16: K 8960, N 1536 26.3 -> 12.2 us; K 18944, N 3584
+// 52 -> 27.4; K 27648, N 5120 75 -> 46.  Weights as M -> x as M: T = 64: K 1536, N 256 5.2 -> 4.4; K 8960,
 // N 1536 18.3 -> 13.4; K 3584, N 4608 10.4 -> 9.0; K 18944, N 3584 37.7 -> 34.5.  linear_unit_kernel -> x as M,
 // T = 100: K 8960, N 1536 24.6 -> 19.6; K 18944, N 3584 52.8 -> 44.9; T = 300: K 1536, N 256 6.5 -> 5.3.
 namespace linn {
