@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 
@@ -210,7 +211,7 @@ struct LinearParams {
     int super_cols;              // pairs, band raster: output columns per CTA, a multiple of 256, at most 4096
     int unit_mode;               // persistent CTAs (pairs) over nunit units
     int ntp;                     // units per column step: row tiles (pairs: pairs of row tiles)
-    int nu, nunit, a_rows;       // columns per unit 64 / 128 / 256 (pairs: 256), units, staged x rows 32 / 64 / 128
+    int nu, nunit, a_rows;       // columns per unit 64 / 128 / 256 (pairs: 256), units, staged x rows 8 / 16 / 32 / 64 / 128
                                  // (narrow outputs: weight rows per CTA 8 .. 64, CTAs, x rows 8 .. 128)
     int kps, nst;                // narrow outputs: K slices per ring stage, stages (12 at most)
     int m;                       // narrow outputs: rows of the M operand if that is x: 64 or 128; 0: the weights
@@ -236,7 +237,10 @@ struct LinearChoice {
     int nu;
     bool units;                  // persistent over units, else the band raster (pairs)
 };
-inline int linear_staged_rows(long long T) { return T <= 32 ? 32 : T <= 64 ? 64 : 128; }
+// Rows of x that a K slice of a call of one row tile stages.  What lies past T arrives as zeros, but not for free: with 32
+// rows for calls of 1 .. 7 the x copies of all CTAs were late (K 8960, N 10240, 1 row 43.6 us, 33.9 with 8; N 12288 43.8,
+// 37.4; 16 rows, N 10240 35.8, 34.3 with 16).
+inline int linear_staged_rows(long long T) { return T <= 8 ? 8 : T <= 16 ? 16 : T <= 32 ? 32 : T <= 64 ? 64 : 128; }
 inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_count) {
     const long long ntile = (T + 127) / 128;
     LinearChoice best = {false, 256, true};
@@ -261,7 +265,7 @@ inline LinearChoice linear_choose(long long T, int K, int N, int a_rows, int sm_
 // fits L2).
 inline LinearChoice linear_wide_choose(const LinearParams& p) {
     if (p.T > 16 * 128) return {true, 256, false};
-    return linear_choose(p.T, p.K, p.N, linear_staged_rows(p.T), p.sm_count);
+    return linear_choose(p.T, p.K, p.N, std::max(32, linear_staged_rows(p.T)), p.sm_count);
 }
 // The narrow schedule: one unit of nu weight rows x one row tile per CTA, nu as few as need no more CTAs than SMs
 // (whole 8-row swizzle atoms; an MMA of 128 rows takes N = 16 i), or one CTA per row tile when there are more of those.

@@ -231,7 +231,7 @@ linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 // rate, so the schedule is built for bytes in flight and even SM load: the grid is one persistent
 // CTA per SM walking units u = blockIdx.x, + gridDim.x, ...; a unit is `nu` = 64, 128 or 256 output columns of
 // one row tile (row tile fastest: the CTAs running at one time share W columns in L2);
-// only `a_rows` = 32, 64 or 128 rows of x are staged per K slice (the MMA spans 64 or 128 rows: rows
+// only `a_rows` = 8, 16, 32, 64 or 128 rows of x are staged per K slice (the MMA spans 64 or 128 rows: rows
 // past a_rows read whatever the stage holds, their accumulator rows are never stored); the ring
 // has as many stages as fit in 192 KiB (3 .. 12) of one, two or four K slices each, and the producer runs ahead
 // into the next unit while the epilogue of the last one drains.

@@ -260,3 +260,24 @@ def test_narrow_linear_at_the_ends_of_its_range(tik, T, K, N):
     assert count_diff(buf[1:T + 1], _band_rows(tik, x, W)) == 0
     assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
     assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("K,N", [(64, 9480), (576, 12288), (1024, 24576), (256, 40000)])
+def test_unit_linear_of_a_few_rows(tik, K, N):
+    """Column units of 128, 256 and 128 columns with 8, 16 or 32 staged rows of x, fewer than an MMA spans: the bits of
+    the band raster, nothing written outside y, and rows of infinities in W stay in their own columns."""
+    x = _randn((40, K), 3900 + K)
+    W = _randn((N, K), 4000 + N % 977, 0.02)
+    y = _band_rows(tik, x, W)
+    W2 = W.clone()
+    W2[5], W2[70] = float("inf"), float("nan")           # (what the MMA reads behind the staged rows is W)
+    keep = torch.ones(N, dtype=torch.bool, device="cuda")
+    keep[5] = keep[70] = False
+    for a, T in [(0, 1), (3, 2), (9, 7), (30, 8), (4, 9), (20, 15), (24, 16), (1, 17), (8, 32)]:
+        assert _schedule(tik, T, K, N) == UNITS
+        buf = torch.full((T + 2, N), -7.0, dtype=torch.bfloat16, device="cuda")
+        tik.tik_linear(x[a:a + T].contiguous(), W, y=buf[1:T + 1])
+        assert count_diff(buf[1:T + 1], y[a:a + T]) == 0, (a, T)
+        assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
+        assert count_diff(tik.tik_linear(x[a:a + T].contiguous(), W2)[:, keep], y[a:a + T][:, keep]) == 0, (a, T)
+    assert tik.device_status() == 0
