@@ -784,6 +784,7 @@ tik_status tik_attn_train_bwd(tik_ctx* ctx, const void* q, const void* k, const 
     p.dq_heads = items < 5ll * ctx->sm_count ? 1 : items < 12ll * ctx->sm_count || max_tiles > 12 ? 2 : 4;
     p.dq_heads = std::min(p.dq_heads, p.G);
     p.dq_groups = (p.G + p.dq_heads - 1) / p.dq_heads;
+    p.dq_tiles_first = max_tiles > 65535;
     cudaError_t e = launch_attn_bwd(d, (max_seqlen + 127) / 128, S, tmQ, tmK, tmV, tmDO, p, o, d_o,
                                     total_tokens * Hq, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_train_bwd");

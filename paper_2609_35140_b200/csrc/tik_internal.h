@@ -312,6 +312,7 @@ struct BwdParams {
     float c;                     // softmax_scale * log2(e)
     float scale;
     int dq_heads, dq_groups;     // query heads per dQ CTA, CTAs per KV head: ceil(G / dq_heads)
+    int dq_tiles_first;          // dQ grid: query tiles fastest (where they would not fit a grid's second axis)
     int* dev_status;
 };
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,
