@@ -125,3 +125,17 @@ def test_backward_of_many_short_sequences_equals_each_alone(tik, S, Hq, Hkv, d):
         for a, b in zip(alone, got):
             assert count_diff(a, b[sl]) == 0, (s, lens[s])
     assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("bound", [65535 * 128, 65535 * 128 + 1])
+def test_backward_under_a_loose_length_bound(tik, bound):
+    """The dQ grid has its query tiles on the second axis as long as they fit there (65535), on the first beyond."""
+    w = synth.custom_workload([1, 1], [299, 128], 4, 2, 128, 64, index=59)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    do, _, _, _ = synth.make_qkv(w, "cuda", seed_offset=9)
+    want = _fwd_bwd(tik, w, q, k, v, cu, do)
+    lse = torch.empty(q.shape[0], w.Hq, dtype=torch.float32, device="cuda")
+    o = tik.tik_attn_train_fwd(q, k, v, cu, max(w.seq_lens), w.softmax_scale, lse=lse)
+    got = tik.tik_attn_train_bwd(q, k, v, o, do, lse, cu, bound, w.softmax_scale)
+    for a, b in zip(got, want):
+        assert count_diff(a, b) == 0
