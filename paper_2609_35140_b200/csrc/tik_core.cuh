@@ -235,11 +235,44 @@ __device__ __forceinline__ float hn_warp_total(float part) {
 __device__ __forceinline__ float hn_block_total(const float* w4) {
     return __fadd_rn(__fadd_rn(w4[0], w4[1]), __fadd_rn(w4[2], w4[3]));
 }
-// silu(g) * u with silu(g) = g * 1 / (1 + 2^(-g log2 e)): ex2.approx, correctly rounded reciprocal
-__device__ __forceinline__ float swiglu_value(float g, float u) {
-    const float e = ex2_ftz(__fmul_rn(g, -LOG2E_F));
-    const float sig = __frcp_rn(__fadd_rn(1.0f, e));
-    return __fmul_rn(__fmul_rn(g, sig), u);
+// silu(g) * u with silu(g) = g * 1 / (1 + 2^(-g log2 e)): ex2.approx, correctly rounded reciprocal, two outputs at a time
+// with two-wide instructions.  1 / x for x = 1 + e in [1, 2^126]: the approximate reciprocal and one
+// Newton step in fused arithmetic (Markstein), which gives the correctly rounded reciprocal for every such x (all of
+// them compared with __frcp_rn); beyond 2^126 -- gates below -87 -- the intrinsic itself.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ void rcp_rn_x2(float x0, float x1, float& r0, float& r1) {
+    const float a0 = rcp_approx(x0), a1 = rcp_approx(x1);
+    asm("{\n\t.reg .b64 rx, ra, re, one;\n\t"
+        "mov.b64 rx, {%2, %3};\n\tmov.b64 ra, {%4, %5};\n\tmov.b64 one, {%6, %6};\n\t"
+        "fma.rn.f32x2 re, rx, ra, one;\n\tfma.rn.f32x2 ra, ra, re, ra;\n\tmov.b64 {%0, %1}, ra;\n\t}"
+        : "=f"(r0), "=f"(r1)
+        : "f"(-x0), "f"(-x1), "f"(a0), "f"(a1), "f"(1.0f));
+}
+__device__ __forceinline__ void swiglu_value_x2(float g0, float g1, float u0, float u1, float& o0, float& o1) {
+    float x0, x1, r0, r1;
+    asm("{\n\t.reg .b64 ra, rb;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\t"
+        "mul.rn.f32x2 ra, ra, rb;\n\tmov.b64 {%0, %1}, ra;\n\t}"
+        : "=f"(x0), "=f"(x1)
+        : "f"(g0), "f"(g1), "f"(-LOG2E_F));
+    x0 = ex2_ftz(x0);
+    x1 = ex2_ftz(x1);
+    asm("{\n\t.reg .b64 ra, rb;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %4};\n\t"
+        "add.rn.f32x2 ra, ra, rb;\n\tmov.b64 {%0, %1}, ra;\n\t}"
+        : "=f"(x0), "=f"(x1)
+        : "f"(x0), "f"(x1), "f"(1.0f));
+    rcp_rn_x2(x0, x1, r0, r1);
+    if (fmaxf(x0, x1) > 0x1p126f) {
+        r0 = __frcp_rn(x0);
+        r1 = __frcp_rn(x1);
+    }
+    asm("{\n\t.reg .b64 rg, rr, ru;\n\tmov.b64 rg, {%2, %3};\n\tmov.b64 rr, {%4, %5};\n\tmov.b64 ru, {%6, %7};\n\t"
+        "mul.rn.f32x2 rg, rg, rr;\n\tmul.rn.f32x2 rg, rg, ru;\n\tmov.b64 {%0, %1}, rg;\n\t}"
+        : "=f"(o0), "=f"(o1)
+        : "f"(g0), "f"(g1), "f"(r0), "f"(r1), "f"(u0), "f"(u1));
 }
 
 // ---- attention backward: weight and score gradient of one (query, key) pair ------------------

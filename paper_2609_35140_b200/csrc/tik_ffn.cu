@@ -91,6 +91,9 @@ __global__ void __launch_bounds__(HN_THREADS) rmsnorm_kernel(const NormParams p)
 // covers 256 * SW_VPT consecutive vectors).  Large calls take four: all eight loads of a thread are
 // issued before the arithmetic, 128 bytes per thread in flight (6.3 -> 6.9 TB/s on 32 768 x 27 648);
 // small calls (decode) take one, which spreads them over more blocks.
+// Inside an FFN the power limit holds the clock at 1.4 GHz and the kernel is bound by its instructions as much as by HBM,
+// so outputs go two at a time (swiglu_value_x2) and a row is found by one division per thread: 5999 x 18944
+// 149.5 -> 126.9 us, 16000 x 8960 172 -> 152, 3001 x 27648 108 -> 94; alone 105.5 -> 102.4, 300 x 8960 4.62 -> 4.15.
 // Five blocks per SM: with four vectors the allocation is 48 registers then, 56 otherwise, and four blocks have fewer
 // bytes in flight (5999 x 18944: 103 us, 112).
 template <int SW_VPT>
@@ -129,7 +132,7 @@ __global__ void __launch_bounds__(256, 5) swiglu_kernel(const __nv_bfloat16* gu,
             unpack8(gv[j], g);
             unpack8(uv[j], u);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) o[e] = swiglu_value(g[e], u[e]);
+            for (int e = 0; e < 8; e += 2) swiglu_value_x2(g[e], g[e + 1], u[e], u[e + 1], o[e], o[e + 1]);
             reinterpret_cast<uint4*>(out)[idx] = pack8(o);
         }
     }
