@@ -281,3 +281,20 @@ def test_unit_linear_of_a_few_rows(tik, K, N):
         assert bool((buf[0] == -7.0).all()) and bool((buf[T + 1] == -7.0).all())
         assert count_diff(tik.tik_linear(x[a:a + T].contiguous(), W2)[:, keep], y[a:a + T][:, keep]) == 0, (a, T)
     assert tik.device_status() == 0
+
+
+@pytest.mark.parametrize("rows,I", [(1, 8), (513, 8), (5, 264), (3, 2056), (700, 12000), (1049000, 8)])
+def test_swiglu_gates_of_every_size(tik, rows, I):
+    """Rows of less than a block's vectors, of more, and a last block that ends in the middle; gates from those whose
+    reciprocal is subnormal to those whose weight is one, infinities and NaN.  One bf16 rounding (2^-9) and fp32
+    arithmetic below it.  Where 2^(-g log2 e) is beyond fp32 (g < -88.72) the weight is 0: off by at most
+    88.73 * 2^-128 * 7 < 1.9e-36, the most that |g| e^g u comes to there (u <= 7)."""
+    g = torch.linspace(-104.0, 104.0, rows * I, device="cuda").to(torch.bfloat16)
+    special = torch.tensor([float("inf"), float("-inf"), float("nan"), 0.0, -87.5, -88.5, -90.0, 88.5], device="cuda")
+    g[:8] = special.to(torch.bfloat16)
+    u = (1.0 + torch.arange(rows * I, device="cuda") % 7).to(torch.bfloat16)
+    got = tik.tik_swiglu(torch.cat([g.view(rows, I), u.view(rows, I)], dim=1).contiguous()).view(-1).double()
+    want = g.double() / (1.0 + torch.exp(-g.double())) * u.double()
+    odd = ~torch.isfinite(want)
+    assert torch.equal(torch.nan_to_num(got[odd], nan=7.0), torch.nan_to_num(want[odd], nan=7.0))
+    assert bool(((got - want).abs()[~odd] <= 2.0 ** -8 * want.abs()[~odd] + 1.9e-36).all())
