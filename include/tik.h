@@ -72,17 +72,20 @@ const char* tik_contract_id(void);
  * kernels that use more than 48 KiB of shared memory are opted in once per (kernel, device), and
  * this exercises that table with stand-in ordinals.  Needs no GPU.  Returns 0 when it holds. */
 int tik_selftest_host(void);
-/* Host-only views of two dispatch rules for tests (no paper counterpart; need no GPU).
+/* Host-only views of dispatch rules for tests (no paper counterpart; need no GPU).
  * tik_selftest_linear: the schedule (TIK_LINEAR_*) that tik_linear takes for x [T][K], W [N][K] on sm_count
  * SMs, its CTAs and the output columns of one of their units.
  * tik_selftest_decode_cluster: CTAs per chunk of a decode call of so many (sequence, KV head, chunk) items on a
- * device that holds max_clusters clusters of the cluster kernel at one time, 0 when another kernel takes it. */
+ * device that holds max_clusters clusters of the cluster kernel at one time, 0 when another kernel takes it.
+ * tik_selftest_bwd_dq: the dQ grid of a tik_attn_train_bwd call: 1 when its query tiles are fastest, 0 when its heads
+ * are, and the query heads of a CTA. */
 #define TIK_LINEAR_NARROW 0        /* one unit of few weight rows per CTA */
 #define TIK_LINEAR_UNITS 1         /* persistent CTAs over column units */
 #define TIK_LINEAR_PAIR_UNITS 2    /* persistent CTA pairs over 256-column units */
 #define TIK_LINEAR_BAND 3          /* CTA pairs, band raster (ctas: 0) */
 int tik_selftest_linear(int64_t T, int K, int N, int sm_count, int* ctas, int* cols);
 int tik_selftest_decode_cluster(int64_t chunks, int max_ctx, int G, int d, int max_clusters);
+int tik_selftest_bwd_dq(int64_t S, int64_t total_tokens, int max_seqlen, int Hq, int Hkv, int d, int sm_count, int* heads);
 
 /* Number of kernels the library has launched in this process so far (all contexts, all streams;
  * every launch site counts itself when it enqueues a kernel).  No paper counterpart: it lets a

@@ -214,6 +214,15 @@ int tik_selftest_linear(int64_t T, int K, int N, int sm_count, int* ctas, int* c
 int tik_selftest_decode_cluster(int64_t chunks, int max_ctx, int G, int d, int max_clusters) {
     return decode_cluster_size(chunks, max_ctx, G, d, max_clusters);
 }
+int tik_selftest_bwd_dq(int64_t S, int64_t total_tokens, int max_seqlen, int Hq, int Hkv, int d, int sm_count, int* heads) {
+    BwdParams p{};
+    p.Hq = Hq;
+    p.Hkv = Hkv;
+    p.G = Hq / Hkv;
+    bwd_dq_choose(p, S, total_tokens, max_seqlen, d, sm_count);
+    *heads = p.dq_heads;
+    return p.dq_tiles_first;
+}
 const char* tik_contract_id(void) { return TIK_CONTRACT_ID; }
 
 size_t tik_workspace_bytes(int op, int64_t rows_or_batch, int Hq, int Hkv, int d, int64_t max_ctx, int H,
@@ -773,18 +782,7 @@ tik_status tik_attn_train_bwd(tik_ctx* ctx, const void* q, const void* k, const 
     p.c = scale_to_c(softmax_scale);
     p.scale = softmax_scale;
     p.dev_status = ctx->dev_status;
-    // Query heads per dQ CTA: a head's set-up, first loads and epilogue run under its neighbour's steps, but longer
-    // CTAs leave a longer tail.  Backward, us, 1 / 2 / 4 heads per CTA, with items (tile, head) per SM:
-    //   (d 128, 64/8 heads) 47 x 45..238 tokens, 41: 331 / 281 / 269;  21 x 77..681, 37: 559 / 478 / 471
-    //   (32/8) 10 x 385..2369, 23: 723 / 667 / 679;  8 x 100..400, 5.0: 65.8 / 61.6 / 64.7;  2048, 3.5: 132 / 135 / 161
-    //   (28/4) 16 x 1280..5120, 73: 3940 / 3817 / 3832;  32 x 60..128, 6.1: 68.7 / 62.9 / 64.0
-    //   (d 64, 4/1) 9 x 3440..7743, 11: 717 / 714 / 762;  40 x 100..500, 3.3: 36.2 / 36.3 / 36.9
-    const long long max_tiles = (max_seqlen + 127) / 128;
-    const long long items = std::min<long long>(total_tokens / 128 + S, max_tiles * S) * Hq;
-    p.dq_heads = items < 5ll * ctx->sm_count ? 1 : items < 12ll * ctx->sm_count || max_tiles > 12 ? 2 : 4;
-    p.dq_heads = std::min(p.dq_heads, p.G);
-    p.dq_groups = (p.G + p.dq_heads - 1) / p.dq_heads;
-    p.dq_tiles_first = max_tiles > 65535;
+    bwd_dq_choose(p, S, total_tokens, max_seqlen, d, ctx->sm_count);
     cudaError_t e = launch_attn_bwd(d, (max_seqlen + 127) / 128, S, tmQ, tmK, tmV, tmDO, p, o, d_o,
                                     total_tokens * Hq, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? TIK_OK : cuda_fail(ctx, e, "tik_attn_train_bwd");

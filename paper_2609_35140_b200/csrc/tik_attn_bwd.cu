@@ -94,11 +94,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const int nq = (len + 127) / 128;                      // tiles of the sequence (query and KV alike)
     int own, head = 0, kvh, n_steps, n_heads = 1;
     if (MODE == BWD_DQ) {
-        // Heads fastest, then query tiles, heaviest first: a sequence's heavy tiles of all heads before the light
-        // ones, which are left for the end of the grid (tiles fastest before, so that the last head's heaviest tile
-        // started last).  3 x 1500 tokens (8/8 heads) 89.3 -> 82.8 us, 21 x 77..681 (64/8) 559 -> 547, 10 x 385..2369
-        // (32/8) 649 -> 640, 16 x 1280..5120 (28/4) 3712 -> 3689, 9001 + 16384 (32/8) 7234 -> 7191.  (The dK/dV grid
-        // in that order: no faster, and 0.5 % slower in a loop of seconds at 9001 + 16384: more heads' Q and dO at a time.)
+        // query tiles from the heaviest down; heads fastest or one after the other: bwd_dq_choose.  (The dK/dV grid with
+        // its heads fastest is no faster.)
         const int group = p.dq_tiles_first ? blockIdx.y : blockIdx.x;
         own = p.dq_tiles_first ? gridDim.x - 1 - blockIdx.x : gridDim.y - 1 - blockIdx.y;
         if (own >= nq) return;                             // (never the last block: its tile is 0)

@@ -312,9 +312,43 @@ struct BwdParams {
     float c;                     // softmax_scale * log2(e)
     float scale;
     int dq_heads, dq_groups;     // query heads per dQ CTA, CTAs per KV head: ceil(G / dq_heads)
-    int dq_tiles_first;          // dQ grid: query tiles fastest (where they would not fit a grid's second axis)
+    int dq_tiles_first;          // dQ grid: query tiles fastest, one head after the other; 0: heads fastest
     int* dev_status;
 };
+// The dQ grid of a backward call: heads per CTA and order.
+//
+// Query heads per CTA: a head's set-up, first loads and epilogue run under its neighbour's steps, but longer
+// CTAs leave a longer tail.  Backward, us, 1 / 2 / 4 heads per CTA in the order below, with items (tile, head) per SM:
+//   (d 128, 64/8 heads) 47 x 45..238 tokens, 41: 381 / 321 / 306;  21 x 77..681, 35: 542 / 468 / 456;  16 x 500..3000, 107:
+//   4280 / 4132 / 4102
+//   (32/8) 10 x 385..2369, 27: 934 / 860 / 844;  8 x 100..400, 4.8: 60.3 / 53.8 / 56.9;  2048, 3.5: 130 / 130 / 130
+//   (28/4) 16 x 1280..5120, 71: 3983 / 3888 / 3855;  32 x 60..128, 6.1: 62.0 / 56.4 / 56.2
+//   (12/2) 16 x 1000..3000, 21: 820 / 774 / 795;  (8/1) 8 x 2000, 6.9: 254 / 258 / 264
+//   (d 64, 4/1) 9 x 3440..7743, 11: 713 / 731 / 765;  40 x 100..500, 3.5: 34.2 / 33.9 / 35.9
+//
+// Order: heads fastest runs the heavy query tiles of all heads first and leaves the light ones for the end of the grid, a
+// tail shorter by ~0.6 us per tile of the longest sequence and head of a CTA.  Tiles fastest where that costs more.
+// Backward, us, tiles fastest / heads fastest:
+//   shorter tail    (8/8) 3 x 1500 66.4 / 60.1;  (32/8) 2 x 4096 918 / 886;  (12/2) 8 x 4096 1355 / 1309;  (16/16) 10240, K and V
+//                   84 MB, 1350 / 1297
+//   K and V of all the heads are in use at a time, and beyond two thirds of L2 are read again
+//                   (32/32) 16384 6475 / 6860;  (64/64) 8192 3469 / 3859;  (32/8) 24576, 101 MB, 13862 / 14146;  65536 96531 /
+//                   100267;  ((16/16) 12288, 101 MB, 1885 / 1845)
+//   many KV heads   (64/64) 4 x 2048 1216 / 1354;  (32/32) 2 x 4096 983 / 997 and 997 / 969;  8 x 1024 433 / 436
+//   empty tiles, of sequences shorter than max_seqlen: a CTA starts every ~12 ns, which hides while other heads' tiles are at
+//   work; all heads' empty tiles in one run do not
+//                   (64/8) 32 x 200..1000 under 8192 1407 / 1472;  8 x 1000 under 16384 806 / 839;  (28/4) 32 x 200..1000 under
+//                   8192 658 / 670;  (64/32) 24 x 126..1500 2201 / 2320;  (32/8) 10 x 385..2369 920 / 915 (heads fastest here)
+inline void bwd_dq_choose(BwdParams& p, int64_t S, int64_t total_tokens, int64_t max_seqlen, int d, int sm_count) {
+    const int64_t max_tiles = (max_seqlen + 127) / 128, most = total_tokens / 128 + S;
+    const int64_t items = (most < max_tiles * S ? most : max_tiles * S) * p.Hq;
+    p.dq_heads = items < 5ll * sm_count ? 1 : items < 12ll * sm_count || max_tiles > 12 ? 2 : 4;
+    p.dq_heads = p.dq_heads < p.G ? p.dq_heads : p.G;
+    p.dq_groups = (p.G + p.dq_heads - 1) / p.dq_heads;
+    const int64_t kv_bytes = (max_seqlen < total_tokens ? max_seqlen : total_tokens) * p.Hkv * d * 4;
+    const bool hidden = (S * max_seqlen - total_tokens) * p.Hkv * p.dq_groups <= 50 * max_seqlen * p.dq_heads;
+    p.dq_tiles_first = max_tiles > 65535 || p.Hkv > 32 || kv_bytes > 80ll << 20 || !hidden;   // (65535: a grid's second axis)
+}
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,
                             const CUtensorMap& tmV, const CUtensorMap& tmDO, const BwdParams& p,
                             const void* o, const void* dout, long long n_vec, cudaStream_t stream);

@@ -35,6 +35,13 @@ def linear_schedule(lib, T: int, K: int, N: int, sms: int = 148):
     return lib.tik_selftest_linear(T, K, N, sms, ctypes.byref(ctas), ctypes.byref(cols)), ctas.value, cols.value
 
 
+def bwd_dq_grid(lib, S: int, tokens: int, max_seqlen: int, Hq: int, Hkv: int, d: int, sms: int = 148):
+    """(query tiles fastest, query heads per CTA) of tik_attn_train_bwd's dQ grid; host code only."""
+    lib.tik_selftest_bwd_dq.argtypes = 2 * [ctypes.c_int64] + 5 * [ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)]
+    heads = ctypes.c_int()
+    return bool(lib.tik_selftest_bwd_dq(S, tokens, max_seqlen, Hq, Hkv, d, sms, ctypes.byref(heads))), heads.value
+
+
 def canary_like(t: torch.Tensor, value: float = -777.0) -> torch.Tensor:
     return torch.full_like(t, value)
 

@@ -3,7 +3,7 @@ import ctypes
 
 import pytest
 
-from gpu_common import NARROW, UNITS, linear_schedule
+from gpu_common import NARROW, UNITS, bwd_dq_grid, linear_schedule
 
 
 @pytest.fixture(scope="module")
@@ -46,3 +46,24 @@ def test_clusters_only_while_all_of_them_run_at_once(lib, max_clusters):
         assert got == (4 if chunks <= max_clusters else 0), chunks
     for refused in ((4, 896, 8, 128), (4, 4000, 9, 128), (4, 4000, 8, 64)):
         assert lib.tik_selftest_decode_cluster(*refused, max_clusters) == 0
+
+
+def test_dq_grid_order(lib):
+    """Heads fastest only where that is no slower than one head after the other: K and V of all heads stay in L2, and few
+    tiles of the grid are empty."""
+    full = [(1, 8192, 32, 8, 128), (2, 4096, 32, 8, 128), (3, 1500, 8, 8, 128), (8, 4096, 12, 2, 128), (1, 16384, 28, 4, 128),
+            (1, 10240, 16, 16, 128), (2, 4096, 32, 32, 128), (1, 20480, 8, 8, 128)]
+    for S, L, Hq, Hkv, d in full:
+        assert bwd_dq_grid(lib, S, S * L, L, Hq, Hkv, d)[0] is False, (S, L, Hq, Hkv)
+        # a bound far above every sequence: many empty tiles
+        assert bwd_dq_grid(lib, 64, 32 * L, L, Hq, Hkv, d)[0] is True, (L, Hq, Hkv)
+    for S, L, Hq, Hkv, d in [(1, 16384, 32, 32, 128), (1, 8192, 64, 64, 128), (1, 65536, 32, 8, 128), (1, 32768, 32, 8, 128),
+                             (4, 2048, 64, 64, 128), (1, 16384, 64, 64, 64), (1, 131072, 12, 2, 128), (1, 16384, 64, 16, 128)]:
+        assert bwd_dq_grid(lib, S, S * L, L, Hq, Hkv, d)[0] is True, (S, L, Hq, Hkv)
+    for S, tokens, bound, Hq, Hkv, d in [(24, 19500, 1500, 16, 16, 128), (24, 19500, 1500, 40, 20, 128), (32, 19200, 8192, 64, 8, 128),
+                                         (8, 8000, 16384, 32, 8, 128), (32, 19200, 8192, 28, 4, 128), (128, 28800, 4096, 28, 4, 128)]:
+        assert bwd_dq_grid(lib, S, tokens, bound, Hq, Hkv, d)[0] is True, (S, tokens, bound, Hq, Hkv)
+    assert bwd_dq_grid(lib, 1, 300, 65535 * 128, 4, 2, 128)[0] is False
+    assert bwd_dq_grid(lib, 1, 300, 65535 * 128 + 1, 4, 2, 128)[0] is True        # beyond the grid's second axis
+    for S, tokens, bound, Hq, Hkv in [(65535, 2 ** 31 - 1, 2 ** 31 - 1, 65535, 65535), (65535, 1, 2 ** 31 - 1, 65535, 1), (1, 2 ** 31 - 1, 1, 1, 1)]:
+        bwd_dq_grid(lib, S, tokens, bound, Hq, Hkv, 128)                           # (nothing overflows)

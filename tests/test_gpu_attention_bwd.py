@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2609_35140_b200 import synth
-from gpu_common import count_diff
+from gpu_common import bwd_dq_grid, count_diff
 
 pytestmark = pytest.mark.gpu
 
@@ -139,3 +139,27 @@ def test_backward_under_a_loose_length_bound(tik, bound):
     got = tik.tik_attn_train_bwd(q, k, v, o, do, lse, cu, bound, w.softmax_scale)
     for a, b in zip(got, want):
         assert count_diff(a, b) == 0
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d,heads", [([300, 17], 18, 9, 64, 1), ([260, 240, 201], 40, 20, 128, 1), ([700, 500, 650] * 2, 28, 4, 128, 2),
+                                                 ([1400, 1300, 1500] * 2, 30, 5, 64, 4)])
+def test_backward_in_both_orders_of_the_dq_grid(tik, lens, Hq, Hkv, d, heads):
+    """Heads fastest under a tight length bound, query tiles fastest under one that leaves most of the grid empty: the same
+    bits, with one, two and four heads per CTA."""
+    total, tight, loose = sum(lens), max(lens), max(lens) + 128 * 300
+    assert bwd_dq_grid(tik.load(), len(lens), total, tight, Hq, Hkv, d) == (False, heads)
+    tiles_first = bwd_dq_grid(tik.load(), len(lens), total, loose, Hq, Hkv, d)[0]
+    w = synth.custom_workload([1] * len(lens), [n - 1 for n in lens], Hq, Hkv, d, 64, index=60)
+    q, k, v, cu = synth.make_qkv(w, "cuda")
+    do, _, _, _ = synth.make_qkv(w, "cuda", seed_offset=9)
+    lse = torch.empty(q.shape[0], w.Hq, dtype=torch.float32, device="cuda")
+    o = tik.tik_attn_train_fwd(q, k, v, cu, tight, w.softmax_scale, lse=lse)
+    got = tik.tik_attn_train_bwd(q, k, v, o, do, lse, cu, tight, w.softmax_scale)
+    bound = loose if tiles_first else 65535 * 128 + 1
+    assert bwd_dq_grid(tik.load(), len(lens), total, bound, Hq, Hkv, d)[0]
+    other = tik.tik_attn_train_bwd(q, k, v, o, do, lse, cu, bound, w.softmax_scale)
+    want = oracle.attn_bwd_packed(q.float().cpu().numpy(), k.float().cpu().numpy(), v.float().cpu().numpy(),
+                                  do.float().cpu().numpy(), w.cu_seqlens(), w.softmax_scale)
+    for name, a, b, c in zip(("dq", "dk", "dv"), got, other, want):
+        _check(a, c, name)
+        assert count_diff(a, b) == 0, name
