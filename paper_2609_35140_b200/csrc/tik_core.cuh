@@ -236,9 +236,11 @@ __device__ __forceinline__ float hn_block_total(const float* w4) {
     return __fadd_rn(__fadd_rn(w4[0], w4[1]), __fadd_rn(w4[2], w4[3]));
 }
 // silu(g) * u with silu(g) = g * 1 / (1 + 2^(-g log2 e)): ex2.approx, correctly rounded reciprocal, two outputs at a time
-// with two-wide instructions.  1 / x for x = 1 + e in [1, 2^126]: the approximate reciprocal and one
-// Newton step in fused arithmetic (Markstein), which gives the correctly rounded reciprocal for every such x (all of
-// them compared with __frcp_rn); beyond 2^126 -- gates below -87 -- the intrinsic itself.
+// with two-wide instructions.  1 / x for x = 1 + e in [1, 2^126] by one Newton step in fused arithmetic from the
+// approximate reciprocal.  From an approximation within one unit in the last place that step rounds correctly, except
+// perhaps where the significand of x is all ones (P. W. Markstein, Computation of elementary functions on the IBM RISC
+// System/6000 processor, IBM J. Res. Dev. 34, 1990); there, and for the unit, it takes this chip's rcp.approx, so
+// tests/swiglu_check.cu compares every float of the range with __frcp_rn.  Beyond 2^126 -- gates below -87 -- the intrinsic.
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

@@ -1,11 +1,16 @@
 """GPU parity of hidden RMSNorm, fused residual + RMSNorm, SwiGLU and the dense linear layer
 against the CPU oracle, and their bit-identity between batched and row-by-row use (the paper's
 operator table verifies each of them bitwise between full-sequence and token-wise execution)."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
 import oracle
+from paper_2609_35140_b200 import build as tik_build
 from gpu_common import BAND, NARROW, PAIR_UNITS, UNITS, count_diff, linear_schedule
 
 pytestmark = pytest.mark.gpu
@@ -298,3 +303,40 @@ def test_swiglu_gates_of_every_size(tik, rows, I):
     odd = ~torch.isfinite(want)
     assert torch.equal(torch.nan_to_num(got[odd], nan=7.0), torch.nan_to_num(want[odd], nan=7.0))
     assert bool(((got - want).abs()[~odd] <= 2.0 ** -8 * want.abs()[~odd] + 1.9e-36).all())
+
+
+@pytest.fixture(scope="module")
+def swiglu_check(tmp_path_factory):
+    """tests/swiglu_check.cu, built with the library's flags against the library's header."""
+    out = str(tmp_path_factory.mktemp("swiglu") / "swiglu_check.so")
+    source = os.path.join(os.path.dirname(os.path.abspath(__file__)), "swiglu_check.cu")
+    r = subprocess.run([tik_build._nvcc()] + tik_build.NVCC_FLAGS + ["-I" + tik_build.CSRC, "-shared", source, "-o", out],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    lib = ctypes.CDLL(out)
+    lib.swiglu_check_rcp.argtypes = [ctypes.c_uint, ctypes.c_uint, ctypes.c_void_p]
+    lib.swiglu_check_gates.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
+    return lib
+
+
+def _float_bits(x):
+    return int(np.float32(x).view(np.uint32))
+
+
+def test_swiglu_reciprocal_is_the_correctly_rounded_one(swiglu_check):
+    """Every float from 1 to 2^126, in both lanes.  The approximate reciprocal alone is not that one everywhere."""
+    first, last = _float_bits(1.0), _float_bits(2.0 ** 126)
+    count = torch.zeros(3, dtype=torch.int64, device="cuda")
+    assert swiglu_check.swiglu_check_rcp(first, last, count.data_ptr()) == 0
+    differ, approx, seen = count.tolist()
+    assert seen == last - first + 1 and approx > 0
+    assert differ == 0
+
+
+def test_swiglu_two_at_a_time_has_the_bits_of_one_at_a_time(swiglu_check):
+    """All 65536 bf16 gates, infinities and NaN among them, beside a gate of another size."""
+    up = torch.tensor([1.0, -1.0, 0.0, 3.0, -0.1, 1e-38, 3e38, float("inf"), float("nan")], device="cuda").to(torch.bfloat16).float()
+    count = torch.zeros(3, dtype=torch.int64, device="cuda")
+    assert swiglu_check.swiglu_check_gates(up.data_ptr(), up.numel(), count.data_ptr()) == 0
+    assert count[2].item() == 65536
+    assert count[0].item() == 0
