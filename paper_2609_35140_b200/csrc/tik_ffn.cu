@@ -13,6 +13,7 @@
 namespace tik {
 
 constexpr int HN_THREADS = 128;
+constexpr unsigned SW_VEC_MAX = 0xfffff000u;      // SwiGLU output vectors per launch
 
 __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
     const uint32_t r[4] = {v.x, v.y, v.z, v.w};
@@ -92,28 +93,27 @@ __global__ void __launch_bounds__(HN_THREADS) rmsnorm_kernel(const NormParams p)
 // issued before the arithmetic, 128 bytes per thread in flight (6.3 -> 6.9 TB/s on 32 768 x 27 648);
 // small calls (decode) take one, which spreads them over more blocks.
 // Inside an FFN the power limit holds the clock at 1.4 GHz and the kernel is bound by its instructions as much as by HBM,
-// so outputs go two at a time (swiglu_value_x2) and a row is found by one division per thread: 5999 x 18944
-// 149.5 -> 126.9 us, 16000 x 8960 172 -> 152, 3001 x 27648 108 -> 94; alone 105.5 -> 102.4, 300 x 8960 4.62 -> 4.15.
-// Five blocks per SM: with four vectors the allocation is 48 registers then, 56 otherwise, and four blocks have fewer
-// bytes in flight (5999 x 18944: 103 us, 112).
+// so outputs go two at a time (swiglu_value_x2), indices have 32 bits and a row is found by one division per thread.  One
+// output at a time with a 64-bit division per vector -> this, us, alone out of HBM: 5999 x 18944 111.7 -> 106.0, 16000 x 8960
+// 182 -> 139, 3001 x 27648 107 -> 84, 700 x 18944 22.6 -> 20.5.  The FFN around it: 5999 rows 2077 -> 2072 (within what runs of
+// one side differ by), 16000 1308 -> 1290, 3000 x 8960 259.8 -> 255.0, 16 x 8960 24.5 -> 23.9; with the division and indices
+// alone 2072, 1294, 257.3 and 24.3.
+// Five blocks per SM: with four vectors the allocation is 48 registers then (nothing spilled), 56 otherwise, and four blocks
+// have fewer bytes in flight (5999 x 18944 106 us both; 8000 x 12288 98, four blocks 102; 3001 x 27648 84, 87).
 template <int SW_VPT>
-__global__ void __launch_bounds__(256, 5) swiglu_kernel(const __nv_bfloat16* gu, __nv_bfloat16* out, long long T, int I) {
-    const int vpr = I / 8;                                   // output vectors per row
-    const long long nvec = T * vpr;
-    const long long base = static_cast<long long>(blockIdx.x) * (256 * SW_VPT) + threadIdx.x;
+__global__ void __launch_bounds__(256, 5) swiglu_kernel(const __nv_bfloat16* gu, __nv_bfloat16* out, unsigned nvec, unsigned vpr,
+                                                        unsigned dt, unsigned dc) {
+    const unsigned base = blockIdx.x * (256u * SW_VPT) + threadIdx.x;    // (nvec is at most SW_VEC_MAX: nothing wraps)
     pdl_wait();
     pdl_launch_dependents();
-    // Row and column of a thread's first vector by one division (32 bits wide where the count is), of the next ones by
-    // adding up: a 64-bit division per vector was a third of the instructions, and at the 1.4 GHz of a power-limited FFN
-    // the kernel was bound by them.
-    long long t = nvec <= 0xffffffffll ? static_cast<unsigned>(base) / static_cast<unsigned>(vpr) : base / vpr;
-    int c = static_cast<int>(base - t * vpr);
-    const int dt = 256 / vpr, dc = 256 - dt * vpr;
+    // Row and column of a thread's first vector by one division, of the next ones, 256 = dt * vpr + dc vectors on, by
+    // adding up: a 64-bit division per vector was a third of the instructions.
+    unsigned t = base / vpr, c = base - t * vpr;
     uint4 gv[SW_VPT], uv[SW_VPT];
 #pragma unroll
     for (int j = 0; j < SW_VPT; ++j) {
         if (base + 256 * j < nvec) {
-            const uint4* row = reinterpret_cast<const uint4*>(gu) + t * 2 * vpr;
+            const uint4* row = reinterpret_cast<const uint4*>(gu) + 2ull * t * vpr;
             gv[j] = row[c];
             uv[j] = row[vpr + c];
         }
@@ -126,14 +126,18 @@ __global__ void __launch_bounds__(256, 5) swiglu_kernel(const __nv_bfloat16* gu,
     }
 #pragma unroll
     for (int j = 0; j < SW_VPT; ++j) {
-        const long long idx = base + 256 * j;
+        const unsigned idx = base + 256 * j;
         if (idx < nvec) {
-            float g[8], u[8], o[8];
-            unpack8(gv[j], g);
-            unpack8(uv[j], u);
+            uint32_t w[4] = {gv[j].x, gv[j].y, gv[j].z, gv[j].w};
+            const uint32_t uw[4] = {uv[j].x, uv[j].y, uv[j].z, uv[j].w};
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) swiglu_value_x2(g[e], g[e + 1], u[e], u[e + 1], o[e], o[e + 1]);
-            reinterpret_cast<uint4*>(out)[idx] = pack8(o);
+            for (int e = 0; e < 4; ++e) {
+                float o0, o1;
+                swiglu_value_x2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u), __uint_as_float(uw[e] << 16),
+                                __uint_as_float(uw[e] & 0xffff0000u), o0, o1);
+                w[e] = pack_bf16x2(o0, o1);
+            }
+            reinterpret_cast<uint4*>(out)[idx] = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 }
@@ -153,11 +157,19 @@ cudaError_t launch_rmsnorm(const NormParams& p, cudaStream_t stream) {
 }
 
 cudaError_t launch_swiglu(const void* gu, void* out, long long T, int I, cudaStream_t stream) {
-    if (T <= 0) return cudaSuccess;
-    const long long n = T * (I / 8);
-    const bool large = n >= (1ll << 20);
-    return launch_pdl(large ? swiglu_kernel<4> : swiglu_kernel<1>, dim3(static_cast<unsigned>(large ? (n + 1023) / 1024 : (n + 255) / 256)),
-                      256, 0, stream, 1, static_cast<const __nv_bfloat16*>(gu), static_cast<__nv_bfloat16*>(out), T, I);
+    const unsigned vpr = I / 8;                              // output vectors per row
+    const auto* g = static_cast<const __nv_bfloat16*>(gu);
+    auto* o = static_cast<__nv_bfloat16*>(out);
+    // a launch takes as many rows as 32-bit vector indices count
+    for (long long rows; T > 0; T -= rows, g += 2 * rows * I, o += rows * I) {
+        rows = std::min<long long>(T, SW_VEC_MAX / vpr);
+        const unsigned n = static_cast<unsigned>(rows * vpr);
+        const bool large = n >= (1u << 20);
+        cudaError_t e = launch_pdl(large ? swiglu_kernel<4> : swiglu_kernel<1>, dim3(large ? (n + 1023) / 1024 : (n + 255) / 256), 256, 0,
+                                   stream, 1, g, o, n, vpr, 256 / vpr, 256 % vpr);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace tik

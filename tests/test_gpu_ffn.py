@@ -340,3 +340,24 @@ def test_swiglu_two_at_a_time_has_the_bits_of_one_at_a_time(swiglu_check):
     assert swiglu_check.swiglu_check_gates(up.data_ptr(), up.numel(), count.data_ptr()) == 0
     assert count[2].item() == 65536
     assert count[0].item() == 0
+
+
+@pytest.mark.parametrize("rows,I", [(33000, 264), (4200, 2040), (8200, 1032), (70000, 120), (12000, 704)])
+def test_swiglu_rows_of_less_than_a_block_in_large_calls(tik, rows, I):
+    """Calls of four vectors per thread whose rows have 15 .. 255 vectors: a step of 256 is dt whole rows and dc vectors,
+    both above zero, with and without a carry, and a last block that ends in the middle.  The bits of the same rows in
+    calls of one vector per thread."""
+    vpr = I // 8
+    assert rows * vpr >= 1 << 20 and rows * vpr % 1024 and 256 // vpr and 256 % vpr
+    gu = _randn((rows, 2 * I), 1400 + I, 3.0)
+    out = torch.full((rows + 1, I), -7.0, dtype=torch.bfloat16, device="cuda")
+    tik.tik_swiglu(gu, out=out[:rows])
+    small = (1 << 20) // vpr - 1
+    for a in range(0, rows, small):
+        part = gu[a:a + small]
+        assert part.shape[0] * vpr < 1 << 20
+        assert count_diff(tik.tik_swiglu(part), out[a:min(a + small, rows)]) == 0, a
+    assert bool((out[rows] == -7.0).all())
+    g, u = gu[:, :I].double(), gu[:, I:].double()
+    want = g / (1.0 + torch.exp(-g)) * u
+    assert bool(((out[:rows].double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-6).all())
