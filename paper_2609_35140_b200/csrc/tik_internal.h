@@ -335,10 +335,12 @@ struct BwdParams {
 //                   (32/32) 16384 6475 / 6860;  (64/64) 8192 3469 / 3859;  (32/8) 24576, 101 MB, 13862 / 14146;  65536 96531 /
 //                   100267;  ((16/16) 12288, 101 MB, 1885 / 1845)
 //   many KV heads   (64/64) 4 x 2048 1216 / 1354;  (32/32) 2 x 4096 983 / 997 and 997 / 969;  8 x 1024 433 / 436
-//   empty tiles, of sequences shorter than max_seqlen: a CTA starts every ~12 ns, which hides while other heads' tiles are at
-//   work; all heads' empty tiles in one run do not
-//                   (64/8) 32 x 200..1000 under 8192 1407 / 1472;  8 x 1000 under 16384 806 / 839;  (28/4) 32 x 200..1000 under
-//                   8192 658 / 670;  (64/32) 24 x 126..1500 2201 / 2320;  (32/8) 10 x 385..2369 920 / 915 (heads fastest here)
+//   empty tiles, of sequences shorter than max_seqlen: a CTA starts every ~10 ns, which hides while other heads' tiles are at
+//   work; all heads' empty tiles in one run do not.  By empty CTAs per tile of max_seqlen and head of a CTA (60: the two even)
+//                   236 (64/8) 32 x 200..2000 3545 / 3577;  180 (64/32) 24 x 126..1500 2201 / 2320;  118 (28/4) 32 x 200..2000
+//                   1577 / 1603;  60.1 (32/8) 8 x 1000 under 16384 410 / 430;  56 (28/4) 16 x 1433..5120 3920 / 3904;
+//                   53 (28/4) 2 x 1000 under 16384 121 / 118;  44 (12/2) 32 x 200..2000 692 / 682;  24 (28/4) 4 x 1000 under 4096
+//                   152 / 146;  6 (32/8) 4000 under 16384 492 / 448
 inline void bwd_dq_choose(BwdParams& p, int64_t S, int64_t total_tokens, int64_t max_seqlen, int d, int sm_count) {
     const int64_t max_tiles = (max_seqlen + 127) / 128, most = total_tokens / 128 + S;
     const int64_t items = (most < max_tiles * S ? most : max_tiles * S) * p.Hq;
@@ -346,7 +348,7 @@ inline void bwd_dq_choose(BwdParams& p, int64_t S, int64_t total_tokens, int64_t
     p.dq_heads = p.dq_heads < p.G ? p.dq_heads : p.G;
     p.dq_groups = (p.G + p.dq_heads - 1) / p.dq_heads;
     const int64_t kv_bytes = (max_seqlen < total_tokens ? max_seqlen : total_tokens) * p.Hkv * d * 4;
-    const bool hidden = (S * max_seqlen - total_tokens) * p.Hkv * p.dq_groups <= 50 * max_seqlen * p.dq_heads;
+    const bool hidden = (S * max_seqlen - total_tokens) * p.Hkv * p.dq_groups <= 60 * max_seqlen * p.dq_heads;
     p.dq_tiles_first = max_tiles > 65535 || p.Hkv > 32 || kv_bytes > 80ll << 20 || !hidden;   // (65535: a grid's second axis)
 }
 cudaError_t launch_attn_bwd(int d, int max_tiles, int S, const CUtensorMap& tmQ, const CUtensorMap& tmK,
