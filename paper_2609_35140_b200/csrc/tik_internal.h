@@ -337,8 +337,8 @@ struct BwdParams {
 //   many KV heads   (64/64) 4 x 2048 1216 / 1354;  (32/32) 2 x 4096 983 / 997 and 997 / 969;  8 x 1024 433 / 436
 //   empty tiles, of sequences shorter than max_seqlen: a CTA starts every ~10 ns, which hides while other heads' tiles are at
 //   work; all heads' empty tiles in one run do not.  By empty CTAs per tile of max_seqlen and head of a CTA (60: the two even)
-//                   236 (64/8) 32 x 200..2000 3545 / 3577;  180 (64/32) 24 x 126..1500 2201 / 2320;  118 (28/4) 32 x 200..2000
-//                   1577 / 1603;  60.1 (32/8) 8 x 1000 under 16384 410 / 430;  56 (28/4) 16 x 1433..5120 3920 / 3904;
+//                   475 (64/8) 32 x 200..1000 under 8192 1370 / 1468;  236 (64/8) 32 x 200..2000 3545 / 3577;  118 (28/4) 32 x
+//                   200..2000 1577 / 1603;  60.1 (32/8) 8 x 1000 under 16384 410 / 430;  56 (28/4) 16 x 1433..5120 3920 / 3904;
 //                   53 (28/4) 2 x 1000 under 16384 121 / 118;  44 (12/2) 32 x 200..2000 692 / 682;  24 (28/4) 4 x 1000 under 4096
 //                   152 / 146;  6 (32/8) 4000 under 16384 492 / 448
 inline void bwd_dq_choose(BwdParams& p, int64_t S, int64_t total_tokens, int64_t max_seqlen, int d, int sm_count) {
